@@ -19,6 +19,13 @@ constexpr int kObsFixed = 3 * kPlane + 2;          // 77: three planes, own leve
 constexpr uint32_t kDomainReset = 0x52534554u;     // key tweak of the placement stream
 constexpr uint32_t kDomainAction = 0x41435431u;    // key tweak of the action-uniform stream
 
+// Whether a block of `count` floats at `p` can leave in 16-byte pieces (bulk copies and vector stores demand it).  Of the address
+// itself: a trajectory that is collected in pieces starts each piece at a later row of the caller's arrays, which for odd
+// batches is no 16-byte boundary.
+__host__ __device__ __forceinline__ bool whole_pieces16(const float *p, int count) {
+  return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (count & 3) == 0;
+}
+
 // Device status word values (0 = fine).
 constexpr int kStatusTimeout = 1;
 constexpr int kStatusBadIndex = 2;  // an environment index of a minibatch was out of range (its rows were skipped)

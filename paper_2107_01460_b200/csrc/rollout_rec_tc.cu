@@ -240,7 +240,7 @@ rollout_rec_tc_kernel(RolloutArgs a, const unsigned char *__restrict__ image, fl
       if (!last) {  // the observation block of this step goes out while the MMAs run
         float *obs_dst = a.buf.obs + row0 * D;
         const int count = n_rows * D;
-        if (((row0 * D) & 3) == 0 && (count & 3) == 0) {
+        if (whole_pieces16(obs_dst, count)) {
           if (tid == 64) { bulk_store(obs_dst, stage_addr, static_cast<uint32_t>(count) * 4u); bulk_pending = true; }
         } else {
           for (int i = tid; i < count; i += kRecThreads) obs_dst[i] = sm.stage[i];

@@ -68,7 +68,7 @@ rollout_simt_kernel(RolloutArgs a, SimtWeights w) {
     if (!last && !ev) {  // the tile's rows are one contiguous block of the time-major obs array
       float *dst = a.buf.obs + row0 * D;
       const int count = n_rows * D;
-      if (((row0 * D) & 3) == 0 && (count & 3) == 0) {
+      if (whole_pieces16(dst, count)) {
         for (int i = tid; i < count / 4; i += kSimtThreads)
           reinterpret_cast<float4 *>(dst)[i] = reinterpret_cast<const float4 *>(sm.obs)[i];
       } else {

@@ -452,15 +452,15 @@ rollout_tc_kernel(RolloutArgs a, const unsigned char *__restrict__ image, int ep
             }
             fence_async_smem();
             __syncwarp();
-            const size_t at = (static_cast<size_t>(k) * M + static_cast<size_t>(e0) * N + wg * S::RPW) * D;
+            float *obs_dst = a.buf.obs + (static_cast<size_t>(k) * M + static_cast<size_t>(e0) * N + wg * S::RPW) * D;
             const int count = n_mine * D;
-            if ((at & 3) == 0 && (count & 3) == 0) {
+            if (whole_pieces16(obs_dst, count)) {
               if (lane == 0) {
-                bulk_store(a.buf.obs + at, chunk, static_cast<uint32_t>(count) * 4u);
+                bulk_store(obs_dst, chunk, static_cast<uint32_t>(count) * 4u);
                 bulk_pending = true;
               }
             } else {
-              for (int i = lane; i < count; i += 32) a.buf.obs[at + i] = lds_f32(chunk + 4u * i);
+              for (int i = lane; i < count; i += 32) obs_dst[i] = lds_f32(chunk + 4u * i);
             }
           }
         }

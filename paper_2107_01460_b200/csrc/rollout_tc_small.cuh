@@ -249,7 +249,7 @@ rollout_tc_small_kernel(RolloutArgs a, const unsigned char *__restrict__ image, 
           const size_t row0 = static_cast<size_t>(k) * M + static_cast<size_t>(e0) * N;
           float *obs_dst = a.buf.obs + row0 * D;
           const int count = n_rows * D;
-          if (((row0 * D) & 3) == 0 && (count & 3) == 0) {
+          if (whole_pieces16(obs_dst, count)) {
             if (lane == 0) {
               bulk_store(obs_dst, stage_addr, static_cast<uint32_t>(count) * 4u);
               bulk_pending = true;

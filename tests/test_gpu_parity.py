@@ -377,3 +377,33 @@ def test_collect_host_delivers_the_bytes_of_run_and_gae(idx, n_envs, T):
             assert torch.equal(out[n][:rows], getattr(a, n)[:rows].cpu()), n
     assert np.array_equal(a.get_state(), b.get_state())
     assert a.status() == 0 and b.status() == 0
+
+
+@pytest.mark.parametrize("name,n_envs,T,precision", [
+    # one kernel form each: few rows (padded and not), 128 rows, two and three robots, recurrent, fp32
+    ("cfg0_tiny_8x8_2p2f_h64", 3, 10, BF16), ("cfg1_8x8_2p2f_h128", 201, 10, BF16), ("cfg1_8x8_2p2f_h128", 2401, 10, BF16),
+    ("wh0_tiny_8x8_2r2s_h64", 2399, 11, BF16), ("rec1_8x8_2p2f_gru64", 5, 10, BF16), ("rec1_8x8_2p2f_gru64", 301, 13, BF16),
+    ("cfg0_tiny_8x8_2p2f_h64", 7, 10, FP32), ("rec1_8x8_2p2f_gru64", 3, 10, FP32),
+    # three agents, 80 features: every piece starts on a boundary whatever the batch
+    ("cfg2_10x10_3p3f_h128", 7, 11, BF16)])
+def test_collect_host_where_a_piece_starts_off_a_16_byte_boundary(name, n_envs, T, precision):
+    """Two agents have 79 features, so after an odd number of steps of an odd number of environments the next row is 8 bytes
+    past a 16-byte boundary, where neither a bulk copy nor a 16-byte store may start (T = 10 is cut at steps 2, 5 and 7)."""
+    import torch
+
+    w = wl.workload(name)
+    if w["n_agents"] == 2:  # what the case is about
+        assert any((T * c // 4) * n_envs * w["n_agents"] * wl.obs_dim(w) % 4 for c in range(1, 4))
+    params = torch.from_numpy(wl.make_params(w, bias_scale=0.1))
+    cfg = binding.make_config(w, precision=precision, max_T=T, n_envs=n_envs, flags=binding.MAVA_FLAG_WRITE_LOGITS)
+    a, b = binding.Rollout(cfg), binding.Rollout(cfg)
+    names = ("obs", "actions", "logp", "values", "rewards", "dones", "adv", "ret", "logits")
+    out = {n: torch.empty_like(getattr(b, n), device="cpu").pin_memory() for n in names}
+    a.run(params.cuda(), T)
+    a.gae(wl.GAMMA, wl.LAMBDA)
+    b.collect_host(params.pin_memory(), T, wl.GAMMA, wl.LAMBDA, out)
+    for n in names:
+        rows = T + 1 if n == "values" else T
+        assert torch.equal(out[n][:rows], getattr(a, n)[:rows].cpu()), n
+    assert np.array_equal(a.get_state(), b.get_state())
+    assert a.status() == 0 and b.status() == 0
