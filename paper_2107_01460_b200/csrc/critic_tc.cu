@@ -36,7 +36,7 @@ struct CriticShape {
 // units 0..127 in the first half of each image, 128..255 in the second), c1 split into bf16 hi + lo
 // in two spare K columns of C1, and the fp32 vectors the epilogue of layer 2 needs.
 template <int N>
-__global__ void prep_critic_kernel(const float *__restrict__ params, unsigned char *__restrict__ image, ParamLayout L) {
+__global__ void prep_critic_kernel(const float *params, unsigned char *image, ParamLayout L) {
   using S = CriticShape<N>;
   constexpr int KJ = S::KJ, K1 = S::K1;
   wait_for_predecessor();
@@ -44,10 +44,10 @@ __global__ void prep_critic_kernel(const float *__restrict__ params, unsigned ch
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
   for (int i = tid; i < kCH * K1; i += nth) {
     const int n = i / K1, k = i - n * K1;
-    __nv_bfloat16 v = __float2bfloat16_rn(k < KJ ? params[L.C1 + static_cast<size_t>(n) * KJ + k] : 0.0f);
+    __nv_bfloat16 v = __float2bfloat16_rn(k < KJ ? __ldcg(params + L.C1 + static_cast<size_t>(n) * KJ + k) : 0.0f);
     if (k == KJ || k == KJ + 1) {
       __nv_bfloat16 hi, lo;
-      split_bf16(params[L.c1 + n], hi, lo);
+      split_bf16(__ldcg(params + L.c1 + n), hi, lo);
       v = (k == KJ) ? hi : lo;
     }
     at(0)[canon_offset(n, k, K1) / 2] = v;
@@ -56,12 +56,12 @@ __global__ void prep_critic_kernel(const float *__restrict__ params, unsigned ch
   for (int i = tid; i < kCH * kCH; i += nth) {
     const int n = i / kCH, k = i - n * kCH;
     reinterpret_cast<__nv_bfloat16 *>(l2 + S::C2_OFF)[canon_offset(n, k, kCH) / 2] =
-        __float2bfloat16_rn(params[L.C2 + static_cast<size_t>(n) * kCH + k]);
+        __float2bfloat16_rn(__ldcg(params + L.C2 + static_cast<size_t>(n) * kCH + k));
   }
   float *cv = reinterpret_cast<float *>(l2 + S::CV_OFF);
   for (int i = tid; i < 2 * kCH + 4; i += nth)
-    cv[i] = i < kCH ? __bfloat162float(__float2bfloat16_rn(params[L.Cv + i]))
-                    : (i == kCH ? params[L.cv] : (i < kCH + 4 ? 0.0f : params[L.c2 + i - kCH - 4]));
+    cv[i] = i < kCH ? __bfloat162float(__float2bfloat16_rn(__ldcg(params + L.Cv + i)))
+                    : (i == kCH ? __ldcg(params + L.cv) : (i < kCH + 4 ? 0.0f : __ldcg(params + L.c2 + i - kCH - 4)));
 }
 
 // ---- both layers in one kernel, on pairs of SMs --------------------------------------------------

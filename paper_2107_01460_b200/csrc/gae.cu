@@ -31,9 +31,8 @@ __device__ __forceinline__ void mbar_arrive_local(uint32_t bar) {
 }
 
 template <int L>
-__global__ void gae_kernel(const float *__restrict__ values, const float *__restrict__ rewards,
-                           const uint8_t *__restrict__ dones, float *__restrict__ adv,
-                           float *__restrict__ ret, int T, int E, int N, float gamma, float lambda) {
+__global__ void gae_kernel(const float *values, const float *rewards, const uint8_t *dones, float *adv, float *ret, int T, int E, int N,
+                           float gamma, float lambda) {
   wait_for_predecessor();
   extern __shared__ float sm[];  // [2][n_chunks][32]
   const int n_chunks = blockDim.y;
@@ -52,13 +51,13 @@ __global__ void gae_kernel(const float *__restrict__ values, const float *__rest
   for (int i = 0; i < L; ++i) {
     if (i < len) {
       const size_t t = static_cast<size_t>(t0 + i);
-      v[i] = values[t * M + col];
-      r[i] = rewards[t * M + col];
-      c[i] = dones[t * E + e] ? 0.0f : 1.0f;
+      v[i] = __ldcg(values + t * M + col);
+      r[i] = __ldcg(rewards + t * M + col);
+      c[i] = __ldcg(dones + t * E + e) ? 0.0f : 1.0f;
     }
   }
   // V at the step after the chunk
-  float v_after = active ? values[static_cast<size_t>(t0 + len) * M + col] : 0.0f;
+  float v_after = active ? __ldcg(values + static_cast<size_t>(t0 + len) * M + col) : 0.0f;
 
   float a_loc[L], p[L];
   float a_run = 0.0f, p_run = 1.0f;
@@ -100,8 +99,8 @@ __global__ void gae_kernel(const float *__restrict__ values, const float *__rest
 // read again here: streaming stores.
 template <int L, int THREADS, int MINB>
 __global__ void __launch_bounds__(THREADS, MINB)
-gae_kernel_v4(const float *__restrict__ values, const float *__restrict__ rewards, const uint8_t *__restrict__ dones,
-              float *__restrict__ adv, float *__restrict__ ret, int T, int E, int N, float gamma, float lambda) {
+gae_kernel_v4(const float *values, const float *rewards, const uint8_t *dones, float *adv, float *ret, int T, int E, int N, float gamma,
+              float lambda) {
   wait_for_predecessor();
   static_assert(4 * L <= 32, "one done bit per step and column");
   extern __shared__ float sm[];  // [2][n_chunks][32] float4
@@ -126,14 +125,14 @@ gae_kernel_v4(const float *__restrict__ values, const float *__restrict__ reward
   for (int i = 0; i < L; ++i) {
     if (i < len) {
       const size_t t = static_cast<size_t>(t0 + i);
-      v[i] = __ldg(v4 + t * M4 + q);
-      r[i] = __ldg(r4 + t * M4 + q);
+      v[i] = __ldcg(v4 + t * M4 + q);
+      r[i] = __ldcg(r4 + t * M4 + q);
       const uint8_t *d = dones + t * E;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) alive |= (__ldg(d + env[j]) ? 0u : 1u) << (4 * i + j);
+      for (int j = 0; j < 4; ++j) alive |= (__ldcg(d + env[j]) ? 0u : 1u) << (4 * i + j);
     }
   }
-  const float4 v_after = active ? __ldg(v4 + static_cast<size_t>(t0 + len) * M4 + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+  const float4 v_after = active ? __ldcg(v4 + static_cast<size_t>(t0 + len) * M4 + q) : make_float4(0.f, 0.f, 0.f, 0.f);
   auto keep = [&](int i) {
     return make_float4(static_cast<float>((alive >> (4 * i)) & 1u), static_cast<float>((alive >> (4 * i + 1)) & 1u),
                        static_cast<float>((alive >> (4 * i + 2)) & 1u), static_cast<float>((alive >> (4 * i + 3)) & 1u));
@@ -193,7 +192,7 @@ constexpr int kGaeStages = 3, kGaeL = 4;
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1)
 gae_tma_kernel(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_r,
-               const __grid_constant__ CUtensorMap map_d, float *__restrict__ adv, float *__restrict__ ret, int T, int E, int N, int C,
+               const __grid_constant__ CUtensorMap map_d, float *adv, float *ret, int T, int E, int N, int C,
                int W, int n_tiles, float gamma, float lambda, int *status, int debug_expire) {
   wait_for_predecessor();
   constexpr int L = kGaeL, S = kGaeStages;

@@ -1,10 +1,17 @@
 // Dependent launches.  A collection is three short kernels or more in a row (weight image, rollout, advantages) and a gradient
 // with its optimiser step four; launched one after the other each pays a launch gap of a few microseconds.  They are launched
 // with programmatic serialization instead: a kernel may start while the one before it still runs, does what needs nothing
-// from it (barriers, tensor memory, zeroed tiles) and then waits, in every thread, until that one is complete and its writes
-// are visible.  Every kernel that is launched like this waits, so a kernel's completion implies that of all before it.
-// A kernel in front of one whose blocks want an SM each does not let it start early: blocks that arrive while others still
-// sit on some SMs are doubled up on the rest (8x8 evaluation block 181 -> 192 us).
+// from it (barriers, tensor memory, zeroed tiles) and then waits until that one is complete and its writes are visible.
+// Rules for a kernel that is launched like this:
+//   - Every block waits, whatever it does before: a kernel's completion then implies that of all before it.  All threads of a
+//     block wait, but for those that only read what an even earlier kernel is known to have finished (the row loaders of
+//     ppo_net_tc_kernel inside mava_ppo_update; launch_ppo_grad has the argument).
+//   - Memory that a kernel in front may still be writing is not constant for the kernel's lifetime, so it must not be declared
+//     so: no __restrict__ on its parameters and no load through the non-coherent path (__ldg, ld.global.nc).  Either lets the
+//     compiler take a load for an invariant and move it over the wait.  Where loads should go out in a batch they are __ldcg.
+//   - A kernel that lets its successor start (dependents_may_start) does so for successors that have room beside it.  The
+//     weight-image kernels in front of a rollout do not: blocks that want an SM each and arrive while others still sit on
+//     some SMs are doubled up on the rest (8x8 evaluation block 181 -> 192 us).
 #pragma once
 #include <cuda_runtime.h>
 

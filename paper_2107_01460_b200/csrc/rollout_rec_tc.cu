@@ -50,36 +50,36 @@ struct RecTcSmem {
   uint32_t tmem_base;
 };
 
-__global__ void prep_rec_tc_kernel(const float *__restrict__ params, unsigned char *__restrict__ image, ParamLayout L, int D) {
+__global__ void prep_rec_tc_kernel(const float *params, unsigned char *image, ParamLayout L, int D) {
   wait_for_predecessor();
   auto bf = [&](uint32_t off) { return reinterpret_cast<__nv_bfloat16 *>(image + off); };
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
   for (int i = tid; i < kRH * kRK1; i += nth) {
     const int n = i / kRK1, k = i - n * kRK1;
-    bf(kW1)[canon_offset(n, k, kRK1) / 2] = __float2bfloat16_rn(k < D ? params[L.W1 + static_cast<size_t>(n) * D + k] : 0.0f);
+    bf(kW1)[canon_offset(n, k, kRK1) / 2] = __float2bfloat16_rn(k < D ? __ldcg(params + L.W1 + static_cast<size_t>(n) * D + k) : 0.0f);
   }
   for (int i = tid; i < 3 * kRH * kRH; i += nth) {
     const int n = i / kRH, k = i - n * kRH;
-    bf(kWih)[canon_offset(n, k, kRH) / 2] = __float2bfloat16_rn(params[L.Wih + i]);
-    bf(kWhh)[canon_offset(n, k, kRH) / 2] = __float2bfloat16_rn(params[L.Whh + i]);
+    bf(kWih)[canon_offset(n, k, kRH) / 2] = __float2bfloat16_rn(__ldcg(params + L.Wih + i));
+    bf(kWhh)[canon_offset(n, k, kRH) / 2] = __float2bfloat16_rn(__ldcg(params + L.Whh + i));
   }
   for (int i = tid; i < kHeadRows * kRH; i += nth) {
     const int n = i / kRH, k = i - n * kRH;
     float v = 0.0f;
-    if (n < kActions) v = params[L.Wa + static_cast<size_t>(n) * kRH + k];
-    else if (n == kActions) v = params[L.Wv + k];
+    if (n < kActions) v = __ldcg(params + L.Wa + static_cast<size_t>(n) * kRH + k);
+    else if (n == kActions) v = __ldcg(params + L.Wv + k);
     bf(kWh)[canon_offset(n, k, kRH) / 2] = __float2bfloat16_rn(v);
   }
   float *b1 = reinterpret_cast<float *>(image + kB1), *brz = reinterpret_cast<float *>(image + kBrz),
         *bin = reinterpret_cast<float *>(image + kBin), *bhn = reinterpret_cast<float *>(image + kBhn), *bh = reinterpret_cast<float *>(image + kBh);
   for (int i = tid; i < kRH; i += nth) {
-    b1[i] = params[L.b1 + i];
-    brz[i] = params[L.bih + i] + params[L.bhh + i];                      // r: both parts' biases
-    brz[kRH + i] = params[L.bih + kRH + i] + params[L.bhh + kRH + i];    // z
-    bin[i] = params[L.bih + 2 * kRH + i];
-    bhn[i] = params[L.bhh + 2 * kRH + i];
+    b1[i] = __ldcg(params + L.b1 + i);
+    brz[i] = __ldcg(params + L.bih + i) + __ldcg(params + L.bhh + i);                      // r: both parts' biases
+    brz[kRH + i] = __ldcg(params + L.bih + kRH + i) + __ldcg(params + L.bhh + kRH + i);    // z
+    bin[i] = __ldcg(params + L.bih + 2 * kRH + i);
+    bhn[i] = __ldcg(params + L.bhh + 2 * kRH + i);
   }
-  if (tid < 8) bh[tid] = tid < kActions ? params[L.ba + tid] : (tid == kActions ? params[L.bv] : 0.0f);
+  if (tid < 8) bh[tid] = tid < kActions ? __ldcg(params + L.ba + tid) : (tid == kActions ? __ldcg(params + L.bv) : 0.0f);
 }
 
 __device__ __forceinline__ uint64_t rdesc(uint32_t tile, int C, int k) { return smem_desc(tile + k * 256, 128, C * 16); }
@@ -97,7 +97,7 @@ __device__ __forceinline__ uint4 lds_v4(uint32_t addr) {
 
 template <int N, int F>
 __global__ void __launch_bounds__(kRecThreads, 1)
-rollout_rec_tc_kernel(RolloutArgs a, const unsigned char *__restrict__ image, float *__restrict__ hidden, int ept, int n_tiles) {
+rollout_rec_tc_kernel(RolloutArgs a, const unsigned char *image, float *hidden, int ept, int n_tiles) {
   constexpr int D = kObsFixed + N, K1 = kRK1, H = kRH;
   constexpr int EPW = 32 / N, RPW = EPW * N;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -417,7 +417,8 @@ size_t rec_tc_weight_bytes(const mava_config_t &) { return kRecImage; }
 
 cudaError_t launch_rollout_rec_tc(mava_rollout *h, const float *params_dev, const RolloutArgs &args) {
   if (h->cfg.hidden != kRH || h->D > kRK1) return cudaErrorNotSupported;
-  cudaError_t err = launch_dependent(prep_rec_tc_kernel, 32, 256, 0, h->stream, params_dev, static_cast<unsigned char *>(h->d_wtc),
+  // 48 blocks: one element of each gate matrix per thread
+  cudaError_t err = launch_dependent(prep_rec_tc_kernel, 48, 256, 0, h->stream, params_dev, static_cast<unsigned char *>(h->d_wtc),
                                      param_layout(h->cfg, h->D, 1), h->D);
   h->launches += 1;
   if (err != cudaSuccess) return err;

@@ -112,7 +112,7 @@ struct TcSmem {
 
 
 template <int N, int H, bool CENTRAL>
-__global__ void prep_tc_kernel(const float *__restrict__ params, unsigned char *__restrict__ image, ParamLayout L, int units) {
+__global__ void prep_tc_kernel(const float *params, unsigned char *image, ParamLayout L, int units) {
   using S = TcShape<N, H>;
   constexpr int D = S::D, K1 = S::K1;
   wait_for_predecessor();
@@ -120,23 +120,23 @@ __global__ void prep_tc_kernel(const float *__restrict__ params, unsigned char *
   const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
   for (int i = tid; i < H * K1; i += nth) {
     const int n = i / K1, k = i - n * K1;
-    __nv_bfloat16 v = __float2bfloat16_rn(k < D && n < units ? params[L.W1 + static_cast<size_t>(n) * D + k] : 0.0f);
+    __nv_bfloat16 v = __float2bfloat16_rn(k < D && n < units ? __ldcg(params + L.W1 + static_cast<size_t>(n) * D + k) : 0.0f);
     if (S::FOLD1 && (k == D || k == D + 1)) {
       __nv_bfloat16 hi, lo;
-      split_bf16(n < units ? params[L.b1 + n] : 0.0f, hi, lo);
+      split_bf16(n < units ? __ldcg(params + L.b1 + n) : 0.0f, hi, lo);
       v = (k == D) ? hi : lo;
     }
     at(S::W1_OFF)[canon_offset(n, k, K1) / 2] = v;
   }
   for (int i = tid; i < H * H; i += nth) {
     const int n = i / H, k = i - n * H;
-    at(S::W2_OFF)[canon_offset(n, k, H) / 2] = __float2bfloat16_rn(n < units && k < units ? params[L.W2 + static_cast<size_t>(n) * units + k] : 0.0f);
+    at(S::W2_OFF)[canon_offset(n, k, H) / 2] = __float2bfloat16_rn(n < units && k < units ? __ldcg(params + L.W2 + static_cast<size_t>(n) * units + k) : 0.0f);
   }
   for (int i = tid; i < kHeadRows * H; i += nth) {
     const int n = i / H, k = i - n * H;
     float v = 0.0f;
-    if (n < kActions && k < units) v = params[L.Wa + static_cast<size_t>(n) * units + k];
-    else if (n == kActions && k < units && !CENTRAL) v = params[L.Wv + k];  // the centralised critic has its own kernels
+    if (n < kActions && k < units) v = __ldcg(params + L.Wa + static_cast<size_t>(n) * units + k);
+    else if (n == kActions && k < units && !CENTRAL) v = __ldcg(params + L.Wv + k);  // the centralised critic has its own kernels
     at(S::WH_OFF)[canon_offset(n, k, H) / 2] = __float2bfloat16_rn(v);
   }
   // bias tiles of the hidden layers (hi, lo, then zeros), the heads' biases as fp32, the ones tile
@@ -147,9 +147,9 @@ __global__ void prep_tc_kernel(const float *__restrict__ params, unsigned char *
     int n;
     if (r < H) {
       if (S::FOLD1) continue;
-      b = r < units ? params[L.b1 + r] : 0.0f; off = S::B1_OFF; n = r;
+      b = r < units ? __ldcg(params + L.b1 + r) : 0.0f; off = S::B1_OFF; n = r;
     } else {
-      b = r - H < units ? params[L.b2 + r - H] : 0.0f; off = S::B2_OFF; n = r - H;
+      b = r - H < units ? __ldcg(params + L.b2 + r - H) : 0.0f; off = S::B2_OFF; n = r - H;
     }
     __nv_bfloat16 hi, lo;
     split_bf16(b, hi, lo);
@@ -157,7 +157,7 @@ __global__ void prep_tc_kernel(const float *__restrict__ params, unsigned char *
   }
   if (tid < 8)
     reinterpret_cast<float *>(image + S::BH_OFF)[tid] =
-        tid < kActions ? params[L.ba + tid] : ((tid == kActions && !CENTRAL) ? params[L.bv] : 0.0f);
+        tid < kActions ? __ldcg(params + L.ba + tid) : ((tid == kActions && !CENTRAL) ? __ldcg(params + L.bv) : 0.0f);
   for (int i = tid; i < kTileRows * 16; i += nth) {
     const int r = i / 16, k = i - r * 16;
     at(S::ONES_OFF)[canon_offset(r, k, 16) / 2] = __float2bfloat16_rn(k < 2 ? 1.0f : 0.0f);
@@ -314,7 +314,7 @@ __device__ __forceinline__ void expand_quads(const QuadPlan<D, K1> &p, uint32_t 
 // ---- the rollout kernel ------------------------------------------------------------------------
 template <int N, int F, int H, bool EVAL, int ENV = 0>
 __global__ void __launch_bounds__(TcShape<N, H>::THREADS, 1)
-rollout_tc_kernel(RolloutArgs a, const unsigned char *__restrict__ image, int ept, int n_tiles, int groups) {
+rollout_tc_kernel(RolloutArgs a, const unsigned char *image, int ept, int n_tiles, int groups) {
   using S = TcShape<N, H>;
   constexpr int D = S::D, K1 = S::K1;
   constexpr bool PP = S::PINGPONG;

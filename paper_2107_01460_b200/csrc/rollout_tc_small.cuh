@@ -129,7 +129,7 @@ constexpr int kSmallIssuer = 3, kSmallHelper = 4;  // warps
 
 template <int N, int F, int H, int RB, bool EVAL, int ENV>
 __global__ void __launch_bounds__(SmallShape<N, H, RB>::THREADS, 1)
-rollout_tc_small_kernel(RolloutArgs a, const unsigned char *__restrict__ image, int ept) {
+rollout_tc_small_kernel(RolloutArgs a, const unsigned char *image, int ept) {
   using S = TcShape<N, H>;
   using Q = SmallShape<N, H, RB>;
   constexpr int D = S::D, K1 = S::K1;

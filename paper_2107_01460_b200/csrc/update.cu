@@ -290,15 +290,14 @@ __global__ void __launch_bounds__(256) moments_kernel(Moments m) {  // of the ad
   moments_block(m);
 }
 
-__global__ void adam_kernel(float *__restrict__ params, const float *__restrict__ grad, float *__restrict__ m, float *__restrict__ v,
-                            size_t n, const double *__restrict__ stats, float max_norm, float lr, float beta1, float beta2,
-                            float eps, float corr1, float corr2) {
+__global__ void adam_kernel(float *params, const float *grad, float *m, float *v, size_t n, const double *stats, float max_norm, float lr,
+                            float beta1, float beta2, float eps, float corr1, float corr2) {
   dependents_may_start();
   wait_for_predecessor();
-  const float norm = static_cast<float>(stats[2]);
+  const float norm = static_cast<float>(__ldcg(stats + 2));
   const float scale = max_norm / fmaxf(norm, max_norm);
   for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const float g = grad[i] * scale;
+    const float g = __ldcg(grad + i) * scale;
     const float mi = beta1 * m[i] + (1.0f - beta1) * g, vi = beta2 * v[i] + (1.0f - beta2) * g * g;
     m[i] = mi; v[i] = vi;
     params[i] -= lr * (mi / corr1) / (sqrtf(vi / corr2) + eps);

@@ -44,7 +44,7 @@ __device__ __forceinline__ long long real_row(const UpdRows &rows, long long q) 
 // of one between two of them, so a batch costs one round trip (with plain conditional loads a batch of 48 took 22 k cycles).
 __device__ __forceinline__ float ldg_if(const float *p, bool pred) {
   float v;
-  asm volatile("{\n.reg .pred q;\nsetp.ne.u32 q, %2, 0;\nmov.f32 %0, 0f00000000;\n@q ld.global.nc.L1::no_allocate.f32 %0, [%1];\n}"
+  asm volatile("{\n.reg .pred q;\nsetp.ne.u32 q, %2, 0;\nmov.f32 %0, 0f00000000;\n@q ld.global.L1::no_allocate.f32 %0, [%1];\n}"
                : "=f"(v)
                : "l"(p), "r"(static_cast<uint32_t>(pred)));
   return v;
@@ -228,7 +228,7 @@ struct IdentityMap {
   __device__ __forceinline__ long long operator()(int j) const { return j; }
 };
 template <class Map>
-__global__ void __launch_bounds__(kReduceThreads) reduce_slices_kernel(const float *__restrict__ partial, int len, int n_slices, float *__restrict__ grad, TermSums terms,
+__global__ void __launch_bounds__(kReduceThreads) reduce_slices_kernel(const float *partial, int len, int n_slices, float *grad, TermSums terms,
                                                             Moments norm, Map map) {
   dependents_may_start();
   wait_for_predecessor();
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(256) grad_moments_kernel(Moments m, int len, M
   if (threadIdx.x < kGradLanes)
     for (int j = static_cast<int>(blockIdx.x) * kGradLanes + static_cast<int>(threadIdx.x); j < len; j += kMomentBlocks * kGradLanes) {
       const long long p = map(j);
-      const float v = p >= 0 ? m.x[p] : 0.0f;
+      const float v = p >= 0 ? __ldcg(m.x + p) : 0.0f;
       if (p >= 0) { a += v; b += static_cast<double>(v) * v; }
     }
   moments_finish(m, a, b);

@@ -91,7 +91,7 @@ __device__ __forceinline__ void PrepImage::operator()(int tid, int nth) const {
       j -= 2 * kUH;
       real = j <= kActions; src = j < kActions ? L.ba + j : L.bv; at = kImgBh + 4 * j; wide = true;
     }
-    const float v = real ? params[src] : 0.0f;
+    const float v = real ? __ldcg(params + src) : 0.0f;
     if (wide) *reinterpret_cast<float *>(image + at) = v;
     else *reinterpret_cast<__nv_bfloat16 *>(image + at) = __float2bfloat16_rn(v);
   }
@@ -132,8 +132,8 @@ struct SliceMap {
 };
 
 __global__ void __launch_bounds__(kUThreads, 1)
-ppo_net_tc_kernel(const unsigned char *__restrict__ image, UpdRows rows, UpdHyper hp, const double *__restrict__ adv_stats,
-                  float *__restrict__ partial, double *__restrict__ term_partial, int *status, int D, bool rows_ready) {
+ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const double *adv_stats,
+                  float *partial, double *term_partial, int *status, int D, bool rows_ready) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   UtcSmem &sm = *reinterpret_cast<UtcSmem *>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -187,8 +187,8 @@ ppo_net_tc_kernel(const unsigned char *__restrict__ image, UpdRows rows, UpdHype
                  dht = smem_u32(sm.dhead);
   const uint32_t b1 = smem_u32(sm.img + kImgB1), b2 = smem_u32(sm.img + kImgB2);
   const float *bh = reinterpret_cast<const float *>(sm.img + kImgBh);
-  const float mean = loader ? 0.0f : static_cast<float>(adv_stats[0]);
-  const float inv_std = loader ? 0.0f : 1.0f / (static_cast<float>(adv_stats[1]) + 1e-8f);
+  const float mean = loader ? 0.0f : static_cast<float>(__ldcg(adv_stats));
+  const float inv_std = loader ? 0.0f : 1.0f / (static_cast<float>(__ldcg(adv_stats + 1)) + 1e-8f);
   const float inv_n = 1.0f / static_cast<float>(rows.n);
   const long long n_tiles = (rows.n + kUR - 1) / kUR;
   const int my_tiles = blockIdx.x < n_tiles ? static_cast<int>((n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;

@@ -140,24 +140,24 @@ __device__ __forceinline__ void Prep256::operator()(int tid, int nth) const {
   for (int i = tid; i < net.slabs * kH * kK1; i += nth) {
     const int a = i / (kH * kK1), r = i - a * (kH * kK1), n = r / kK1, k = r - n * kK1;
     reinterpret_cast<__nv_bfloat16 *>(image + static_cast<size_t>(a) * kImgW2)[canon_offset(n, k, kK1) / 2] =
-        __float2bfloat16_rn(k < D ? params[net.W1 + static_cast<size_t>(n) * net.w1_ld + a * D + k] : 0.0f);
+        __float2bfloat16_rn(k < D ? __ldcg(params + net.W1 + static_cast<size_t>(n) * net.w1_ld + a * D + k) : 0.0f);
   }
   unsigned char *rest = image + static_cast<size_t>(net.slabs) * kImgW2 - kImgW2;  // so that rest + kImgX is where X lies
   auto bf = [&](uint32_t off) { return reinterpret_cast<__nv_bfloat16 *>(rest + off); };
   for (int i = tid; i < kH * kH; i += nth) {
     const int n = i / kH, k = i - n * kH;
-    bf(kImgW2)[canon_offset(n, k, kH) / 2] = __float2bfloat16_rn(params[net.W2 + static_cast<size_t>(n) * kH + k]);
+    bf(kImgW2)[canon_offset(n, k, kH) / 2] = __float2bfloat16_rn(__ldcg(params + net.W2 + static_cast<size_t>(n) * kH + k));
   }
   for (int i = tid; i < kHeads * kH; i += nth) {
     const int n = i / kH, k = i - n * kH;
     float v = 0.0f;
-    if (n < kActions && net.has_actor) v = params[net.Wa + static_cast<size_t>(n) * kH + k];
-    else if (n == kActions && net.has_value) v = params[net.Wv + k];
+    if (n < kActions && net.has_actor) v = __ldcg(params + net.Wa + static_cast<size_t>(n) * kH + k);
+    else if (n == kActions && net.has_value) v = __ldcg(params + net.Wv + k);
     bf(kImgWh)[canon_offset(n, k, kH) / 2] = __float2bfloat16_rn(v);
   }
   float *b1 = reinterpret_cast<float *>(rest + kImgB1), *b2 = reinterpret_cast<float *>(rest + kImgB2), *bh = reinterpret_cast<float *>(rest + kImgBh);
-  for (int i = tid; i < kH; i += nth) { b1[i] = params[net.b1 + i]; b2[i] = params[net.b2 + i]; }
-  if (tid < 8) bh[tid] = (tid < kActions && net.has_actor) ? params[net.ba + tid] : ((tid == kActions && net.has_value) ? params[net.bv] : 0.0f);
+  for (int i = tid; i < kH; i += nth) { b1[i] = __ldcg(params + net.b1 + i); b2[i] = __ldcg(params + net.b2 + i); }
+  if (tid < 8) bh[tid] = (tid < kActions && net.has_actor) ? __ldcg(params + net.ba + tid) : ((tid == kActions && net.has_value) ? __ldcg(params + net.bv) : 0.0f);
 }
 
 __device__ __forceinline__ uint64_t desc_k(uint32_t tile, int C, int k) { return smem_desc(tile + k * 256, 128, C * 16); }

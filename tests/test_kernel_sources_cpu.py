@@ -1,0 +1,57 @@
+"""Rules of the kernel sources that no output shows until a compiler makes use of them: read from the sources themselves."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2107_01460_b200", "csrc")
+
+
+def _sources():
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh"))):
+        text = re.sub(r"/\*.*?\*/", "", open(path).read(), flags=re.S)
+        yield os.path.basename(path), re.sub(r"//[^\n]*", "", text)
+
+
+def _closing(text, at, pair):
+    depth = 0
+    for i in range(at, len(text)):
+        depth += (text[i] == pair[0]) - (text[i] == pair[1])
+        if depth == 0:
+            return i
+    raise AssertionError("unbalanced")
+
+
+def _kernels():
+    """(file, name, parameter list, body) of every __global__ function that is defined in the sources."""
+    for name, text in _sources():
+        for m in re.finditer(r"__global__\b", text):
+            at = m.end()
+            while True:  # return type and attributes, then the name in front of the parameter list
+                word = re.compile(r"\s*(\w+)\s*").match(text, at)
+                at = word.end()
+                if word.group(1).startswith("__"):
+                    at = _closing(text, at, "()") + 1
+                elif word.group(1) != "void":
+                    break
+            close = _closing(text, at, "()")
+            start = text.index("{", close)
+            yield name, word.group(1), text[at:close], text[start:_closing(text, start, "{}") + 1]
+
+
+def test_every_kernel_is_found():
+    names = [k for _, k, _, _ in _kernels()]
+    assert len(names) == len(set(names)) == sum(t.count("__global__") for _, t in _sources())
+    assert {"rollout_tc_kernel", "gae_kernel_v4", "critic_kernel", "ppo_net_tc_kernel", "adam_kernel"} <= set(names)
+
+
+@pytest.mark.parametrize("file,name,params,body", [pytest.param(*k, id=k[1]) for k in _kernels() if "wait_for_predecessor()" in k[3]])
+def test_a_dependent_kernel_declares_nothing_constant_that_its_predecessor_may_write(file, name, params, body):
+    assert "__restrict__" not in params, f"{file}: {name}"
+    assert not re.search(r"\b__ldg\s*\(", body), f"{file}: {name}"
+
+
+def test_no_load_takes_the_non_coherent_path_by_hand():
+    for name, text in _sources():
+        assert "ld.global.nc" not in text, name
