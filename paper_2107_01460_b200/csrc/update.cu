@@ -395,7 +395,7 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
   cudaStream_t st = h->stream;
   UpdRows rows{};
   rows.x = h->buf.obs; rows.actions = h->buf.actions; rows.logp_old = h->buf.logp; rows.adv = h->buf.adv; rows.n = R;
-  rows.env_ids = env_ids_dev; rows.n_ids = n_env; rows.E = E; rows.per_env = N;
+  set_minibatch(rows, env_ids_dev, n_env, E, N);
   if (!central) { rows.value_old = h->buf.values; rows.ret = h->buf.ret; rows.vstride = 1; }
 
   if (update_takes_tensor_cores(cfg, D)) {
@@ -411,7 +411,7 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
 
   UpdRows crows{};  // the centralised critic's: a row is an environment-step
   crows.x = h->buf.obs; crows.value_old = h->buf.values; crows.ret = h->buf.ret; crows.vstride = N; crows.n = S;
-  crows.env_ids = env_ids_dev; crows.n_ids = n_env; crows.E = E; crows.per_env = 1;
+  set_minibatch(crows, env_ids_dev, n_env, E, 1);
 
   // H = 256 on the tensor cores: the actor / shared-torso net and, one input slab per agent, the centralised critic's
   if (update_takes_tensor_cores_256(cfg, D)) {

@@ -27,17 +27,51 @@ struct UpdRows {
   // nullptr = every environment in order (row q is row q of the arrays)
   const int32_t *env_ids;
   int n_ids, E, per_env;
+  uint64_t per_step_recip, per_env_recip;  // of n_ids * per_env and of per_env (quotient), in 64 and in 32 bits
+  uint32_t per_step_recip32, per_env_recip32;
 };
+inline void set_minibatch(UpdRows &rows, const int32_t *env_ids, int n_ids, int E, int per_env) {
+  const uint64_t per_step = static_cast<uint64_t>(n_ids) * per_env;
+  rows.env_ids = env_ids; rows.n_ids = n_ids; rows.E = E; rows.per_env = per_env;
+  rows.per_step_recip = ~uint64_t{0} / per_step; rows.per_env_recip = ~uint64_t{0} / per_env;
+  rows.per_step_recip32 = static_cast<uint32_t>(~uint32_t{0} / per_step); rows.per_env_recip32 = ~uint32_t{0} / per_env;
+}
 
-// Row of the trajectory arrays behind row q of the batch; -1 when the environment index is out of range.  (32-bit divisions:
-// a row is 340 bytes of observation alone, so the rows that fit a GPU are far below 2^31.)
-__device__ __forceinline__ long long real_row(const UpdRows &rows, long long q) {
-  if (!rows.env_ids) return q;
-  const uint32_t per_env = static_cast<uint32_t>(rows.per_env), per_step = static_cast<uint32_t>(rows.n_ids) * per_env, q32 = static_cast<uint32_t>(q);
-  const uint32_t t = q32 / per_step, rem = q32 - t * per_step, i = rem / per_env, slot = rem - i * per_env;
+// floor(q / d) and the remainder by recip = floor((2^w - 1) / d), w = 32 or 64 the width: the product's upper half is the
+// quotient or one less, because q recip / 2^w > q / d - 1.
+__device__ __forceinline__ uint32_t mul_high(uint32_t a, uint32_t b) { return __umulhi(a, b); }
+__device__ __forceinline__ uint64_t mul_high(uint64_t a, uint64_t b) { return __umul64hi(a, b); }
+template <class U>
+__device__ __forceinline__ U quotient(U q, U d, U recip, U &rem) {
+  U t = mul_high(q, recip);
+  rem = q - t * d;
+  if (rem >= d) { ++t; rem -= d; }
+  return t;
+}
+// Row of the trajectory arrays behind row q of the batch; -1 when the environment index is out of range.  U holds the batch's
+// row numbers: 32 bits for what is cut from a trajectory without repetition (a row is 340 bytes of observation alone, so
+// fewer than 2^31 fit a GPU); a minibatch that repeats environments may be longer than its trajectory and need 64.
+template <class U>
+__device__ __forceinline__ long long real_row_as(const UpdRows &rows, U q) {
+  const U per_env = static_cast<U>(rows.per_env);
+  U rem, slot, t, i;
+  if constexpr (sizeof(U) == 4) {
+    t = quotient(q, static_cast<U>(rows.n_ids) * per_env, rows.per_step_recip32, rem);
+    i = quotient(rem, per_env, rows.per_env_recip32, slot);
+  } else {
+    t = quotient(q, static_cast<U>(rows.n_ids) * per_env, rows.per_step_recip, rem);
+    i = quotient(rem, per_env, rows.per_env_recip, slot);
+  }
   const int e = rows.env_ids[i];
   if (e < 0 || e >= rows.E) return -1;
-  return static_cast<long long>((t * static_cast<uint32_t>(rows.E) + static_cast<uint32_t>(e)) * per_env + slot);
+  return static_cast<long long>((static_cast<uint32_t>(t) * static_cast<uint32_t>(rows.E) + static_cast<uint32_t>(e)) * static_cast<uint32_t>(rows.per_env) +
+                                static_cast<uint32_t>(slot));
+}
+__device__ __forceinline__ bool rows_need_64_bits(const UpdRows &rows, long long n) { return rows.env_ids && (n >> 32) != 0; }
+__device__ __forceinline__ long long real_row(const UpdRows &rows, long long q) {
+  if (!rows.env_ids) return q;
+  if (rows_need_64_bits(rows, rows.n)) return real_row_as<uint64_t>(rows, static_cast<uint64_t>(q));
+  return real_row_as<uint32_t>(rows, static_cast<uint32_t>(q));
 }
 
 // A predicated load (zero otherwise), in program order with its like: the compiler neither branches around it nor puts a use
@@ -117,21 +151,29 @@ __device__ __forceinline__ void moments_finish(const Moments &m, double a, doubl
   const double mean = a / static_cast<double>(m.n), var = fmax(b / static_cast<double>(m.n) - mean * mean, 0.0);
   m.out[0] = mean; m.out[1] = sqrt(var); m.out[2] = sqrt(b);
 }
-__device__ __forceinline__ void moments_block(const Moments &m) {
-  constexpr int kBatch = 8;  // loads in flight per thread (one at a time: 44 us for 16.8 million elements)
+template <bool WIDE>
+__device__ __forceinline__ void moments_sums(const Moments &m, double &a, double &b) {
+  // loads in flight per thread (one at a time: 44 us for 16.8 million elements); the wide form, of which a batch takes seconds, must
+  // not cost the kernel registers, i.e. blocks beside those of the kernels in front (58 instead of 32: 0.35 us a minibatch)
+  constexpr int kBatch = WIDE ? 1 : 8;
   constexpr long long kStep = 256LL * kMomentBlocks;
-  double a = 0.0, b = 0.0;
   for (long long i = blockIdx.x * 256LL + threadIdx.x; i < m.n; i += kBatch * kStep) {
     float v[kBatch];
 #pragma unroll
     for (int k = 0; k < kBatch; ++k) {
-      const long long q = i + k * kStep, row = real_row(m.map, q < m.n ? q : i);  // (loads without a branch around them)
+      const long long q = i + k * kStep, in = q < m.n ? q : i;  // (loads without a branch around them)
+      const long long row = !m.map.env_ids ? in : (WIDE ? real_row_as<uint64_t>(m.map, static_cast<uint64_t>(in)) : real_row_as<uint32_t>(m.map, static_cast<uint32_t>(in)));
       v[k] = __ldcg(m.x + (row >= 0 ? row : 0));
       if (q >= m.n || row < 0) v[k] = 0.0f;
     }
 #pragma unroll
     for (int k = 0; k < kBatch; ++k) { a += v[k]; b += static_cast<double>(v[k]) * v[k]; }
   }
+}
+__device__ __forceinline__ void moments_block(const Moments &m) {
+  double a = 0.0, b = 0.0;
+  if (rows_need_64_bits(m.map, m.n)) moments_sums<true>(m, a, b);
+  else moments_sums<false>(m, a, b);
   moments_finish(m, a, b);
 }
 // What a gradient call starts with: the advantages' moments and, by the other blocks, the weight image (prep(i, n): thread i

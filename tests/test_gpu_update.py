@@ -329,3 +329,26 @@ def test_h256_update_where_its_tiles_and_rings_turn_over(idx, n_envs, T):
     terms2, grad2 = ro.ppo_grad(new)
     assert torch.equal(grad, grad2) and torch.equal(terms, terms2)
     ro.close()
+
+
+@pytest.mark.parametrize("idx,T", [(0, 256), (2, 128)])
+def test_a_batch_of_more_than_2_to_the_32_rows(idx, T):
+    """Environments may be repeated in a minibatch, so it can be longer than its trajectory.  Every environment taken the same
+    number of times gives the loss terms of the plain call (their sums are kept in double: what is left is the order, below
+    1e-9).  The returns are made to depend on the step, so that rows of wrong steps would show in the value term."""
+    import torch
+
+    n_envs = 64
+    w, ro, params = _rolled_out(idx, n_envs, T, BF16, flags=0)
+    ro.ret.copy_(torch.arange(T, device="cuda", dtype=torch.float32).view(T, 1, 1).expand_as(ro.ret) / T)
+    per_env = T * w["n_agents"]
+    repeats = int(1.25 * 2**32) // (per_env * n_envs)
+    assert repeats * n_envs * per_env > 2**32
+    ids = torch.arange(n_envs, dtype=torch.int32, device="cuda").repeat(repeats)
+    want, _ = ro.ppo_grad(params)
+    got, grad = ro.ppo_grad(params, env_ids=ids)
+    assert ro.status() == binding.MAVA_OK
+    want, got = want.cpu().numpy(), got.cpu().numpy()
+    assert np.all(np.abs(got - want) <= 1e-6 * (1 + np.abs(want))), (got, want)  # (the terms are stored in binary32)
+    assert bool(torch.isfinite(grad).all())
+    ro.close()
