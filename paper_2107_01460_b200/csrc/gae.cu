@@ -30,15 +30,19 @@ __device__ __forceinline__ void mbar_arrive_local(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-template <int L>
-__global__ void gae_kernel(const float *values, const float *rewards, const uint8_t *dones, float *adv, float *ret, int T, int E, int N,
+// COLS columns by up to 32 chunks of L steps a block.  A thread keeps five floats per step, so the longer chunks take half as
+// many columns: 1024 threads of more than 64 registers do not fit an SM, and such a block is not launched at all.  (One block
+// per SM as the least, for chunks of eight only: it gives the loads 59 registers instead of 42, 5.5 against 5.9 us for 600 columns x
+// 256 steps; with sixteen and 32 it would make them spill.)
+template <int L, int COLS>
+__global__ void __launch_bounds__(32 * COLS, L == 8 ? 1 : 0) gae_kernel(const float *values, const float *rewards, const uint8_t *dones, float *adv, float *ret, int T, int E, int N,
                            float gamma, float lambda) {
   wait_for_predecessor();
   extern __shared__ float sm[];  // [2][n_chunks][32]
   const int n_chunks = blockDim.y;
-  float *sA = sm, *sP = sm + n_chunks * kGaeCols;
+  float *sA = sm, *sP = sm + n_chunks * COLS;
   const size_t M = static_cast<size_t>(E) * N;
-  const size_t col = static_cast<size_t>(blockIdx.x) * kGaeCols + threadIdx.x;
+  const size_t col = static_cast<size_t>(blockIdx.x) * COLS + threadIdx.x;
   const int chunk = threadIdx.y;
   const int t0 = chunk * L;
   const bool active = col < M && t0 < T;
@@ -72,13 +76,13 @@ __global__ void gae_kernel(const float *values, const float *rewards, const uint
       p[i] = p_run;
     }
   }
-  sA[chunk * kGaeCols + threadIdx.x] = a_run;  // value at the chunk's first step (A_in = 0)
-  sP[chunk * kGaeCols + threadIdx.x] = p_run;
+  sA[chunk * COLS + threadIdx.x] = a_run;  // value at the chunk's first step (A_in = 0)
+  sP[chunk * COLS + threadIdx.x] = p_run;
   __syncthreads();
   if (!active) return;
   float a_in = 0.0f;  // A at the first step of the next chunk
   for (int k = n_chunks - 1; k > chunk; --k)
-    a_in = sA[k * kGaeCols + threadIdx.x] + sP[k * kGaeCols + threadIdx.x] * a_in;
+    a_in = sA[k * COLS + threadIdx.x] + sP[k * COLS + threadIdx.x] * a_in;
 #pragma unroll
   for (int i = 0; i < L; ++i) {
     if (i < len) {
@@ -350,12 +354,12 @@ gae_tma_kernel(const __grid_constant__ CUtensorMap map_v, const __grid_constant_
 cudaError_t launch_gae(mava_rollout *h, float gamma, float lambda) {
   const int T = h->last_T, E = h->cfg.n_envs, N = h->cfg.n_agents;
   const size_t M = static_cast<size_t>(E) * N;
-  const unsigned blocks = static_cast<unsigned>((M + kGaeCols - 1) / kGaeCols);
   const mava_buffers_t &b = h->buf;
-  auto go = [&](auto kern, int L) {
+  auto go = [&](auto kern, int L, int cols) {
     const int n_chunks = (T + L - 1) / L;
-    const size_t smem = 2 * static_cast<size_t>(n_chunks) * kGaeCols * sizeof(float);
-    return launch_dependent(kern, blocks, dim3(kGaeCols, n_chunks), smem, h->stream, b.values, b.rewards, b.dones, b.adv, b.ret, T, E, N, gamma, lambda);
+    const size_t smem = 2 * static_cast<size_t>(n_chunks) * cols * sizeof(float);
+    return launch_dependent(kern, static_cast<unsigned>((M + cols - 1) / cols), dim3(cols, n_chunks), smem, h->stream, b.values, b.rewards, b.dones,
+                            b.adv, b.ret, T, E, N, gamma, lambda);
   };
   // the float4 variant pays off once there are enough columns to fill the GPU with its larger blocks
   const bool vec = M % 4 == 0 && M >= 16384 && reinterpret_cast<uintptr_t>(b.values) % 16 == 0 && reinterpret_cast<uintptr_t>(b.rewards) % 16 == 0 &&
@@ -404,9 +408,9 @@ cudaError_t launch_gae(mava_rollout *h, float gamma, float lambda) {
   h->launches += 1;
   if (vec && T <= 4 * 16) return go4(gae_kernel_v4<4, 512, 2>, 4);
   if (vec && T <= 4 * 32) return go4(gae_kernel_v4<4, 1024, 1>, 4);
-  if (T <= 8 * 32) return go(gae_kernel<8>, 8);
-  if (T <= 16 * 32) return go(gae_kernel<16>, 16);
-  if (T <= 32 * 32) return go(gae_kernel<32>, 32);
+  if (T <= 8 * 32) return go(gae_kernel<8, 32>, 8, 32);
+  if (T <= 16 * 32) return go(gae_kernel<16, 16>, 16, 16);
+  if (T <= 32 * 32) return go(gae_kernel<32, 16>, 32, 16);
   return cudaErrorInvalidValue;
 }
 

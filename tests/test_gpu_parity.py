@@ -5,7 +5,7 @@ import pytest
 import oracle
 from paper_2107_01460_b200 import binding, workloads as wl
 
-from parity import check_against_oracle, run_gpu
+from parity import GAE_TOL, check_against_oracle, run_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -277,6 +277,27 @@ def test_gae_on_random_trajectories(idx, n_envs, T):
         ga, gr = ro.adv.cpu().numpy(), ro.ret.cpu().numpy()
         assert np.max(np.abs(ga - adv) / np.maximum(1, np.abs(adv))) <= 1e-5
         assert np.max(np.abs(gr - ret) / np.maximum(1, np.abs(ret))) <= 1e-5
+
+
+@pytest.mark.parametrize("idx,n_envs,T", [(1, 33, 256), (1, 33, 257), (1, 300, 320), (3, 5, 321), (1, 8, 512), (2, 47, 513), (0, 7, 777),
+                                          (1, 300, 1000), (2, 5488, 1024)])
+def test_gae_on_long_trajectories(idx, n_envs, T):
+    """Up to MAVA_GAE_MAX_T steps: the last length of each chunk size and the first of the next (blocks of 1024 threads with more
+    than 64 registers each are refused at launch, which once was every length above 320)."""
+    import torch
+
+    w = wl.workload(idx)
+    ro = binding.Rollout(binding.make_config(w, precision=BF16, max_T=T, n_envs=n_envs))
+    ro.run(torch.from_numpy(wl.make_params(w)).cuda(), T)
+    g = torch.Generator(device="cuda").manual_seed(T)
+    ro.values.copy_(torch.randn(ro.values.shape, generator=g, device="cuda"))
+    ro.rewards.copy_(torch.rand(ro.rewards.shape, generator=g, device="cuda"))
+    ro.dones.copy_((torch.rand(ro.dones.shape, generator=g, device="cuda") < 0.02).to(torch.uint8))
+    ro.gae(0.99, 0.95)
+    assert ro.status() == binding.MAVA_OK
+    adv, ret = oracle.gae(ro.values.cpu().numpy(), ro.rewards.cpu().numpy(), ro.dones.cpu().numpy(), float(np.float32(0.99)), float(np.float32(0.95)))
+    assert np.max(np.abs(ro.adv.cpu().numpy() - adv) / np.maximum(1, np.abs(adv))) <= GAE_TOL
+    assert np.max(np.abs(ro.ret.cpu().numpy() - ret) / np.maximum(1, np.abs(ret))) <= GAE_TOL
 
 
 # ---- tensor-core path: determinism, continuation, sharding, forcing, degenerate sizes ----------
