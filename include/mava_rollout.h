@@ -272,8 +272,9 @@ int mava_rollout_collect_host(mava_rollout_t *h, const float *params_host, int32
  * re-laid-out weights) lives in one static device array of MAVA_STATIC_SCRATCH_BYTES that every
  * GPU loading the library holds until the process exits.
  *   - The scratch of a shape is 256 bytes + 60 bytes per environment + the re-laid-out weights, each part
- *     rounded up to 256 bytes.  The weights depend on the shape and the precision: bf16 images take 18 KB
- *     (H = 64), 70 KB (H = 128) or 205 KB (H = 256, about 13 000 environments fit beside them); the fp32 path
+ *     rounded up to 256 bytes.  The weights depend on the shape and the precision: bf16 images take 29 KB
+ *     (H = 64; 70 KB for up to 8192 environments without a flag for the 128-row kernel; 16 900 environments fit), 70 KB
+ *     (H = 128) or 205 KB (H = 256, about 13 000 environments fit beside them); the fp32 path
  *     keeps 4 bytes per parameter (24 KB ... 350 KB for the shared-torso shapes, 930 KB with the centralised
  *     critic, which leaves room for about 1 600 environments).  A shape whose scratch is larger than the
  *     array is refused with MAVA_ERR_CAPACITY, and so is T > cfg->max_T.  The bf16 path with the centralised

@@ -752,13 +752,17 @@ rollout_tc_kernel(RolloutArgs a, const unsigned char *image, int ept, int n_tile
 
 #include "rollout_tc_small.cuh"
 
+// SMs that the few-rows form counts on at most (no GPU has more): the size of the weight image is settled for all devices alike.
+constexpr int kFewRowsMaxSms = 512;
+
 // Rows per tile of the few-rows form that serves this batch (0: the 128-row kernel).
 template <int N, int H>
-int few_rows_tile(const mava_rollout *h, int sms) {
+int few_rows_tile(const mava_config_t &cfg, int sms) {
   if constexpr (H == kTileRows) {
-    if ((h->cfg.flags & (MAVA_FLAG_WIDE_TILES | MAVA_FLAG_HIDDEN_IN_TMEM)) == 0) {  // either flag asks for the 128-row kernel
-      if (h->cfg.n_envs <= sms * SmallShape<N, H, 16>::EPT_MAX) return 16;
-      if (h->cfg.n_envs <= sms * SmallShape<N, H, 32>::EPT_MAX) return 32;
+    if (sms > kFewRowsMaxSms) sms = kFewRowsMaxSms;
+    if ((cfg.flags & (MAVA_FLAG_WIDE_TILES | MAVA_FLAG_HIDDEN_IN_TMEM)) == 0) {  // either flag asks for the 128-row kernel
+      if (cfg.n_envs <= sms * SmallShape<N, H, 16>::EPT_MAX) return 16;
+      if (cfg.n_envs <= sms * SmallShape<N, H, 32>::EPT_MAX) return 32;
     }
   }
   return 0;
@@ -766,7 +770,7 @@ int few_rows_tile(const mava_rollout *h, int sms) {
 
 template <int N, int F, int ENV>
 cudaError_t launch_few_rows(mava_rollout *h, const RolloutArgs &args, int sms) {
-  return few_rows_tile<N, kTileRows>(h, sms) == 16 ? launch_tc_small<N, F, kTileRows, 16, ENV>(h, args, sms)
+  return few_rows_tile<N, kTileRows>(h->cfg, sms) == 16 ? launch_tc_small<N, F, kTileRows, 16, ENV>(h, args, sms)
                                                    : launch_tc_small<N, F, kTileRows, 32, ENV>(h, args, sms);
 }
 
@@ -778,7 +782,7 @@ cudaError_t launch_tc_variant(mava_rollout *h, const RolloutArgs &args) {
   if (err != cudaSuccess) return err;
   // Few rows per SM: the form with the rows as the N operand of the MMA.
   if constexpr (H == kTileRows)
-    if (few_rows_tile<N, H>(h, sms) != 0) return launch_few_rows<N, F, ENV>(h, args, sms);
+    if (few_rows_tile<N, H>(h->cfg, sms) != 0) return launch_few_rows<N, F, ENV>(h, args, sms);
   auto kern = args.eval ? rollout_tc_kernel<N, F, H, true, ENV> : rollout_tc_kernel<N, F, H, false, ENV>;
   const size_t smem = sizeof(TcSmem<N, F, H>);
   err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -814,7 +818,7 @@ cudaError_t launch_prep_variant(mava_rollout *h, const float *params_dev) {
 // A net of 64 units takes the few-rows form as one of 128 with zeros (the products with them add exactly nothing).  8x8-2p-2f,
 // 16 environments x 32 steps: 67.9 -> 63.1 us, evaluation block of 64 steps 114.8 -> 88.9; 1184 environments 131.6 -> 122.4 and 119.7 ->
 // 95.0; 2368 (32 rows a tile) 135.5 -> 132.3.
-bool padded_few_rows(const mava_rollout *h, int sms) { return h->variant == 0 && few_rows_tile<2, 128>(h, sms) != 0; }
+bool padded_few_rows(const mava_rollout *h, int sms) { return h->variant == 0 && few_rows_tile<2, 128>(h->cfg, sms) != 0; }
 cudaError_t sm_count(const mava_rollout *h, int *sms) { return cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, h->device); }
 
 }  // namespace
@@ -829,14 +833,15 @@ bool tc_rollout_is_wide(const mava_rollout *h) {
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess) return false;
   if ((h->cfg.flags & MAVA_FLAG_HIDDEN_IN_TMEM) != 0) return true;
-  if (h->variant <= 1) return few_rows_tile<2, 128>(h, sms) == 0;
-  if (h->variant == 2) return few_rows_tile<3, 128>(h, sms) == 0;
+  if (h->variant <= 1) return few_rows_tile<2, 128>(h->cfg, sms) == 0;
+  if (h->variant == 2) return few_rows_tile<3, 128>(h->cfg, sms) == 0;
   return true;
 }
 
 size_t tc_weight_bytes(const mava_config_t &cfg, int) {
   switch (find_variant(cfg)) {
-    case 0:  // (padded_few_rows)
+    case 0:  // the padded image only for a batch that the few-rows form may take (padded_few_rows)
+      return few_rows_tile<2, 128>(cfg, kFewRowsMaxSms) != 0 ? TcShape<2, 128>::IMAGE_BYTES : TcShape<2, 64>::IMAGE_BYTES;
     case 1: return TcShape<2, 128>::IMAGE_BYTES;
     case 2: return TcShape<3, 128>::IMAGE_BYTES;
     case 3: return TcShape<4, 256>::IMAGE_BYTES;

@@ -79,6 +79,22 @@ def test_create_without_a_gpu_fails_cleanly(lib):
     assert not out.value
 
 
+@pytest.mark.parametrize("idx,n_envs,flags,fits", [
+    (0, 8192, 0, True), (0, 8193, 0, True), (0, 16900, 0, True), (0, 16900, binding.MAVA_FLAG_WIDE_TILES, True), (0, 17100, 0, False),
+    ("wh0_tiny_8x8_2r2s_h64", 16900, 0, True), (1, 16250, 0, True), (1, 16400, 0, False), (4, 13900, 0, True), (4, 14200, 0, False)])
+def test_static_scratch_capacity(lib, idx, n_envs, flags, fits):
+    """What the allocation-free entry point's array holds (60 bytes per environment beside the weight image of the kernel that
+    serves the batch): the capacity check comes before anything touches CUDA."""
+    import torch
+
+    if torch.cuda.is_available():
+        pytest.skip("a GPU is present")
+    cfg = binding.make_config(wl.workload(idx), precision=binding.MAVA_PRECISION_BF16, n_envs=n_envs, max_T=4, flags=flags)
+    bufs = binding.mava_buffers_t(*([16] * 9))  # never dereferenced
+    rc = binding.mava_rollout_run_static(cfg, bufs, 16, 1, None)
+    assert rc == (binding.MAVA_ERR_CUDA if fits else binding.MAVA_ERR_CAPACITY)
+
+
 def test_product_path_never_imports_the_oracle():
     pkg = os.path.join(ROOT, "paper_2107_01460_b200")
     for dirpath, _, files in os.walk(pkg):

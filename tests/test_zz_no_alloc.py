@@ -19,7 +19,11 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("idx,precision,n_envs,T", [(1, binding.MAVA_PRECISION_BF16, 300, 40),
                                                     (4, binding.MAVA_PRECISION_BF16, 70, 20),
-                                                    (3, binding.MAVA_PRECISION_FP32, 50, 20)])
+                                                    (3, binding.MAVA_PRECISION_FP32, 50, 20),
+                                                    # H = 64: the few-rows form on the image padded to 128 units, and a
+                                                    # batch for which the scratch has room beside the image of 64 only
+                                                    (0, binding.MAVA_PRECISION_BF16, 40, 20),
+                                                    (0, binding.MAVA_PRECISION_BF16, 16900, 5)])
 def test_static_scratch_rollout_matches_handle_rollout(idx, precision, n_envs, T):
     import torch
 
