@@ -248,6 +248,13 @@ int mava_ppo_update(mava_rollout_t *h, float *params_dev, float *m_dev, float *v
       minibatches > h->cfg.n_envs)
     return MAVA_ERR_INVALID_ARG;
   const int E = h->cfg.n_envs;
+  if (h->last_T < 1 || !h->buf.adv || !h->buf.ret) return MAVA_ERR_INVALID_ARG;
+  if (!(hp->clip_eps > 0.0f)) return MAVA_ERR_INVALID_ARG;
+  if (h->cfg.net_kind == MAVA_NET_RECURRENT) return MAVA_ERR_UNSUPPORTED;
+  {  // scratch for pieces of both sizes before the first of them: growing it in between would wait for the GPU
+    DeviceGuard guard(h->device);
+    if (!guard.ok || reserve_update(h, E / minibatches, (E + minibatches - 1) / minibatches) != cudaSuccess) return MAVA_ERR_CUDA;
+  }
   int step = first_step;
   for (int e = 0; e < epochs; ++e)
     for (int k = 0; k < minibatches; ++k) {

@@ -369,9 +369,64 @@ static cudaError_t ensure_update_bytes(mava_rollout *h, size_t bytes) {
   return cudaMemsetAsync(h->d_upd, 0, 128, h->stream);  // the counters of the moments
 }
 static cudaError_t ensure_update_ring(mava_rollout *h, size_t bytes) { return ensure_bytes(&h->d_upd_ring, &h->upd_ring_bytes, bytes); }
-static cudaError_t ensure_update_scratch(mava_rollout *h, size_t n_params, int slices) {
-  return ensure_update_bytes(h, kHeadBytes + sizeof(double) * 3 * 8 * slices + sizeof(float) * ((n_params + 3) / 4 * 4) +
-                                    image_room() + sizeof(float) * n_params * slices);
+static size_t update_scratch_bytes(size_t n_params, int slices) {
+  return kHeadBytes + sizeof(double) * 3 * 8 * slices + sizeof(float) * ((n_params + 3) / 4 * 4) + image_room() + sizeof(float) * n_params * slices;
+}
+
+// How a gradient over the rows of `n_env` environments is cut up, and what it and the optimiser step behind it need.
+using Fp32Kernel = void (*)(UpdNet, UpdRows, UpdHyper, const double *, float *, size_t, double *, int *);
+struct UpdPlan {
+  int sms, slices;
+  Tc256Need net, critic;  // H = 256 on the tensor cores
+  Fp32Kernel kern;        // fp32 path
+  size_t scratch, ring;
+};
+static cudaError_t plan_update(const mava_rollout *h, int n_env, UpdPlan &plan) {
+  const mava_config_t &cfg = h->cfg;
+  const int N = cfg.n_agents, H = cfg.hidden;
+  const size_t P = param_layout(cfg, h->D, 1).total;
+  const long long S = static_cast<long long>(h->last_T) * n_env, R = S * N;  // environment-steps, rows
+  const bool central = cfg.net_kind == MAVA_NET_CENTRAL_CRITIC;
+  plan = UpdPlan{};
+  cudaError_t err = cudaDeviceGetAttribute(&plan.sms, cudaDevAttrMultiProcessorCount, h->device);
+  if (err != cudaSuccess) return err;
+  const auto at_most = [](long long tiles, long long ctas) { return static_cast<int>(tiles < ctas ? tiles : ctas); };
+  if (update_takes_tensor_cores(cfg, h->D)) {  // H <= 128: one CTA (= one gradient slice) per SM over tiles of 128 rows
+    plan.slices = at_most((R + 127) / 128, plan.sms);
+    plan.scratch = update_scratch_bytes(ppo_tc_slice_floats(), plan.slices);
+  } else if (update_takes_tensor_cores_256(cfg, h->D)) {
+    plan.net = ppo_tc256_need(R, plan.sms, 1);
+    if (central) plan.critic = ppo_tc256_need(S, plan.sms, N);
+    plan.scratch = kHeadBytes + plan.net.scratch + plan.critic.scratch;
+    plan.ring = plan.net.ring > plan.critic.ring ? plan.net.ring : plan.critic.ring;
+  } else {  // fp32: as many CTAs (= gradient slices) as are resident at once with the larger of the two nets' shared-memory needs
+    const size_t smem_max = upd_smem_bytes(central ? N * h->D : h->D, H);
+    plan.kern = H == 64 ? ppo_net_kernel<64> : (H == 128 ? ppo_net_kernel<128> : (H == 256 ? ppo_net_kernel<256> : nullptr));
+    if (!plan.kern) return cudaErrorNotSupported;
+    err = cudaFuncSetAttribute(plan.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_max));
+    if (err != cudaSuccess) return err;
+    int per_sm = 1;
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, plan.kern, H, smem_max);
+    if (err != cudaSuccess) return err;
+    plan.slices = at_most((R + kUpdRows - 1) / kUpdRows, static_cast<long long>(plan.sms) * (per_sm < 1 ? 1 : per_sm));
+    plan.scratch = update_scratch_bytes(P, plan.slices);
+  }
+  const size_t step = update_scratch_bytes(P, 1);  // launch_adam_step
+  if (plan.scratch < step) plan.scratch = step;
+  return cudaSuccess;
+}
+static cudaError_t ensure_update(mava_rollout *h, const UpdPlan &plan) {
+  const cudaError_t err = ensure_update_bytes(h, plan.scratch);
+  return err == cudaSuccess && plan.ring > 0 ? ensure_update_ring(h, plan.ring) : err;
+}
+cudaError_t reserve_update(mava_rollout *h, int n_small, int n_large) {
+  UpdPlan small, plan;
+  cudaError_t err = plan_update(h, n_small, small);
+  if (err == cudaSuccess) err = plan_update(h, n_large, plan);
+  if (err != cudaSuccess) return err;
+  if (plan.scratch < small.scratch) plan.scratch = small.scratch;
+  if (plan.ring < small.ring) plan.ring = small.ring;
+  return ensure_update(h, plan);
 }
 
 // `seq`: how many gradients and optimiser steps, and nothing else, this call's caller has launched directly before.  From the second
@@ -384,12 +439,13 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
   const int T = h->last_T, E = cfg.n_envs, N = cfg.n_agents, D = h->D, H = cfg.hidden;
   const ParamLayout L = param_layout(cfg, D, 1);
   const size_t P = L.total;
-  int sms = 0;
-  cudaError_t err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-  if (err != cudaSuccess) return err;
   const int n_env = env_ids_dev ? n_ids : E;  // environments in the minibatch
+  UpdPlan plan;
+  cudaError_t err = plan_update(h, n_env, plan);
+  if (err == cudaSuccess) err = ensure_update(h, plan);
+  if (err != cudaSuccess) return err;
+  const int slices = plan.slices;
   const long long R = static_cast<long long>(T) * n_env * N, S = static_cast<long long>(T) * n_env;
-  const long long tiles128 = (R + 127) / 128;
   const bool central = cfg.net_kind == MAVA_NET_CENTRAL_CRITIC;
   const UpdHyper hp{hyper.clip_eps, hyper.ent_coef, hyper.vf_coef};
   cudaStream_t st = h->stream;
@@ -399,10 +455,6 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
   if (!central) { rows.value_old = h->buf.values; rows.ret = h->buf.ret; rows.vstride = 1; }
 
   if (update_takes_tensor_cores(cfg, D)) {
-    // H <= 128: one CTA (= one gradient slice) per SM over tiles of 128 rows
-    const int slices = static_cast<int>(tiles128 < sms ? tiles128 : sms);
-    err = ensure_update_scratch(h, ppo_tc_slice_floats(), slices);
-    if (err != cudaSuccess) return err;
     const UpdScratch sc = carve(h, ppo_tc_slice_floats(), slices);
     const TermSums terms{sc.term_part, sc.term_part, 8 * slices, 8 * slices, R, R, hp, terms_dev};
     return launch_ppo_net_tc(h, params_dev, L, rows, hp, moments_of(h, seq & 1 ? kAdvMoments2 : kAdvMoments, h->buf.adv, R, rows, seq > 0), sc.image, sc.partial, sc.term_part, slices,
@@ -415,10 +467,7 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
 
   // H = 256 on the tensor cores: the actor / shared-torso net and, one input slab per agent, the centralised critic's
   if (update_takes_tensor_cores_256(cfg, D)) {
-    const Tc256Need need = ppo_tc256_need(R, sms, 1), cneed = central ? ppo_tc256_need(S, sms, N) : Tc256Need{0, 0};
-    err = ensure_update_bytes(h, kHeadBytes + need.scratch + cneed.scratch);
-    if (err == cudaSuccess) err = ensure_update_ring(h, need.ring > cneed.ring ? need.ring : cneed.ring);
-    if (err != cudaSuccess) return err;
+    const int sms = plan.sms;
     unsigned char *p = static_cast<unsigned char *>(h->d_upd) + kHeadBytes;
     const Moments adv = moments_of(h, kAdvMoments, h->buf.adv, R, rows);
     const double *stats = adv.out;
@@ -431,25 +480,11 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
     err = launch_ppo_net_tc256(h, params_dev, anet, rows, hp, adv, stats, p, h->d_upd_ring, sms, grad_dev, terms);
     if (err != cudaSuccess) return err;
     const Tc256Net cnet{L.C1, L.c1, L.C2, L.c2, 0, 0, L.Cv, L.cv, N, false, true};
-    return launch_ppo_net_tc256(h, params_dev, cnet, crows, hp, Moments{}, stats, p + need.scratch, h->d_upd_ring, sms, grad_dev, terms);
+    return launch_ppo_net_tc256(h, params_dev, cnet, crows, hp, Moments{}, stats, p + plan.net.scratch, h->d_upd_ring, sms, grad_dev, terms);
   }
 
-  const long long tiles = (R + kUpdRows - 1) / kUpdRows;
-  // fp32 kernel: as many CTAs (= gradient slices) as are resident at once with the larger of the two nets' shared-memory needs
   const int joint = N * D;
-  const size_t smem_max = upd_smem_bytes(central ? joint : D, H);
-  using KernelT = void (*)(UpdNet, UpdRows, UpdHyper, const double *, float *, size_t, double *, int *);
-  const KernelT kern = H == 64 ? ppo_net_kernel<64> : (H == 128 ? ppo_net_kernel<128> : (H == 256 ? ppo_net_kernel<256> : nullptr));
-  if (!kern) return cudaErrorNotSupported;
-  err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_max));
-  if (err != cudaSuccess) return err;
-  int per_sm = 1;
-  err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, H, smem_max);
-  if (err != cudaSuccess) return err;
-  if (per_sm < 1) per_sm = 1;
-  const int slices = static_cast<int>(tiles < static_cast<long long>(sms) * per_sm ? tiles : static_cast<long long>(sms) * per_sm);
-  err = ensure_update_scratch(h, P, slices);
-  if (err != cudaSuccess) return err;
+  const Fp32Kernel kern = plan.kern;
   const UpdScratch sc = carve(h, P, slices);
   // transposed copies of the hidden layers' weights, in the parameters' own order
   auto tr = [&](size_t off, int out, int in) {
@@ -502,7 +537,7 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
 cudaError_t launch_adam_step(mava_rollout *h, float *params_dev, const float *grad_dev, float *m_dev, float *v_dev, int32_t step,
                              const mava_ppo_hyper_t &hp, bool norm_known) {
   const size_t P = param_layout(h->cfg, h->D, 1).total;
-  cudaError_t err = ensure_update_scratch(h, P, 1);
+  cudaError_t err = ensure_update_bytes(h, update_scratch_bytes(P, 1));
   if (err != cudaSuccess) return err;
   const Moments norm = moments_of(h, kGradMoments, grad_dev, static_cast<long long>(P), UpdRows{});
   if (!norm_known) {

@@ -352,3 +352,31 @@ def test_a_batch_of_more_than_2_to_the_32_rows(idx, T):
     assert np.all(np.abs(got - want) <= 1e-6 * (1 + np.abs(want))), (got, want)  # (the terms are stored in binary32)
     assert bool(torch.isfinite(grad).all())
     ro.close()
+
+
+@pytest.mark.parametrize("idx,n_envs,T,minibatches,precision", [(1, 97, 32, 4, BF16), (1, 97, 32, 4, FP32), (4, 3, 1, 2, BF16), (3, 11, 9, 3, BF16)])
+def test_an_update_is_enqueued_without_waiting_for_the_gpu(idx, n_envs, T, minibatches, precision):
+    """The first update of a handle, with pieces of different sizes (the smaller first): the scratch is made once, so the
+    call returns while the GPU is still busy with what was enqueued before it."""
+    import torch
+
+    def update(ro, params):
+        p = params.clone()
+        perm = torch.arange(n_envs, dtype=torch.int32, device="cuda").view(1, -1)
+        ro.ppo_update(p, torch.zeros_like(p), torch.zeros_like(p), perm, minibatches, 1, hp)
+        return p
+
+    hp = binding.ppo_defaults()
+    _, first, params = _rolled_out(idx, n_envs, T, precision, flags=0)
+    want = update(first, params)  # (the kernels are loaded now)
+    _, ro, params = _rolled_out(idx, n_envs, T, precision, flags=0)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(400_000_000)  # clock cycles: a fifth of a second
+    slept = torch.cuda.Event()
+    slept.record()
+    got = update(ro, params)
+    assert not slept.query()
+    assert ro.status() == binding.MAVA_OK and first.status() == binding.MAVA_OK
+    assert torch.equal(got, want)
+    ro.close()
+    first.close()
