@@ -25,6 +25,13 @@ EnvParams env_params(const mava_rollout *h) {
                    static_cast<uint32_t>(h->cfg.seed), static_cast<uint32_t>(h->cfg.seed >> 32), h->cfg.env_kind};
 }
 
+// What every entry point answers when a CUDA call failed.  The runtime also keeps the error for whoever asks next (the next launch
+// check of the caller's own code, in the same process): the return code has told of it, so it is taken out.
+int cuda_failed() {
+  cudaGetLastError();
+  return MAVA_ERR_CUDA;
+}
+
 struct DeviceGuard {  // makes the handle's device current for the duration of a call
   int prev = -1;
   bool ok = true;
@@ -54,7 +61,7 @@ int run_common(mava_rollout *h, const float *params_dev, int32_t T, const int32_
   if (T < 1 || t_first < 0) return MAVA_ERR_INVALID_ARG;
   if (!ev && t_first + T > h->cfg.max_T) return MAVA_ERR_CAPACITY;  // an evaluation block stores no trajectory
   DeviceGuard guard(h->device);
-  if (!guard.ok) return MAVA_ERR_CUDA;
+  if (!guard.ok) return cuda_failed();
   RolloutArgs args{};
   args.env = env_params(h);
   args.buf = h->buf;
@@ -96,7 +103,7 @@ int run_common(mava_rollout *h, const float *params_dev, int32_t T, const int32_
     err = launch_prep_simt(h, params_dev);
     if (err == cudaSuccess) err = launch_rollout_simt(h, args);
   }
-  if (err != cudaSuccess) return MAVA_ERR_CUDA;
+  if (err != cudaSuccess) return cuda_failed();
   h->t_global += static_cast<uint32_t>(T);
   if (!ev) h->last_T = t_first + T;
   return MAVA_OK;
@@ -132,13 +139,13 @@ int mava_rollout_create(const mava_config_t *cfg, const mava_buffers_t *buffers,
   if (cfg->precision == MAVA_PRECISION_BF16 && !tc_supported(*cfg)) return MAVA_ERR_UNSUPPORTED;
 
   int device = 0;
-  if (cudaGetDevice(&device) != cudaSuccess) return MAVA_ERR_CUDA;
+  if (cudaGetDevice(&device) != cudaSuccess) return cuda_failed();
   int major = 0;  // (the whole property record takes 2.5 ms and more to fetch, an attribute a microsecond)
-  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess) return MAVA_ERR_CUDA;
+  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess) return cuda_failed();
   if (major != 10) return MAVA_ERR_UNSUPPORTED;  // kernels are built for sm_100a only
 
   mava_rollout *h = new (std::nothrow) mava_rollout();
-  if (!h) return MAVA_ERR_CUDA;
+  if (!h) return cuda_failed();
   h->cfg = *cfg;
   h->buf = b;
   h->stream = static_cast<cudaStream_t>(cuda_stream);
@@ -163,9 +170,8 @@ int mava_rollout_create(const mava_config_t *cfg, const mava_buffers_t *buffers,
   if (ok) ok = launch_env_init(h) == cudaSuccess;
   if (ok) ok = cudaStreamSynchronize(h->stream) == cudaSuccess;
   if (!ok) {
-    cudaGetLastError();
     mava_rollout_destroy(h);
-    return MAVA_ERR_CUDA;
+    return cuda_failed();
   }
   *out = h;
   return MAVA_OK;
@@ -192,8 +198,8 @@ int mava_gae(mava_rollout_t *h, float gamma, float lambda) {
   if (!(gamma >= 0.0f && gamma <= 1.0f && lambda >= 0.0f && lambda <= 1.0f)) return MAVA_ERR_INVALID_ARG;
   if (h->last_T > MAVA_GAE_MAX_T) return MAVA_ERR_CAPACITY;
   DeviceGuard guard(h->device);
-  if (!guard.ok) return MAVA_ERR_CUDA;
-  return launch_gae(h, gamma, lambda) == cudaSuccess ? MAVA_OK : MAVA_ERR_CUDA;
+  if (!guard.ok) return cuda_failed();
+  return launch_gae(h, gamma, lambda) == cudaSuccess ? MAVA_OK : cuda_failed();
 }
 
 int mava_debug_expire_next_wait(mava_rollout_t *h, int32_t which) {
@@ -214,8 +220,8 @@ int mava_ppo_grad(mava_rollout_t *h, const float *params_dev, const mava_ppo_hyp
   if (!(hp->clip_eps > 0.0f)) return MAVA_ERR_INVALID_ARG;
   if (h->cfg.net_kind == MAVA_NET_RECURRENT) return MAVA_ERR_UNSUPPORTED;  // no update block for the recurrent policy
   DeviceGuard guard(h->device);
-  if (!guard.ok) return MAVA_ERR_CUDA;
-  return launch_ppo_grad(h, params_dev, *hp, grad_dev, terms_dev, nullptr, 0) == cudaSuccess ? MAVA_OK : MAVA_ERR_CUDA;
+  if (!guard.ok) return cuda_failed();
+  return launch_ppo_grad(h, params_dev, *hp, grad_dev, terms_dev, nullptr, 0) == cudaSuccess ? MAVA_OK : cuda_failed();
 }
 
 static int grad_envs(mava_rollout_t *h, const float *params_dev, const mava_ppo_hyper_t *hp, const int32_t *env_ids_dev,
@@ -225,8 +231,8 @@ static int grad_envs(mava_rollout_t *h, const float *params_dev, const mava_ppo_
   if (!(hp->clip_eps > 0.0f)) return MAVA_ERR_INVALID_ARG;
   if (h->cfg.net_kind == MAVA_NET_RECURRENT) return MAVA_ERR_UNSUPPORTED;
   DeviceGuard guard(h->device);
-  if (!guard.ok) return MAVA_ERR_CUDA;
-  return launch_ppo_grad(h, params_dev, *hp, grad_dev, terms_dev, env_ids_dev, n_ids, seq) == cudaSuccess ? MAVA_OK : MAVA_ERR_CUDA;
+  if (!guard.ok) return cuda_failed();
+  return launch_ppo_grad(h, params_dev, *hp, grad_dev, terms_dev, env_ids_dev, n_ids, seq) == cudaSuccess ? MAVA_OK : cuda_failed();
 }
 
 int mava_ppo_grad_envs(mava_rollout_t *h, const float *params_dev, const mava_ppo_hyper_t *hp, const int32_t *env_ids_dev,
@@ -238,8 +244,8 @@ int mava_adam_step(mava_rollout_t *h, float *params_dev, const float *grad_dev, 
                    const mava_ppo_hyper_t *hp) {
   if (!h || !params_dev || !grad_dev || !m_dev || !v_dev || !hp || step < 1) return MAVA_ERR_INVALID_ARG;
   DeviceGuard guard(h->device);
-  if (!guard.ok) return MAVA_ERR_CUDA;
-  return launch_adam_step(h, params_dev, grad_dev, m_dev, v_dev, step, *hp, false) == cudaSuccess ? MAVA_OK : MAVA_ERR_CUDA;
+  if (!guard.ok) return cuda_failed();
+  return launch_adam_step(h, params_dev, grad_dev, m_dev, v_dev, step, *hp, false) == cudaSuccess ? MAVA_OK : cuda_failed();
 }
 
 int mava_ppo_update(mava_rollout_t *h, float *params_dev, float *m_dev, float *v_dev, float *grad_dev, const mava_ppo_hyper_t *hp,
@@ -253,7 +259,7 @@ int mava_ppo_update(mava_rollout_t *h, float *params_dev, float *m_dev, float *v
   if (h->cfg.net_kind == MAVA_NET_RECURRENT) return MAVA_ERR_UNSUPPORTED;
   {  // scratch for pieces of both sizes before the first of them: growing it in between would wait for the GPU
     DeviceGuard guard(h->device);
-    if (!guard.ok || reserve_update(h, E / minibatches, (E + minibatches - 1) / minibatches) != cudaSuccess) return MAVA_ERR_CUDA;
+    if (!guard.ok || reserve_update(h, E / minibatches, (E + minibatches - 1) / minibatches) != cudaSuccess) return cuda_failed();
   }
   int step = first_step;
   for (int e = 0; e < epochs; ++e)
@@ -263,7 +269,7 @@ int mava_ppo_update(mava_rollout_t *h, float *params_dev, float *m_dev, float *v
       int rc = grad_envs(h, params_dev, hp, perm_dev + static_cast<size_t>(e) * E + lo, hi - lo, grad_dev, terms, e * minibatches + k);
       if (rc != MAVA_OK) return rc;
       DeviceGuard guard(h->device);
-      if (!guard.ok || launch_adam_step(h, params_dev, grad_dev, m_dev, v_dev, step++, *hp, ppo_grad_leaves_norm(h)) != cudaSuccess) return MAVA_ERR_CUDA;
+      if (!guard.ok || launch_adam_step(h, params_dev, grad_dev, m_dev, v_dev, step++, *hp, ppo_grad_leaves_norm(h)) != cudaSuccess) return cuda_failed();
     }
   return MAVA_OK;
 }
@@ -271,24 +277,24 @@ int mava_ppo_update(mava_rollout_t *h, float *params_dev, float *m_dev, float *v
 int mava_rollout_reset(mava_rollout_t *h, uint64_t seed) {
   if (!h) return MAVA_ERR_INVALID_ARG;
   DeviceGuard guard(h->device);
-  if (!guard.ok) return MAVA_ERR_CUDA;
+  if (!guard.ok) return cuda_failed();
   h->cfg.seed = seed;
   h->t_global = 0;
   h->last_T = 0;
   if (h->d_hidden &&
       cudaMemsetAsync(h->d_hidden, 0, sizeof(float) * static_cast<size_t>(h->cfg.n_envs) * h->cfg.n_agents * h->cfg.hidden, h->stream) != cudaSuccess)
-    return MAVA_ERR_CUDA;
-  return launch_env_init(h) == cudaSuccess ? MAVA_OK : MAVA_ERR_CUDA;
+    return cuda_failed();
+  return launch_env_init(h) == cudaSuccess ? MAVA_OK : cuda_failed();
 }
 
 int mava_rollout_status(mava_rollout_t *h) {
   if (!h) return MAVA_ERR_INVALID_ARG;
   DeviceGuard guard(h->device);
-  if (!guard.ok) return MAVA_ERR_CUDA;
+  if (!guard.ok) return cuda_failed();
   int status = 0;
   if (cudaMemcpyAsync(&status, h->d_status, sizeof(int), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
       cudaStreamSynchronize(h->stream) != cudaSuccess)
-    return MAVA_ERR_CUDA;
+    return cuda_failed();
   if (status != 0) {
     cudaMemsetAsync(h->d_status, 0, sizeof(int), h->stream);
     return status == kStatusBadIndex ? MAVA_ERR_INVALID_ARG : MAVA_ERR_DEVICE_TIMEOUT;
@@ -299,13 +305,13 @@ int mava_rollout_status(mava_rollout_t *h) {
 int mava_rollout_get_state(mava_rollout_t *h, int32_t *records_host) {
   if (!h || !records_host) return MAVA_ERR_INVALID_ARG;
   DeviceGuard guard(h->device);
-  if (!guard.ok) return MAVA_ERR_CUDA;
+  if (!guard.ok) return cuda_failed();
   const int E = h->cfg.n_envs, N = h->cfg.n_agents, F = h->cfg.n_food;
   std::vector<EnvRec> recs(static_cast<size_t>(E));
   if (cudaMemcpyAsync(recs.data(), h->d_state, sizeof(EnvRec) * recs.size(), cudaMemcpyDeviceToHost, h->stream) !=
           cudaSuccess ||
       cudaStreamSynchronize(h->stream) != cudaSuccess)
-    return MAVA_ERR_CUDA;
+    return cuda_failed();
   const int len = 3 * (N + F) + 3;
   for (int e = 0; e < E; ++e) {
     int32_t *o = records_host + static_cast<size_t>(e) * len;
@@ -320,7 +326,7 @@ int mava_rollout_get_state(mava_rollout_t *h, int32_t *records_host) {
 int mava_rollout_set_state(mava_rollout_t *h, const int32_t *records_host) {
   if (!h || !records_host) return MAVA_ERR_INVALID_ARG;
   DeviceGuard guard(h->device);
-  if (!guard.ok) return MAVA_ERR_CUDA;
+  if (!guard.ok) return cuda_failed();
   const int E = h->cfg.n_envs, N = h->cfg.n_agents, F = h->cfg.n_food, G = h->cfg.grid;
   const int len = 3 * (N + F) + 3;
   std::vector<EnvRec> recs(static_cast<size_t>(E));
@@ -344,18 +350,18 @@ int mava_rollout_set_state(mava_rollout_t *h, const int32_t *records_host) {
   }
   if (cudaStreamSynchronize(h->stream) != cudaSuccess ||
       cudaMemcpy(h->d_state, recs.data(), sizeof(EnvRec) * recs.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-    return MAVA_ERR_CUDA;
+    return cuda_failed();
   return MAVA_OK;
 }
 
 int mava_rollout_get_hidden(mava_rollout_t *h, float *hidden_host) {
   if (!h || !hidden_host || !h->d_hidden) return MAVA_ERR_INVALID_ARG;
   DeviceGuard guard(h->device);
-  if (!guard.ok) return MAVA_ERR_CUDA;
+  if (!guard.ok) return cuda_failed();
   const size_t bytes = sizeof(float) * static_cast<size_t>(h->cfg.n_envs) * h->cfg.n_agents * h->cfg.hidden;
   if (cudaMemcpyAsync(hidden_host, h->d_hidden, bytes, cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
       cudaStreamSynchronize(h->stream) != cudaSuccess)
-    return MAVA_ERR_CUDA;
+    return cuda_failed();
   return MAVA_OK;
 }
 
@@ -365,16 +371,16 @@ int mava_rollout_collect_host(mava_rollout_t *h, const float *params_host, int32
   if (T < 1) return MAVA_ERR_INVALID_ARG;
   if (T > h->cfg.max_T || (h->buf.adv && h->buf.ret && T > MAVA_GAE_MAX_T)) return MAVA_ERR_CAPACITY;  // before anything is enqueued
   DeviceGuard guard(h->device);
-  if (!guard.ok) return MAVA_ERR_CUDA;
+  if (!guard.ok) return cuda_failed();
   const size_t np = param_layout(h->cfg, h->D, 1).total;
   if (cudaMemcpyAsync(h->d_params_stage, params_host, np * sizeof(float), cudaMemcpyHostToDevice, h->stream) !=
       cudaSuccess)
-    return MAVA_ERR_CUDA;
+    return cuda_failed();
   if (!h->copy_ready) {
     bool made = cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking) == cudaSuccess;
     for (int i = 0; made && i <= kCollectChunks; ++i)
       made = cudaEventCreateWithFlags(&h->chunk_done[i], cudaEventDisableTiming) == cudaSuccess;
-    if (!made) return MAVA_ERR_CUDA;
+    if (!made) return cuda_failed();
     h->copy_ready = true;
   }
   // The copies are bound by the host link and take several times as long as the kernels, so the
@@ -396,7 +402,7 @@ int mava_rollout_collect_host(mava_rollout_t *h, const float *params_host, int32
     if (rc != MAVA_OK) return rc;
     if (cudaEventRecord(h->chunk_done[c], h->stream) != cudaSuccess ||
         cudaStreamWaitEvent(h->copy_stream, h->chunk_done[c], 0) != cudaSuccess)
-      return MAVA_ERR_CUDA;
+      return cuda_failed();
     const size_t r0 = M * t0, rn = M * (t1 - t0);
     back(out->obs, h->buf.obs, r0 * h->D * sizeof(float), rn * h->D * sizeof(float));
     back(out->actions, h->buf.actions, r0 * sizeof(int32_t), rn * sizeof(int32_t));
@@ -412,12 +418,12 @@ int mava_rollout_collect_host(mava_rollout_t *h, const float *params_host, int32
     if (rc != MAVA_OK) return rc;
     if (cudaEventRecord(h->chunk_done[kCollectChunks], h->stream) != cudaSuccess ||
         cudaStreamWaitEvent(h->copy_stream, h->chunk_done[kCollectChunks], 0) != cudaSuccess)
-      return MAVA_ERR_CUDA;
+      return cuda_failed();
     back(out->adv, h->buf.adv, 0, M * T * sizeof(float));
     back(out->ret, h->buf.ret, 0, M * T * sizeof(float));
   }
   if (!ok || cudaStreamSynchronize(h->copy_stream) != cudaSuccess || cudaStreamSynchronize(h->stream) != cudaSuccess)
-    return MAVA_ERR_CUDA;
+    return cuda_failed();
   return MAVA_OK;
 }
 
@@ -440,10 +446,7 @@ unsigned char *static_scratch(int device) {
   std::lock_guard<std::mutex> lock(g_scratch_mutex);
   if (!g_scratch_addr[device]) {
     void *ptr = nullptr;
-    if (cudaGetSymbolAddress(&ptr, g_static_scratch) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
+    if (cudaGetSymbolAddress(&ptr, g_static_scratch) != cudaSuccess) return nullptr;
     g_scratch_addr[device] = static_cast<unsigned char *>(ptr);
   }
   return g_scratch_addr[device];
@@ -476,12 +479,12 @@ int mava_rollout_run_static(const mava_config_t *cfg, const mava_buffers_t *buff
   if (256 + state_bytes + weight_bytes > MAVA_STATIC_SCRATCH_BYTES) return MAVA_ERR_CAPACITY;
 
   int device = 0;
-  if (cudaGetDevice(&device) != cudaSuccess) return MAVA_ERR_CUDA;
+  if (cudaGetDevice(&device) != cudaSuccess) return cuda_failed();
   int major = 0;
-  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess) return MAVA_ERR_CUDA;
+  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess) return cuda_failed();
   if (major != 10) return MAVA_ERR_UNSUPPORTED;
   unsigned char *scratch = static_scratch(device);
-  if (!scratch) return MAVA_ERR_CUDA;
+  if (!scratch) return cuda_failed();
 
   mava_rollout h{};  // a handle on the stack whose device state lives in the static array
   h.cfg = *cfg;
@@ -497,14 +500,14 @@ int mava_rollout_run_static(const mava_config_t *cfg, const mava_buffers_t *buff
 
   // the array keeps what the previous call left: the status word must start at zero; the
   // states and the weights are fully rewritten by the kernels below
-  if (cudaMemsetAsync(h.d_status, 0, sizeof(int), h.stream) != cudaSuccess) return MAVA_ERR_CUDA;
-  if (launch_env_init(&h) != cudaSuccess) return MAVA_ERR_CUDA;
+  if (cudaMemsetAsync(h.d_status, 0, sizeof(int), h.stream) != cudaSuccess) return cuda_failed();
+  if (launch_env_init(&h) != cudaSuccess) return cuda_failed();
   const int rc = run_common(&h, params_dev, T, nullptr);
   if (rc != MAVA_OK) return rc;
   int status = 0;
   if (cudaMemcpyAsync(&status, h.d_status, sizeof(int), cudaMemcpyDeviceToHost, h.stream) != cudaSuccess ||
       cudaStreamSynchronize(h.stream) != cudaSuccess)
-    return MAVA_ERR_CUDA;
+    return cuda_failed();
   return status != 0 ? MAVA_ERR_DEVICE_TIMEOUT : MAVA_OK;
 }
 

@@ -95,6 +95,12 @@ def test_static_scratch_capacity(lib, idx, n_envs, flags, fits):
     assert rc == (binding.MAVA_ERR_CUDA if fits else binding.MAVA_ERR_CAPACITY)
 
 
+def test_every_entry_point_answers_a_failed_cuda_call_through_one_function():
+    """The one that also takes the error out of the runtime's own record (tests/test_gpu_failure.py has the behaviour)."""
+    source = open(os.path.join(ROOT, "paper_2107_01460_b200", "csrc", "api.cu")).read()
+    assert source.count("return MAVA_ERR_CUDA;") == 1 and not re.search(r"[?:]\s*MAVA_ERR_CUDA\s*;", source)
+
+
 def test_product_path_never_imports_the_oracle():
     pkg = os.path.join(ROOT, "paper_2107_01460_b200")
     for dirpath, _, files in os.walk(pkg):

@@ -68,3 +68,40 @@ def test_gae_longer_than_its_limit_is_a_capacity_error():
         ro.gae(wl.GAMMA, wl.LAMBDA)
     assert e.value.code == binding.MAVA_ERR_CAPACITY
     assert ro.status() == binding.MAVA_OK
+
+
+@pytest.mark.parametrize("idx", [1, 4])
+def test_a_failed_launch_leaves_no_error_behind(idx):
+    """A launch that the runtime refuses on the host (into a stream capture that is no longer valid): the return code tells of it,
+    and the runtime's own record, which the caller's process would take for a failure of whatever it launches next, is clear."""
+    import ctypes as C
+
+    import torch
+
+    w = wl.workload(idx)
+    T, n_envs = 8, 32
+    p_dev = torch.from_numpy(wl.make_params(w)).cuda()
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        ro = binding.Rollout(binding.make_config(w, precision=BF16, max_T=T, n_envs=n_envs))
+        ro.run(p_dev, T)
+        ro.gae(wl.GAMMA, wl.LAMBDA)
+    ro.ppo_grad(p_dev)
+    torch.cuda.synchronize()
+    want = ro.obs.clone(), ro.logp.clone()
+    rt = C.CDLL("libcudart.so.12")  # the instance that the library and torch share
+    s, graph = C.c_void_p(stream.cuda_stream), C.c_void_p()
+    assert rt.cudaStreamBeginCapture(s, 2) == 0  # relaxed: only this stream is concerned
+    assert rt.cudaStreamSynchronize(s) != 0      # not allowed while capturing: the capture is invalid from here on
+    rt.cudaGetLastError()
+    codes = [binding.lib().mava_rollout_run(ro.handle, p_dev.data_ptr(), T), binding.lib().mava_gae(ro.handle, 0.99, 0.95)]
+    record = rt.cudaPeekAtLastError()
+    assert rt.cudaStreamEndCapture(s, C.byref(graph)) != 0
+    rt.cudaGetLastError()
+    assert codes == [binding.MAVA_ERR_CUDA] * 2 and record == 0
+    ro.reset(w["seed"])
+    ro.run(p_dev, T)
+    ro.gae(wl.GAMMA, wl.LAMBDA)
+    assert ro.status() == binding.MAVA_OK
+    assert torch.equal(ro.obs, want[0]) and torch.equal(ro.logp, want[1])
+    ro.close()
