@@ -102,7 +102,7 @@ __device__ __forceinline__ void add2(uint32_t &lo, uint32_t &hi, float blo, floa
 }
 __device__ __forceinline__ float4 lds_float4(uint32_t addr) {
   float4 v;
-  asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
   return v;
 }
 

@@ -55,3 +55,12 @@ def test_a_dependent_kernel_declares_nothing_constant_that_its_predecessor_may_w
 def test_no_load_takes_the_non_coherent_path_by_hand():
     for name, text in _sources():
         assert "ld.global.nc" not in text, name
+
+
+def test_inline_assembly_that_reads_memory_is_kept_in_order():
+    """Without `volatile` an asm statement is a pure function of its operands: a load may then move over the wait for what it
+    reads, or be done once for several uses."""
+    for name, text in _sources():
+        for m in re.finditer(r"\basm\s*\(", text):  # (asm volatile does not match)
+            statement = text[m.start():_closing(text, m.end() - 1, "()")]
+            assert not re.search(r"\b(ld|tcgen05\.ld|ldmatrix|atom|red|st|mbarrier)\b", statement), (name, statement[:120])
