@@ -380,3 +380,76 @@ def test_an_update_is_enqueued_without_waiting_for_the_gpu(idx, n_envs, T, minib
     assert torch.equal(got, want)
     ro.close()
     first.close()
+
+
+@pytest.mark.parametrize("idx,n_envs,T,epochs,minibatches", [(1, 1777, 64, 4, 4), (2, 3001, 61, 2, 3), (0, 1031, 40, 3, 5), (4, 601, 16, 1, 3)])
+def test_update_loop_with_several_ragged_tiles_per_sm(idx, n_envs, T, epochs, minibatches):
+    """The loop whose minibatches overlap (moments and first rows of one while the one before it finishes) against the calls one
+    by one, where it has work for it: two to four tiles per SM (148), a ragged last one, pieces of different sizes, up to
+    sixteen minibatches; idx 4: the kernel whose SMs take roles, which is chained without the overlap.  Same bytes, every time."""
+    import torch
+
+    w, ro, params = _rolled_out(idx, n_envs, T, BF16, flags=0)
+    g = torch.Generator(device="cuda").manual_seed(11)
+    perm = torch.stack([torch.randperm(n_envs, generator=g, device="cuda") for _ in range(epochs)]).to(torch.int32).contiguous()
+    hp = binding.ppo_defaults()
+    p2, m2, v2 = params.clone(), torch.zeros_like(params), torch.zeros_like(params)
+    terms2, step = [], 0
+    for e in range(epochs):
+        for k in range(minibatches):
+            ids = perm[e, n_envs * k // minibatches: n_envs * (k + 1) // minibatches].contiguous()
+            t, grad = ro.ppo_grad(p2, hp, env_ids=ids)
+            torch.cuda.synchronize()  # nothing overlaps here
+            step += 1
+            ro.adam_step(p2, grad, m2, v2, step, hp)
+            terms2.append(t.clone())
+    terms2 = torch.stack(terms2)
+    for _ in range(20):
+        p1, m1, v1 = params.clone(), torch.zeros_like(params), torch.zeros_like(params)
+        terms1 = ro.ppo_update(p1, m1, v1, perm, minibatches, 1, hp)
+        assert torch.equal(terms1, terms2) and torch.equal(p1, p2) and torch.equal(m1, m2) and torch.equal(v1, v2)
+    assert ro.status() == binding.MAVA_OK
+    assert not torch.equal(p2, params)
+    ro.close()
+
+
+def test_centralised_critics_gradient_where_its_ring_turns_over():
+    """1024 tiles of the critic's net: its ring of at most 3 x 148 slots is used more than twice (each use is read by the W2 SM and
+    by a W1 SM per pair of input slabs) and every weight SM adds its accumulators to memory after 48 tiles, which smaller
+    batches do not reach.  The value loss is a plain mean over environment-steps, so the critic's gradient of the whole
+    batch is the mean of the gradients of equal pieces of environments, each small enough (256 tiles) for the path that
+    the oracle comparisons cover.  Same products: what differs is the order of the fp32 sums, chains of 48 tiles in an accumulator
+    (1e-5 of the sum) and their sum."""
+    import torch
+
+    n_envs, T, pieces = 2048, 64, 4
+    w, ro, params = _rolled_out(3, n_envs, T, BF16, flags=0)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    new = params + 0.6 * torch.randn(params.shape, generator=g, device="cuda") * params.std()
+    terms, grad = ro.ppo_grad(new)
+    perm = torch.randperm(n_envs, generator=g, device="cuda").to(torch.int32)
+    parts = [ro.ppo_grad(new, env_ids=perm[n_envs * k // pieces: n_envs * (k + 1) // pieces].contiguous()) for k in range(pieces)]
+    assert ro.status() == binding.MAVA_OK
+    mean = torch.stack([p[1].double() for p in parts]).mean(0).cpu().numpy()
+    value = torch.stack([p[0][3].double() for p in parts]).mean().item()
+    gg = grad.double().cpu().numpy()
+    assert abs(terms[3].item() - value) <= 1e-6 * (1 + abs(value))
+    shapes = ppo.layer_shapes(wl.obs_dim(w), w["hidden"], w["n_agents"], w["net_kind"])
+    off, seen = 0, 0
+    for name, (o, i) in shapes:
+        for lo, hi in ((off, off + o * i), (off + o * i, off + o * i + o)):
+            if lo >= _critic_offset(w):
+                seg = np.max(np.abs(mean[lo:hi]))
+                assert seg > 0 and np.max(np.abs(gg[lo:hi] - mean[lo:hi])) <= 1e-4 * seg, (name, lo)
+                seen += hi - lo
+        off += o * i + o
+    assert seen == wl.params_count(w) - _critic_offset(w)
+    terms2, grad2 = ro.ppo_grad(new)
+    assert torch.equal(grad, grad2) and torch.equal(terms, terms2)
+    ro.close()
+
+
+def _critic_offset(w):
+    """Where the centralised critic's parameters start (behind the actor's W1 b1 W2 b2 Wa ba)."""
+    D, H = wl.obs_dim(w), w["hidden"]
+    return H * D + H + H * H + H + 6 * H + 6
