@@ -428,7 +428,10 @@ __device__ __forceinline__ bool window_cell(uint32_t e, uint32_t bias, int &cell
 __device__ __forceinline__ uint32_t window_bias(uint32_t me) {
   return 0x4242u - (me & 0xFFFFu);  // 64 + view radius - coordinate, per byte
 }
-// fp32 value (as bits) of entity k's plane entry; zero: nothing there.
+// fp32 value (as bits) of entity k's plane entry, and whether it has one: a foraging entity of level 0 (collected food) shows nothing,
+// its cell may hold another entity of the same plane; in the warehouse the last shelf of a cell shows, whatever its status.
+template <int ENV>
+__device__ __forceinline__ bool plane_shows(bool in_window, uint32_t value) { return in_window && (ENV != 0 || value != 0u); }
 template <int N, int ENV>
 __device__ __forceinline__ uint32_t plane_value(uint32_t e, int k) {
   const uint32_t l = e >> 16;
@@ -491,8 +494,7 @@ __device__ __forceinline__ void write_row_bf16(const EnvRegs<N, F> &s, const Env
     const bool in = window_cell(s.ent[k], bias, cell);
     const int j = cell + (k < N ? 0 : kPlane);
     const uint32_t v = plane_value<N, ENV>(s.ent[k], k);
-    // (an entity of level 0 -- collected food -- shows nothing: its cell may hold another entity of the same plane)
-    sts_u16_if(row + static_cast<uint32_t>(j >> 3) * kChunk + static_cast<uint32_t>(j & 7) * 2u, v >> 16, in && v != 0u);
+    sts_u16_if(row + static_cast<uint32_t>(j >> 3) * kChunk + static_cast<uint32_t>(j & 7) * 2u, v >> 16, plane_shows<ENV>(in, v));
   }
 }
 // The fp32 row over a zero background, in the three parts that different warps may write.
@@ -513,7 +515,7 @@ __device__ __forceinline__ void write_entities_f32(const EnvRegs<N, F> &s, uint3
     int cell;
     const bool in = window_cell(s.ent[k], bias, cell);
     const uint32_t v = plane_value<N, ENV>(s.ent[k], k);
-    sts_u32_if(row + 4u * static_cast<uint32_t>(cell + (k < N ? 0 : kPlane)), v, in && v != 0u);
+    sts_u32_if(row + 4u * static_cast<uint32_t>(cell + (k < N ? 0 : kPlane)), v, plane_shows<ENV>(in, v));
   }
 }
 template <int ENV>

@@ -116,3 +116,34 @@ def test_warehouse_shards_reproduce_the_whole_batch():
     for name in ("obs", "actions", "rewards", "dones", "logp", "values"):
         full = getattr(whole, name)
         assert torch.equal(full[:, :cut], getattr(lo, name)) and torch.equal(full[:, cut:], getattr(hi, name)), name
+
+
+@pytest.mark.parametrize("name,flags", [(WH0, 0), (WH1, 0), (WH0, binding.MAVA_FLAG_WIDE_TILES), (WH1, binding.MAVA_FLAG_WIDE_TILES)])
+def test_shelves_in_one_cell_are_seen_as_on_the_fp32_path(name, flags):
+    """States that only set_state can make: several shelves in a cell, some of status 0.  The last shelf of the cell shows."""
+    import torch
+
+    w = wl.workload(name)
+    N, F, E = w["n_agents"], w["n_food"], 64
+    rng = np.random.default_rng(3)
+    states = np.zeros((E, 3 * (N + F) + 3), dtype=np.int32)
+    for e in range(E):
+        cells = rng.integers(0, w["grid"], size=(N + F, 2))
+        cells[N:] = cells[N + rng.integers(0, F, size=F)]  # shelves share cells
+        cells[0] = np.clip(cells[N] + rng.integers(-1, 2, size=2), 0, w["grid"] - 1)  # in sight of robot 0
+        for k in range(N + F):
+            states[e, 3 * k:3 * k + 2] = cells[k]
+        states[e, 3 * N + 2:3 * (N + F):3] = rng.integers(0, 3, size=F)
+    params = torch.from_numpy(wl.make_params(w)).cuda()
+    acts = torch.zeros((1, E, N), dtype=torch.int32, device="cuda")  # nobody moves
+    obs = []
+    for precision, f in ((FP32, 0), (BF16, flags)):
+        ro = binding.Rollout(binding.make_config(w, precision=precision, max_T=1, n_envs=E, flags=f))
+        ro.set_state(states)
+        ro.run_forced(params, 1, acts)
+        assert ro.status() == binding.MAVA_OK
+        obs.append(ro.obs.clone())
+        ro.close()
+    assert torch.equal(obs[0], obs[1])
+    plane = obs[0][0, :, 0, 25:50].cpu().numpy()
+    assert (states[:, 3 * N + 2:3 * (N + F):3] == 0).any() and (plane != 0).any()
