@@ -245,37 +245,6 @@ __device__ void wh_reset_env(EnvRegs<N, F> &s, const EnvParams &p, uint32_t env,
   s.step = 0; s.episode = static_cast<int32_t>(episode); s.total = 0;
 }
 
-// Non-zero observation entries of robot `ag`.
-template <int N, int F, class Sink>
-__device__ __forceinline__ void wh_observe_env(const EnvRegs<N, F> &s, const EnvParams &p, int ag, Sink sink) {
-  const uint32_t me = own_entity(s, ag);
-  const int r0 = me & 0xFF, c0 = (me >> 8) & 0xFF, G = p.grid;
-#pragma unroll
-  for (int dy = 0; dy < kWindow; ++dy) {
-    const int rr = r0 + dy - kViewRadius;
-#pragma unroll
-    for (int dx = 0; dx < kWindow; ++dx) {
-      const int cc = c0 + dx - kViewRadius;
-      const bool outside = rr < 0 || rr >= G || cc < 0 || cc >= G;
-      if (outside) sink(2 * kPlane + dy * kWindow + dx, 1.0f);
-      else if (rr == 0) sink(2 * kPlane + dy * kWindow + dx, 0.5f);
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < N + F; ++k) {
-    const uint32_t e = s.ent[k];
-    const int dy = static_cast<int>(e & 0xFF) - r0 + kViewRadius, dx = static_cast<int>((e >> 8) & 0xFF) - c0 + kViewRadius;
-    const int lvl = static_cast<int>(e >> 16);
-    if (dy >= 0 && dy < kWindow && dx >= 0 && dx < kWindow) {
-      if (k < N) sink(dy * kWindow + dx, lvl > 0 ? 2.0f : 1.0f);
-      else sink(kPlane + dy * kWindow + dx, static_cast<float>(lvl));
-    }
-  }
-  sink(3 * kPlane, (me >> 16) != 0 ? 2.0f : 1.0f);
-  sink(3 * kPlane + 1, __fdiv_rn(static_cast<float>(s.step), static_cast<float>(p.cap)));
-  sink(kObsFixed + ag, 1.0f);
-}
-
 // One transition of the environment whose N robot threads occupy lanes [base, base + N): every lane of the warp calls it.
 // wh_transition's rules; each lane decides for its own robot, the decisions travel by shuffles and every lane applies them to
 // its own copy of the state in robot order, so the copies stay identical (with the whole transition on every lane a step's

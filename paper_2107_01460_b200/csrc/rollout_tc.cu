@@ -212,45 +212,10 @@ __device__ __forceinline__ void issue_layer(uint32_t d_tmem, uint32_t a_addr, ui
   __syncwarp();
 }
 
-// Observation rows [first, first + n) of a tile (compact numbering; tile row = tile_row0 + i),
-// expanded from the bf16 A tile to fp32 and written to `dst` (row stride D); consecutive lanes
-// write consecutive floats.  The exact step/cap replaces the rounded bf16 one.  Four rows are in
-// flight at a time.
-template <int D, int K1>
-__device__ __forceinline__ void expand_rows(uint32_t a_tile, uint32_t step_frac, float *dst, int first, int n,
-                                            int tile_row0, int lane) {
-  constexpr int Q = (D + 31) / 32;
-  uint32_t off[Q];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) off[q] = a_offset<K1>(0, lane + 32 * q);
-  for (int l0 = 0; l0 < n; l0 += 4) {
-    uint32_t raw[4][Q];
-    float sf[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int tr = tile_row0 + min(l0 + r, n - 1);
-      const uint32_t arow = a_tile + a_offset<K1>(tr, 0);
-#pragma unroll
-      for (int q = 0; q < Q; ++q) raw[r][q] = (lane + 32 * q < D) ? lds_u16(arow + off[q]) : 0u;
-      sf[r] = lds_f32(step_frac + 4u * static_cast<uint32_t>(tr));
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      if (l0 + r < n) {
-        float *orow = dst + static_cast<size_t>(first + l0 + r) * D;
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-          const int j = lane + 32 * q;
-          if (j < D) orow[j] = (j == 3 * kPlane + 1) ? sf[r] : __uint_as_float(raw[r][q] << 16);
-        }
-      }
-    }
-  }
-}
-
-// The same job for row counts that are multiples of four: four rows are one 16-byte aligned run
-// of 4*D floats, written as float4 by consecutive lanes.  Which (row of the four, column) a lane's
-// elements are does not depend on the quad, so their tile offsets are computed once.
+// Observation rows [first, first + n) of a tile (compact numbering; tile row = tile_row0 + i), expanded from the bf16 A tile to fp32
+// and written to `dst` (row stride D); the exact step/cap replaces the rounded bf16 one.  For row counts that are multiples of
+// four: four rows are one 16-byte aligned run of 4*D floats, written as float4 by consecutive lanes.  Which (row of the four,
+// column) a lane's elements are does not depend on the quad, so their tile offsets are computed once.
 template <int D, int K1>
 struct QuadPlan {
   static constexpr int V = (D + 31) / 32;  // float4 per lane per quad (D float4 in all)
@@ -471,8 +436,9 @@ rollout_tc_kernel(RolloutArgs a, const unsigned char *image, int ept, int n_tile
       // until the step's observations are in the tile, expand the rows the group asks for to fp32 in the obs array
       // (warp w the rows of the group's warp w), and let go of the tile.  The loop bounds are those of the groups,
       // which in ping-pong mode walk through every step's barriers whatever happens to them.
+      static_assert(N % 4 == 0, "rows go out four at a time");
       QuadPlan<D, K1> quad_plan;
-      if (N % 4 == 0) plan_quads<D, K1>(quad_plan, lane);
+      plan_quads<D, K1>(quad_plan, lane);
       pair_arrive(kBarTile + 0, TP);  // group 0 goes first
       const volatile int *copy_rows = sm.copy_rows;
       for (int it = 0;; ++it) {
@@ -486,10 +452,7 @@ rollout_tc_kernel(RolloutArgs a, const unsigned char *image, int ept, int n_tile
               const int e0 = (tile0 + hg) * ept;
               float *dst = (t == a.T) ? a.obs_last + static_cast<size_t>(e0) * N * D
                                       : a.buf.obs + (static_cast<size_t>(t) * M + static_cast<size_t>(e0) * N) * D;
-              if constexpr (N % 4 == 0)
-                expand_quads<D, K1>(quad_plan, a_addr, frac_addr, dst, wg * S::RPW, min(S::RPW, n_rows - wg * S::RPW), wg * 32, lane);
-              else
-                expand_rows<D, K1>(a_addr, frac_addr, dst, wg * S::RPW, min(S::RPW, n_rows - wg * S::RPW), wg * 32, lane);
+              expand_quads<D, K1>(quad_plan, a_addr, frac_addr, dst, wg * S::RPW, min(S::RPW, n_rows - wg * S::RPW), wg * 32, lane);
             }
             pair_arrive(kBarTile + (1 - hg), TP);
           }
