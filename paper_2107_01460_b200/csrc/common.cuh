@@ -159,7 +159,7 @@ cudaError_t launch_rollout_rec_simt(mava_rollout *h, const float *params_dev, co
 cudaError_t launch_rollout_rec_tc(mava_rollout *h, const float *params_dev, const RolloutArgs &args);
 size_t rec_tc_weight_bytes(const mava_config_t &cfg);
 
-// Update block (fp32).
+// Update block.
 cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava_ppo_hyper_t &hp, float *grad_dev, float *terms_dev,
                             const int32_t *env_ids_dev, int32_t n_ids, int seq = 0);
 cudaError_t reserve_update(mava_rollout *h, int n_small, int n_large);  // scratch of gradients over n_small or n_large environments of the last run and

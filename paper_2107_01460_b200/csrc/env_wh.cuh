@@ -23,8 +23,6 @@ namespace mava {
 
 constexpr uint32_t kDomainRequest = 0x52455153u;  // key tweak of the replacement-request stream
 
-__device__ __forceinline__ int wh_requests(int F) { return F / 2 > 0 ? F / 2 : 1; }
-
 // ---- placement -------------------------------------------------------------------------------------------------------
 // F shelf cells (r-th free cell of rows 1..G-1), N robot cells (r-th cell of the whole grid free of shelves and earlier
 // robots), then the requests (r-th still idle shelf); draw i = word i % 4 of block (i / 4, env, episode, 0).

@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(256) grad_moments_kernel(Moments m, int len, M
 }
 
 // Tensor-core path for H = 256 (update_tc256.cu): a net with hidden width 256 whose first layer takes `slabs` observation
-// slabs of width 64 < D <= 94 side by side (1: the actor / shared-torso net; n_agents: the centralised critic).  Offsets are
+// slabs of width 64 < D <= 95 side by side (1: the actor / shared-torso net; n_agents: the centralised critic).  Offsets are
 // those of the net's layers in the flat parameter array.  Writes the net's gradient and, after the net with the value head,
 // the loss terms.
 struct Tc256Net {

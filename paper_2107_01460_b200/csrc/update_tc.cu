@@ -12,8 +12,9 @@
 //              -> d h2 -> d z2 -> d h1 -> d z1, and on the side d Wh^T += h2^T . dhead, d W2 += d z2^T . h1,
 //              d W1 += d z1^T . x, d b2 += d z2^T . 1, d b1 += d z1^T . 1 (the ones are column 7 of the dhead tile).
 // The weight-gradient accumulators stay in tensor memory for all tiles of the CTA and are written once, into the CTA's
-// own slice of the partial-gradient array; a last kernel adds the slices in slice order (update.cu), so the gradient
-// is the same bytes on every call.  Rounding points are those of the bf16-operand mode of the float64 oracle.
+// own slice of the partial-gradient array; a last kernel adds the slices in a fixed order (reduce_slices_kernel: four quarters of
+// them, each in slice order), so the gradient is the same bytes on every call.  Rounding points are those of the bf16-operand
+// mode of the float64 oracle.
 // A hidden width below 128 is padded with zero units (their activations, gates and gradients are exactly zero).
 // MMAs are issued by one elected lane; tcgen05.commit tracks all MMAs issued before it, so a tile buffer may be rewritten as
 // soon as a later commit has been waited for.  Every mbarrier wait is bounded.

@@ -2,7 +2,8 @@
 // centralised critic of the two largest shapes.  The weight gradient of the second layer alone (256 x 256 fp32) fills all
 // 512 columns of an SM's tensor memory, and the weights (184 KB in bf16) leave no room for bf16 activation tiles in shared
 // memory, so no SM can do a tile's row pass and its weight gradients.  One cooperative kernel therefore gives every SM one
-// of three roles for the whole batch, and tiles travel between them through a ring of slots that stays in L2:
+// of three roles for the whole batch, and tiles travel between them through a ring of slots (three per row SM; about what L2
+// holds beside the observations: most of what passes through is read from L2, and most of it is written back as well):
 //   row SMs      per 128-row tile: forward and backward through the layers with the activations in tensor memory as the A
 //                operand of the next product, the loss and its per-row derivatives in fp32; every bf16 matrix that a weight
 //                gradient needs (x, h1, h2, d z2, d z1, the heads' derivatives) is stored to the tile's slot in the canonical
@@ -18,9 +19,11 @@
 // the order of every sum is fixed too.  The launch is cooperative because the roles wait for one another.
 // Rounding points are those of the bf16-operand mode of the float64 oracle.  Every wait is bounded.
 //
-// What bounds it: a row SM stores 284 KB per tile and an SM's store path into L2 takes about 30 bytes per cycle (measured:
-// 7.9 TB/s over 148 SMs), which is longer than the tile's products (5.2 k cycles); a weight SM reads the same bytes at
-// 70 bytes per cycle and more.
+// What bounds it (8 agents on 20x20): row SMs by themselves take 16.1 k cycles a tile, 12.4 k without the stores to the ring:
+// eight epilogue warps for two groups' seven passes over half an accumulator each, the products (5.2 k) beside them.  The
+// stores, 287 KB a tile at the 30 bytes per cycle that an SM's path into L2 takes, are 9.8 k.  A W2 SM by itself takes 3.1 k
+// cycles a tile for its shared-memory reads.  Side by side they compete for L2: of the 4.75 GB that 4096 environments x 64
+// steps send through the ring 3.8 GB are written back to HBM.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -948,8 +951,13 @@ __global__ void reduce256_kernel(float *__restrict__ grad, Net256 net, Split sp,
   }
 }
 
-// SMs per role.  A row SM needs about 10.5 k cycles per tile (its stores), a W2 SM 2.3 k and a W1 SM 2.5 k plus 0.9 k per
-// further slab of its group.
+// SMs per role, in proportion to weights that come from timing splits of 148 SMs (the roles slow one another through L2, so the
+// cycles that each takes by itself, see above, are no guide).  One gradient, us:
+//   one slab (8 agents, 4096 environments x 64 steps; the rule gives 102 row, 22 W2, 24 W1 SMs: 1850)
+//     W2 SMs 16 / 19 / 22 / 25 / 28 with 24 W1: 2171 / 1912 / 1850 / 1803 / 1917;  W1 18 / 21 / 27 / 30 with 22 W2: 2112 / 1863 / 1807 / 2000
+//   four slabs (actor and critic of 4 agents, 4096 x 64; the rule gives the critic 100, 12 and 2 x 18: 1470)
+//     W2 SMs 6 / 9 / 15 / 18: 1714 / 1500 / 1465 / 1484;  W1 12 / 15 / 21 / 24 per pair of slabs: 1557 / 1472 / 1473 / 1510
+// Too few of a role costs much, a few more than the rule gives little either way (full batches, under the power cap: within 5 %).
 Split make_split(long long tiles, int sms, int slabs) {
   Split s{};
   s.n_tiles = static_cast<int>(tiles);

@@ -1,6 +1,6 @@
 """Run one workload a few times through the C ABI and print the device times (for profilers).
 
-    python -m paper_2107_01460_b200.run_once --workload 2 [--precision bf16|fp32] [--repeats 3] [--envs E] [--update]
+    python -m paper_2107_01460_b200.run_once --workload 2|NAME [--precision bf16|fp32] [--repeats 3] [--envs E] [--update]
 """
 from __future__ import annotations
 
@@ -13,7 +13,7 @@ from . import binding, build, workloads as wl
 
 def main():
     ap = argparse.ArgumentParser()
-    ap.add_argument("--workload", type=int, default=1)
+    ap.add_argument("--workload", type=lambda v: int(v) if v.isdigit() else v, default=1, help="index or name")
     ap.add_argument("--precision", default=None, choices=[None, "bf16", "fp32"])
     ap.add_argument("--repeats", type=int, default=3)
     ap.add_argument("--envs", type=int, default=None, help="override the number of environments")

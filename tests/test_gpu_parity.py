@@ -76,9 +76,8 @@ def test_reduced_configs_fp32(idx, n_envs, T):
                                                # round in which one thread group of a CTA has no tile (on 148 SMs)
                                                (4, 4737, 12, ""), (3, 9473, 7, "")])
 def test_reduced_configs_bf16(idx, n_envs, T, mode):
-    """mode "tmem" keeps the hidden activations in tensor memory (the layout H = 256 always uses);
-    "wide" forces 128-row tiles where the batch is small enough for the few-rows form of the kernel
-    (H = 128: up to 16 rows per SM at 333 / 300 environments, up to 32 at 1500 / 1000)."""
+    """"wide" and "tmem" (two flags that ask for the same) force 128-row tiles where the batch is small enough for the few-rows
+    form of the kernel (up to 16 rows per SM at 16 / 333 / 300 environments, up to 32 at 1500 / 1000)."""
     w = wl.workload(idx)
     if not _tc_available(w):
         pytest.skip("bf16 tensor-core path not compiled for this shape")
