@@ -192,6 +192,7 @@ gae_kernel_v4(const float *values, const float *rewards, const uint8_t *dones, f
 // advantages and returns with streaming 16-byte stores.  The done flag selects the factor (gamma or 0,
 // gamma lambda or 0) instead of multiplying it in.  Every mbarrier wait is bounded.
 constexpr int kGaeStages = 3, kGaeL = 4;
+constexpr size_t kGaeMaxSmem = 232000;  // of a block (the limit is 232448)
 
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1)
@@ -383,10 +384,10 @@ cudaError_t launch_gae(mava_rollout *h, float gamma, float lambda) {
       const size_t stage = (static_cast<size_t>(2 * T + 1) * C * 4 + static_cast<size_t>(T) * W + 127) / 128 * 128;
       smem = kGaeStages * stage + 2 * static_cast<size_t>(n_chunks) * (C / 4) * sizeof(float4) + 2 * kGaeStages * 8;
       threads = ((C / 4) * n_chunks + 31) / 32 * 32;
-      if (C == 32 || (smem <= 232000 && threads <= 1024 && M / C >= static_cast<size_t>(4 * sms))) break;
+      if (C == 32 || (smem <= kGaeMaxSmem && threads <= 1024 && M / C >= static_cast<size_t>(4 * sms))) break;
     }
     CUtensorMap map_v, map_r, map_d;
-    if (threads <= 1024 && smem <= 232000 && W <= 256 &&
+    if (threads <= 1024 && smem <= kGaeMaxSmem && W <= 256 &&
         encode_f32_map(&map_v, b.values, M, static_cast<unsigned long long>(T) + 1, C, T + 1, CU_TENSOR_MAP_SWIZZLE_NONE) &&
         encode_f32_map(&map_r, b.rewards, M, T, C, T, CU_TENSOR_MAP_SWIZZLE_NONE) &&
         encode_map_2d(&map_d, b.dones, true, E, T, W, T, CU_TENSOR_MAP_SWIZZLE_NONE)) {
@@ -394,7 +395,9 @@ cudaError_t launch_gae(mava_rollout *h, float gamma, float lambda) {
       const int expire = (h->expire_next & MAVA_EXPIRE_GAE) ? 1 : 0;
       h->expire_next &= ~MAVA_EXPIRE_GAE;
       auto run = [&](auto kern) {
-        cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        // the most that any launch takes, not this launch's: the attribute belongs to the kernel, and another thread may be
+        // launching it with another size
+        cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kGaeMaxSmem));
         if (err != cudaSuccess) return err;
         h->launches += 1;
         return launch_dependent(kern, n_tiles < sms ? n_tiles : sms, threads, smem, h->stream, map_v, map_r, map_d, b.adv, b.ret, T, E, N, C, W, n_tiles,

@@ -403,7 +403,8 @@ static cudaError_t plan_update(const mava_rollout *h, int n_env, UpdPlan &plan) 
     const size_t smem_max = upd_smem_bytes(central ? N * h->D : h->D, H);
     plan.kern = H == 64 ? ppo_net_kernel<64> : (H == 128 ? ppo_net_kernel<128> : (H == 256 ? ppo_net_kernel<256> : nullptr));
     if (!plan.kern) return cudaErrorNotSupported;
-    err = cudaFuncSetAttribute(plan.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_max));
+    // (the most of any shape: the attribute belongs to the kernel, and another thread may be launching it for another shape)
+    err = cudaFuncSetAttribute(plan.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(upd_smem_bytes(kMaxAgents * (kObsFixed + kMaxAgents), 256)));
     if (err != cudaSuccess) return err;
     int per_sm = 1;
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, plan.kern, H, smem_max);
@@ -501,8 +502,6 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
   if (err != cudaSuccess) return err;
   auto run_net = [&](const UpdNet &net, const UpdRows &rows) {
     const size_t smem = upd_smem_bytes(net.Din, net.H);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
     kern<<<slices, net.H, smem, st>>>(net, rows, hp, adv.out, sc.partial, P, sc.term_part, h->d_status);
     h->launches += 1;
     return cudaGetLastError();

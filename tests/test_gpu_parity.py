@@ -427,3 +427,56 @@ def test_collect_host_where_a_piece_starts_off_a_16_byte_boundary(name, n_envs, 
         assert torch.equal(out[n][:rows], getattr(a, n)[:rows].cpu()), n
     assert np.array_equal(a.get_state(), b.get_state())
     assert a.status() == 0 and b.status() == 0
+
+
+@pytest.mark.parametrize("work,shapes", [("gae", [(2, BF16, 5488, 40), (2, BF16, 5488, 101), (1, BF16, 8208, 64)]),
+                                         ("grad", [(3, FP32, 8, 4), (4, FP32, 8, 4), (1, FP32, 8, 4)])])
+def test_handles_in_threads_of_their_own(work, shapes):
+    """Handles of different shapes, each with a stream and a host thread of its own, that share kernels: every call is
+    accepted and leaves the bytes that the handle leaves alone.  (The largest shared-memory size a kernel may be launched
+    with belongs to the kernel: set to each launch's own need, one thread's launch was refused after another's setting.)"""
+    import ctypes as C
+    import threading
+
+    import torch
+
+    lib, hp, jobs, keep = binding.lib(), binding.ppo_defaults(), [], []
+    for idx, precision, n_envs, T in shapes:
+        w = wl.workload(idx)
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            ro = binding.Rollout(binding.make_config(w, precision=precision, max_T=T, n_envs=n_envs))
+            p = torch.from_numpy(wl.make_params(w)).cuda()
+            ro.run(p, T)
+            ro.gae(wl.GAMMA, wl.LAMBDA)
+            grad = torch.zeros_like(p)
+        if work == "gae":
+            def job(ro=ro):
+                return lib.mava_gae(ro.handle, wl.GAMMA, wl.LAMBDA)
+            out = ro.adv
+        else:
+            def job(ro=ro, p=p, grad=grad):
+                return lib.mava_ppo_grad(ro.handle, p.data_ptr(), C.byref(hp), grad.data_ptr(), None)
+            out = grad
+        assert job() == binding.MAVA_OK
+        torch.cuda.synchronize()
+        keep.append((ro, p, out, out.clone()))
+        jobs.append(job)
+    refused = [0] * len(jobs)
+    start = threading.Barrier(len(jobs))
+
+    def many(i):
+        start.wait()
+        for _ in range(1000):
+            refused[i] += jobs[i]() != binding.MAVA_OK
+
+    threads = [threading.Thread(target=many, args=(i,)) for i in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert refused == [0] * len(jobs)
+    for ro, _, out, alone in keep:
+        assert ro.status() == binding.MAVA_OK and torch.equal(out, alone)
+        ro.close()
