@@ -59,7 +59,7 @@ ppo_net_kernel(UpdNet net, UpdRows rows, UpdHyper hp, const double *__restrict__
     const long long row0 = tile * kUpdRows;
     const int n_valid = static_cast<int>(min(static_cast<long long>(kUpdRows), rows.n - row0));
     if (j < kUpdRows) {
-      const long long row = j < n_valid ? real_row(rows, row0 + j) : -1;
+      const long long row = j < n_valid ? real_row_any(rows, row0 + j) : -1;
       rmap[j] = row;
       if (j < n_valid && row < 0) atomicExch(status, kStatusBadIndex);
     }
@@ -284,10 +284,11 @@ ppo_net_kernel(UpdNet net, UpdRows rows, UpdHyper hp, const double *__restrict__
   }
 }
 
+template <class U>
 __global__ void __launch_bounds__(256) moments_kernel(Moments m) {  // of the advantages
   dependents_may_start();
   wait_for_predecessor();
-  moments_block(m);
+  moments_block<U>(m);
 }
 
 __global__ void adam_kernel(float *params, const float *grad, float *m, float *v, size_t n, const double *stats, float max_norm, float lr,
@@ -452,7 +453,7 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
   cudaStream_t st = h->stream;
   UpdRows rows{};
   rows.x = h->buf.obs; rows.actions = h->buf.actions; rows.logp_old = h->buf.logp; rows.adv = h->buf.adv; rows.n = R;
-  set_minibatch(rows, env_ids_dev, n_env, E, N);
+  rows.env_ids = env_ids_dev; rows.n_ids = n_env; rows.E = E; rows.per_env = N;
   if (!central) { rows.value_old = h->buf.values; rows.ret = h->buf.ret; rows.vstride = 1; }
 
   if (update_takes_tensor_cores(cfg, D)) {
@@ -464,7 +465,7 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
 
   UpdRows crows{};  // the centralised critic's: a row is an environment-step
   crows.x = h->buf.obs; crows.value_old = h->buf.values; crows.ret = h->buf.ret; crows.vstride = N; crows.n = S;
-  set_minibatch(crows, env_ids_dev, n_env, E, 1);
+  crows.env_ids = env_ids_dev; crows.n_ids = n_env; crows.E = E; crows.per_env = 1;
 
   // H = 256 on the tensor cores: the actor / shared-torso net and, one input slab per agent, the centralised critic's
   if (update_takes_tensor_cores_256(cfg, D)) {
@@ -495,7 +496,7 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
   tr(L.W1, H, D); tr(L.W2, H, H);
   if (central) { tr(L.C1, H, joint); tr(L.C2, H, H); }
   const Moments adv = moments_of(h, kAdvMoments, h->buf.adv, R, rows);
-  err = launch_dependent(moments_kernel, kMomentBlocks, 256, 0, st, adv);
+  err = launch_dependent(rows_need_64_bits(rows, R) ? moments_kernel<uint64_t> : moments_kernel<uint32_t>, kMomentBlocks, 256, 0, st, adv);
   h->launches += 1;
   if (err == cudaSuccess) err = cudaMemsetAsync(sc.term_part, 0, sizeof(double) * 3 * 8 * slices, st);
   if (err == cudaSuccess) err = cudaMemsetAsync(sc.partial, 0, sizeof(float) * P * slices, st);

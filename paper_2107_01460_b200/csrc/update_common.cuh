@@ -27,51 +27,24 @@ struct UpdRows {
   // nullptr = every environment in order (row q is row q of the arrays)
   const int32_t *env_ids;
   int n_ids, E, per_env;
-  uint64_t per_step_recip, per_env_recip;  // of n_ids * per_env and of per_env (quotient), in 64 and in 32 bits
-  uint32_t per_step_recip32, per_env_recip32;
 };
-inline void set_minibatch(UpdRows &rows, const int32_t *env_ids, int n_ids, int E, int per_env) {
-  const uint64_t per_step = static_cast<uint64_t>(n_ids) * per_env;
-  rows.env_ids = env_ids; rows.n_ids = n_ids; rows.E = E; rows.per_env = per_env;
-  rows.per_step_recip = ~uint64_t{0} / per_step; rows.per_env_recip = ~uint64_t{0} / per_env;
-  rows.per_step_recip32 = static_cast<uint32_t>(~uint32_t{0} / per_step); rows.per_env_recip32 = ~uint32_t{0} / per_env;
-}
 
-// floor(q / d) and the remainder by recip = floor((2^w - 1) / d), w = 32 or 64 the width: the product's upper half is the
-// quotient or one less, because q recip / 2^w > q / d - 1.
-__device__ __forceinline__ uint32_t mul_high(uint32_t a, uint32_t b) { return __umulhi(a, b); }
-__device__ __forceinline__ uint64_t mul_high(uint64_t a, uint64_t b) { return __umul64hi(a, b); }
-template <class U>
-__device__ __forceinline__ U quotient(U q, U d, U recip, U &rem) {
-  U t = mul_high(q, recip);
-  rem = q - t * d;
-  if (rem >= d) { ++t; rem -= d; }
-  return t;
-}
 // Row of the trajectory arrays behind row q of the batch; -1 when the environment index is out of range.  U holds the batch's
 // row numbers: 32 bits for what is cut from a trajectory without repetition (a row is 340 bytes of observation alone, so
-// fewer than 2^31 fit a GPU); a minibatch that repeats environments may be longer than its trajectory and need 64.
+// fewer than 2^31 fit a GPU); a minibatch that repeats environments may be longer than its trajectory and need 64.  The kernels
+// of the small nets are compiled for either (choosing at run time cost them 0.5 to 0.9 us a minibatch).
 template <class U>
-__device__ __forceinline__ long long real_row_as(const UpdRows &rows, U q) {
-  const U per_env = static_cast<U>(rows.per_env);
-  U rem, slot, t, i;
-  if constexpr (sizeof(U) == 4) {
-    t = quotient(q, static_cast<U>(rows.n_ids) * per_env, rows.per_step_recip32, rem);
-    i = quotient(rem, per_env, rows.per_env_recip32, slot);
-  } else {
-    t = quotient(q, static_cast<U>(rows.n_ids) * per_env, rows.per_step_recip, rem);
-    i = quotient(rem, per_env, rows.per_env_recip, slot);
-  }
+__device__ __forceinline__ long long real_row(const UpdRows &rows, long long row) {
+  if (!rows.env_ids) return row;
+  const U q = static_cast<U>(row), per_env = static_cast<U>(rows.per_env), per_step = static_cast<U>(rows.n_ids) * per_env;
+  const U t = q / per_step, rem = q - t * per_step, i = rem / per_env, slot = rem - i * per_env;
   const int e = rows.env_ids[i];
   if (e < 0 || e >= rows.E) return -1;
-  return static_cast<long long>((static_cast<uint32_t>(t) * static_cast<uint32_t>(rows.E) + static_cast<uint32_t>(e)) * static_cast<uint32_t>(rows.per_env) +
-                                static_cast<uint32_t>(slot));
+  return static_cast<long long>((t * static_cast<uint32_t>(rows.E) + static_cast<uint32_t>(e)) * per_env + slot);
 }
-__device__ __forceinline__ bool rows_need_64_bits(const UpdRows &rows, long long n) { return rows.env_ids && (n >> 32) != 0; }
-__device__ __forceinline__ long long real_row(const UpdRows &rows, long long q) {
-  if (!rows.env_ids) return q;
-  if (rows_need_64_bits(rows, rows.n)) return real_row_as<uint64_t>(rows, static_cast<uint64_t>(q));
-  return real_row_as<uint32_t>(rows, static_cast<uint32_t>(q));
+__host__ __device__ __forceinline__ bool rows_need_64_bits(const UpdRows &rows, long long n) { return rows.env_ids && (n >> 32) != 0; }
+__device__ __forceinline__ long long real_row_any(const UpdRows &rows, long long row) {
+  return rows_need_64_bits(rows, rows.n) ? real_row<uint64_t>(rows, row) : real_row<uint32_t>(rows, row);
 }
 
 // A predicated load (zero otherwise), in program order with its like: the compiler neither branches around it nor puts a use
@@ -151,48 +124,41 @@ __device__ __forceinline__ void moments_finish(const Moments &m, double a, doubl
   const double mean = a / static_cast<double>(m.n), var = fmax(b / static_cast<double>(m.n) - mean * mean, 0.0);
   m.out[0] = mean; m.out[1] = sqrt(var); m.out[2] = sqrt(b);
 }
-template <bool WIDE>
-__device__ __forceinline__ void moments_sums(const Moments &m, double &a, double &b) {
-  // loads in flight per thread (one at a time: 44 us for 16.8 million elements); the wide form, of which a batch takes seconds, must
-  // not cost the kernel registers, i.e. blocks beside those of the kernels in front (58 instead of 32: 0.35 us a minibatch)
-  constexpr int kBatch = WIDE ? 1 : 8;
+template <class U>
+__device__ __forceinline__ void moments_block(const Moments &m) {
+  constexpr int kBatch = 8;  // loads in flight per thread (one at a time: 44 us for 16.8 million elements)
   constexpr long long kStep = 256LL * kMomentBlocks;
+  double a = 0.0, b = 0.0;
   for (long long i = blockIdx.x * 256LL + threadIdx.x; i < m.n; i += kBatch * kStep) {
     float v[kBatch];
 #pragma unroll
     for (int k = 0; k < kBatch; ++k) {
-      const long long q = i + k * kStep, in = q < m.n ? q : i;  // (loads without a branch around them)
-      const long long row = !m.map.env_ids ? in : (WIDE ? real_row_as<uint64_t>(m.map, static_cast<uint64_t>(in)) : real_row_as<uint32_t>(m.map, static_cast<uint32_t>(in)));
+      const long long q = i + k * kStep, row = real_row<U>(m.map, q < m.n ? q : i);  // (loads without a branch around them)
       v[k] = __ldcg(m.x + (row >= 0 ? row : 0));
       if (q >= m.n || row < 0) v[k] = 0.0f;
     }
 #pragma unroll
     for (int k = 0; k < kBatch; ++k) { a += v[k]; b += static_cast<double>(v[k]) * v[k]; }
   }
-}
-__device__ __forceinline__ void moments_block(const Moments &m) {
-  double a = 0.0, b = 0.0;
-  if (rows_need_64_bits(m.map, m.n)) moments_sums<true>(m, a, b);
-  else moments_sums<false>(m, a, b);
   moments_finish(m, a, b);
 }
 // What a gradient call starts with: the advantages' moments and, by the other blocks, the weight image (prep(i, n): thread i
 // of n).  Early moments are taken while the kernels in front (the last minibatch's reduction and optimiser step) still run.
-template <class Prep>
+template <class U, class Prep>
 __global__ void __launch_bounds__(256) prologue_kernel(Moments m, Prep prep) {
   dependents_may_start();
   const int first = m.x ? kMomentBlocks : 0, b = static_cast<int>(blockIdx.x);
-  if (b < first && m.early) moments_block(m);
+  if (b < first && m.early) moments_block<U>(m);
   wait_for_predecessor();
   if (b < first) {
-    if (!m.early) moments_block(m);
+    if (!m.early) moments_block<U>(m);
     return;
   }
   prep((b - first) * 256 + static_cast<int>(threadIdx.x), (static_cast<int>(gridDim.x) - first) * 256);
 }
 template <class Prep>
 cudaError_t launch_prologue(const Moments &m, const Prep &prep, int prep_blocks, cudaStream_t stream) {
-  return launch_dependent(prologue_kernel<Prep>, (m.x ? kMomentBlocks : 0) + prep_blocks, 256, 0, stream, m, prep);
+  return launch_dependent(rows_need_64_bits(m.map, m.n) ? prologue_kernel<uint64_t, Prep> : prologue_kernel<uint32_t, Prep>, (m.x ? kMomentBlocks : 0) + prep_blocks, 256, 0, stream, m, prep);
 }
 
 struct UpdHyper { float clip_eps, ent_coef, vf_coef; };

@@ -132,6 +132,7 @@ struct SliceMap {
   }
 };
 
+template <class U>  // row numbers of the batch (real_row)
 __global__ void __launch_bounds__(kUThreads, 1)
 ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const double *adv_stats,
                   float *partial, double *term_partial, int *status, int D, bool rows_ready) {
@@ -266,7 +267,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
       for (int e = lane; e < 64; e += 32) {  // where this warp's rows lie (both look-ups in flight, before the wait)
         const int c = lw + kULoaders * (e / 16);
         const long long q = tile_of(i) * kUR + 16 * c + (e & 15);
-        if (c < kUR / 16) sm.rmap[16 * c + (e & 15)] = static_cast<int>(q < rows.n ? real_row(rows, q) : -1);
+        if (c < kUR / 16) sm.rmap[16 * c + (e & 15)] = static_cast<int>(q < rows.n ? real_row<U>(rows, q) : -1);
       }
       __syncwarp();
       if (i >= 2) timed_out = !mbar_wait_warp(bar_end, static_cast<uint32_t>(i) & 1u);  // d W1 of tile i - 2 has read this x tile
@@ -368,7 +369,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
   for (int i = 0; i < my_tiles && !timed_out; ++i) {
     const long long row0 = tile_of(i) * kUR;
     const int n_valid = static_cast<int>(min(static_cast<long long>(kUR), rows.n - row0));
-    const long long my_row = row < n_valid ? real_row(rows, row0 + row) : -1;
+    const long long my_row = row < n_valid ? real_row<U>(rows, row0 + row) : -1;
     int action = 0;
     float logp_old = 0.0f, adv = 0.0f, v_old = 0.0f, ret = 0.0f;
     if (half == 0) {
@@ -517,9 +518,10 @@ cudaError_t launch_ppo_net_tc(mava_rollout *h, const float *params_dev, const Pa
   cudaError_t err = launch_prologue(adv, prep, kPrepBlocks, h->stream);
   if (err != cudaSuccess) return err;
   const size_t smem = sizeof(UtcSmem);
-  err = cudaFuncSetAttribute(ppo_net_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const auto kern = rows_need_64_bits(rows, rows.n) ? ppo_net_tc_kernel<uint64_t> : ppo_net_tc_kernel<uint32_t>;
+  err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (err != cudaSuccess) return err;
-  err = launch_dependent(ppo_net_tc_kernel, slices, kUThreads, smem, h->stream, static_cast<const unsigned char *>(image), rows, hp,
+  err = launch_dependent(kern, slices, kUThreads, smem, h->stream, static_cast<const unsigned char *>(image), rows, hp,
                          static_cast<const double *>(adv.out), partial, term_partial, h->d_status, h->D, adv.early);
   if (err != cudaSuccess) return err;
   h->launches += 3;

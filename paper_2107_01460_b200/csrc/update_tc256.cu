@@ -322,7 +322,7 @@ __device__ __forceinline__ bool row_role(const Upd256Args &a, RowSmem &sm, uint3
       const int lt = tile_of(s);
       const long long row0 = static_cast<long long>(lt) * kR;
       unsigned char *slot = a.ring + static_cast<size_t>(lt % sp.n_slots) * slot_size;
-      const long long my_row = row0 + row < a.rows.n ? real_row(a.rows, row0 + row) : -1;
+      const long long my_row = row0 + row < a.rows.n ? real_row_any(a.rows, row0 + row) : -1;
       int action = 0;
       float logp_old = 0.0f, adv = 0.0f, v_old = 0.0f, ret = 0.0f;
       if (row0 + row < a.rows.n && my_row < 0) atomicExch(a.status, kStatusBadIndex);
@@ -440,7 +440,7 @@ __device__ __forceinline__ bool row_role(const Upd256Args &a, RowSmem &sm, uint3
       const int lt = tile_of(s), use = lt / sp.n_slots, slot_no = lt - use * sp.n_slots;
       const long long q = static_cast<long long>(lt) * kR + 32 * lw + lane;
       __syncwarp();
-      sm.rmap[32 * lw + lane] = static_cast<int>(q < a.rows.n ? real_row(a.rows, q) : -1);
+      sm.rmap[32 * lw + lane] = static_cast<int>(q < a.rows.n ? real_row_any(a.rows, q) : -1);
       __syncwarp();
       unsigned char *slot = a.ring + static_cast<size_t>(slot_no) * slot_size;
       for (int sl = 0; sl < slabs && ok; ++sl, ++n) {
