@@ -286,6 +286,7 @@ __device__ __forceinline__ bool epilogue_half(uint32_t acc, uint32_t hid, uint32
 // order, one group half a tile behind the other (one group's epilogue runs beside the other's products, and tiles are
 // finished one by one: with both groups in step they came in pairs and the ring of slots ran dry).  Warp 13: hands finished
 // tiles over.
+template <class U>  // row numbers of the batch (real_row)
 __device__ __forceinline__ bool row_role(const Upd256Args &a, RowSmem &sm, uint32_t tmem) {
   const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;  // (warp: uniform to the compiler)
   const Split &sp = a.sp;
@@ -322,7 +323,7 @@ __device__ __forceinline__ bool row_role(const Upd256Args &a, RowSmem &sm, uint3
       const int lt = tile_of(s);
       const long long row0 = static_cast<long long>(lt) * kR;
       unsigned char *slot = a.ring + static_cast<size_t>(lt % sp.n_slots) * slot_size;
-      const long long my_row = row0 + row < a.rows.n ? real_row_any(a.rows, row0 + row) : -1;
+      const long long my_row = row0 + row < a.rows.n ? real_row<U>(a.rows, row0 + row) : -1;
       int action = 0;
       float logp_old = 0.0f, adv = 0.0f, v_old = 0.0f, ret = 0.0f;
       if (row0 + row < a.rows.n && my_row < 0) atomicExch(a.status, kStatusBadIndex);
@@ -440,7 +441,7 @@ __device__ __forceinline__ bool row_role(const Upd256Args &a, RowSmem &sm, uint3
       const int lt = tile_of(s), use = lt / sp.n_slots, slot_no = lt - use * sp.n_slots;
       const long long q = static_cast<long long>(lt) * kR + 32 * lw + lane;
       __syncwarp();
-      sm.rmap[32 * lw + lane] = static_cast<int>(q < a.rows.n ? real_row_any(a.rows, q) : -1);
+      sm.rmap[32 * lw + lane] = static_cast<int>(q < a.rows.n ? real_row<U>(a.rows, q) : -1);
       __syncwarp();
       unsigned char *slot = a.ring + static_cast<size_t>(slot_no) * slot_size;
       for (int sl = 0; sl < slabs && ok; ++sl, ++n) {
@@ -832,6 +833,7 @@ __device__ __forceinline__ bool weight_role(const Upd256Args &a, WgtSmem &sm, ui
   return ok;
 }
 
+template <class U>
 __global__ void __launch_bounds__(kThreads, 1) ppo_update256_kernel(const __grid_constant__ Upd256Args a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -887,7 +889,7 @@ __global__ void __launch_bounds__(kThreads, 1) ppo_update256_kernel(const __grid
     }
     ok = mbar_wait(smem_u32(&rs.bar_load), 0);
     ok = __syncthreads_and(ok) != 0;
-    if (ok) ok = row_role(a, rs, tmem);
+    if (ok) ok = row_role<U>(a, rs, tmem);
     ok = __syncthreads_and(ok) != 0;
     if (tid <= kActions) {
       float s = 0.0f;
@@ -1021,11 +1023,12 @@ cudaError_t launch_ppo_net_tc256(mava_rollout *h, const float *params_dev, const
   if (desc.has_value) { terms.value = a.term_partial; terms.n_value_part = 8 * a.sp.n_row; }
   cudaError_t err = launch_prologue(adv, Prep256{params_dev, base + L.image, net, a.full, 3 * a.sp.n_slots}, 64, h->stream);
   if (err != cudaSuccess) return err;
-  err = cudaFuncSetAttribute(ppo_update256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes));
+  const auto kern = rows_need_64_bits(rows, rows.n) ? ppo_update256_kernel<uint64_t> : ppo_update256_kernel<uint32_t>;
+  err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes));
   if (err != cudaSuccess) return err;
   void *args[] = {&a};
   const int grid = a.sp.n_row + a.sp.n_w2 + a.sp.groups * a.sp.n_w1;
-  err = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(ppo_update256_kernel), dim3(grid), dim3(kThreads), args, kSmemBytes, h->stream);
+  err = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kern), dim3(grid), dim3(kThreads), args, kSmemBytes, h->stream);
   if (err != cudaSuccess) return err;
   reduce256_kernel<<<2 * sms, 256, 0, h->stream>>>(grad, net, a.sp, a.part_w2, a.part_w1, a.part_head, desc.has_value ? terms : TermSums{});
   h->launches += 3;

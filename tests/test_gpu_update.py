@@ -331,7 +331,7 @@ def test_h256_update_where_its_tiles_and_rings_turn_over(idx, n_envs, T):
     ro.close()
 
 
-@pytest.mark.parametrize("idx,T", [(0, 256), (2, 128)])
+@pytest.mark.parametrize("idx,T", [(0, 256), (2, 128), (4, 64)])
 def test_a_batch_of_more_than_2_to_the_32_rows(idx, T):
     """Environments may be repeated in a minibatch, so it can be longer than its trajectory.  Every environment taken the same
     number of times gives the loss terms of the plain call (their sums are kept in double: what is left is the order, below
