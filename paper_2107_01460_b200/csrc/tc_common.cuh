@@ -41,6 +41,22 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
 }
 // The same by all lanes of a warp, with one answer for all of them: what follows may need the warp converged (elect_one).
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) { return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity)) != 0; }
+// The same where many warps wait at once: each try sleeps for up to kSleepNs, so that the polls of the sleepers do not take the
+// issue slots and the shared-memory pipe of the warps that work.  Limit: kSleepLimit tries, about four seconds.
+constexpr uint32_t kSleepNs = 4000, kSleepLimit = 1u << 20;
+__device__ __forceinline__ bool mbar_sleep_warp(uint32_t bar, uint32_t parity) {
+  uint32_t ok = 0;
+#pragma unroll 1
+  for (uint32_t i = 0; i < kSleepLimit && !ok; ++i)
+    asm volatile(
+        "{\n.reg .pred p;\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
+        "selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity), "r"(kSleepNs)
+        : "memory");
+  return __all_sync(0xFFFFFFFFu, ok) != 0;
+}
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                "l"(src), "r"(bytes), "r"(bar)

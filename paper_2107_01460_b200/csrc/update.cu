@@ -458,7 +458,7 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
 
   if (update_takes_tensor_cores(cfg, D)) {
     const UpdScratch sc = carve(h, ppo_tc_slice_floats(), slices);
-    const TermSums terms{sc.term_part, sc.term_part, 8 * slices, 8 * slices, R, R, hp, terms_dev};
+    const TermSums terms{sc.term_part, sc.term_part, 4 * slices, 4 * slices, R, R, hp, terms_dev};
     return launch_ppo_net_tc(h, params_dev, L, rows, hp, moments_of(h, seq & 1 ? kAdvMoments2 : kAdvMoments, h->buf.adv, R, rows, seq > 0), sc.image, sc.partial, sc.term_part, slices,
                              grad_dev, terms, moments_of(h, kGradMoments, grad_dev, static_cast<long long>(P), UpdRows{}));
   }

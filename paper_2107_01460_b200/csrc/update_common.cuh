@@ -56,6 +56,24 @@ __device__ __forceinline__ float ldg_if(const float *p, bool pred) {
                : "l"(p), "r"(static_cast<uint32_t>(pred)));
   return v;
 }
+// The same for lines that another load of the warp reads as well.
+__device__ __forceinline__ float ldg_if_cached(const float *p, bool pred) {
+  float v;
+  asm volatile("{\n.reg .pred q;\nsetp.ne.u32 q, %2, 0;\nmov.f32 %0, 0f00000000;\n@q ld.global.f32 %0, [%1];\n}" : "=f"(v) : "l"(p), "r"(static_cast<uint32_t>(pred)));
+  return v;
+}
+// real_row in two parts, so that the look-up of the environment can be on its way while other work goes on: the row is
+// at + e * per_env for an e that is one of the environments.
+struct RowLookup { int at, e; };
+template <class U>
+__device__ __forceinline__ RowLookup row_lookup(const UpdRows &rows, long long row, bool valid) {
+  if (!rows.env_ids) return RowLookup{static_cast<int>(row), valid ? 0 : -1};
+  const U q = static_cast<U>(row), per_env = static_cast<U>(rows.per_env), per_step = static_cast<U>(rows.n_ids) * per_env;
+  const U t = q / per_step, rem = q - t * per_step, i = rem / per_env, slot = rem - i * per_env;
+  const int e = __float_as_int(ldg_if_cached(reinterpret_cast<const float *>(rows.env_ids) + (valid ? i : 0), valid));
+  return RowLookup{static_cast<int>(static_cast<uint32_t>(t) * static_cast<uint32_t>(rows.E) * static_cast<uint32_t>(rows.per_env) + static_cast<uint32_t>(slot)), valid ? e : -1};
+}
+__device__ __forceinline__ int row_found(const UpdRows &rows, RowLookup l) { return l.e >= 0 && l.e < rows.E ? l.at + l.e * rows.per_env : -1; }
 // ---- two accumulator columns at a time: the epilogues of the tensor-core kernels --------------------------------------------
 // All-ones in each half of the result whose bf16 in `v` is positive.
 __device__ __forceinline__ uint32_t positive_mask(uint32_t v) {
@@ -170,7 +188,7 @@ size_t ppo_tc_slice_floats();
 struct TermSums;
 // Enqueues the prologue (moments of the advantages, weight image), the loss/gradient kernel and the reduction of its slices
 // into `grad`, the loss terms and the gradient's moments; `partial` holds `slices` slices of ppo_tc_slice_floats() floats (one
-// per CTA), `term_partial` 8 x 3 doubles per slice.
+// per CTA), `term_partial` 4 x 3 doubles per slice.
 cudaError_t launch_ppo_net_tc(mava_rollout *h, const float *params_dev, const ParamLayout &L, const UpdRows &rows, const UpdHyper &hp,
                               const Moments &adv, void *image, float *partial, double *term_partial, int slices, float *grad, const TermSums &terms,
                               const Moments &norm);

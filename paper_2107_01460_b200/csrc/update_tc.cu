@@ -11,6 +11,15 @@
 //   per tile:  x -> z1 -> h1 -> z2 -> h2 -> logits, value -> loss and its per-row derivatives (fp32, thread = row)
 //              -> d h2 -> d z2 -> d h1 -> d z1, and on the side d Wh^T += h2^T . dhead, d W2 += d z2^T . h1,
 //              d W1 += d z1^T . x, d b2 += d z2^T . 1, d b1 += d z1^T . 1 (the ones are column 7 of the dhead tile).
+// Two tiles are in flight: tile s goes forward while tile s - 1 goes backward, so that one's epilogue runs beside the other's products.
+// Both fit an SM because d z2 takes h2's place and d z1 h1's (behind the weight-gradient products that read them), and
+// the heads' derivatives are kept once, eight columns wide.  Sixteen warps share every epilogue (32 rows x 32 columns each), eight
+// bring the rows in, one issues the MMAs in a fixed order, one fetches what the loss needs.  What bounds it (10x10, 61 k rows a
+// gradient): 6.7 k cycles per tile and SM against 8 k for one tile at a time; the products are 3.4 k of them, the rest is the
+// row of dependent epilogues (0.6 to 0.8 k each, half of it conversions and gate bits at half rate) and the waits between them.
+// Rows: fewer than 40 KB can be on their way through the 28 KB of L1 that are left; with more loads in flight, or the look-up of a
+// row in front of an epilogue, every other access of the SM stalls behind them.  Two passes of three minibatches over 549 k rows:
+// 407 -> 376 us; sixteen minibatches of 33 k rows: 502 -> 478.
 // The weight-gradient accumulators stay in tensor memory for all tiles of the CTA and are written once, into the CTA's
 // own slice of the partial-gradient array; a last kernel adds the slices in a fixed order (reduce_slices_kernel: four quarters of
 // them, each in slice order), so the gradient is the same bytes on every call.  Rounding points are those of the bf16-operand
@@ -19,6 +28,7 @@
 // MMAs are issued by one elected lane; tcgen05.commit tracks all MMAs issued before it, so a tile buffer may be rewritten as
 // soon as a later commit has been waited for.  Every mbarrier wait is bounded.
 #include <cuda_bf16.h>
+#include <stddef.h>
 
 #include "common.cuh"
 #include "layout.h"
@@ -31,35 +41,48 @@ namespace {
 constexpr int kUR = 128;        // rows per tile (M of the per-row products, K of the weight-gradient products)
 constexpr int kUH = 128;        // hidden width, padded
 constexpr int kUK1 = 80;        // input width, padded to the MMA's K step
-constexpr int kUHeads = 16;     // six logits, the value, a column of ones, eight columns of zeros
-constexpr int kUMain = 256;     // threads of the epilogues: thread = (row, column half)
-constexpr int kULoaders = 3;    // warps that bring the rows in (with a fourth, 13 warps would leave 128 registers per thread, which spill)
-constexpr int kUThreads = kUMain + 32 * kULoaders + 32;  // and one that issues the MMAs
+constexpr int kUHeads = 16;     // N of the products with the heads: six logits, the value, a column of ones; the other eight repeat or are not read
+constexpr int kUHeadRows = 8;   // of which these exist in memory
+constexpr int kUMain = 512;     // threads of the epilogues: a warp has 32 rows x 32 columns of a tile
+constexpr int kLossWarps = 8;   // of which these also do the loss: four the actor's part, four the value's, a row per thread
+constexpr int kULoaders = 8;    // warps that bring the rows in, 16 rows each
+constexpr int kUThreads = kUMain + 32 * kULoaders + 128;  // and a warpgroup: one warp issues the MMAs, one fetches what the loss needs
 
-// weight image: bf16 tiles W1 [H][K1], W2 [H][H], Wh [16][H]; then fp32 b1 [H], b2 [H], bh [8]
-constexpr uint32_t kImgW1 = 0, kImgW2 = kImgW1 + kUH * kUK1 * 2, kImgWh = kImgW2 + kUH * kUH * 2;
-constexpr uint32_t kImgB1 = kImgWh + kUHeads * kUH * 2, kImgB2 = kImgB1 + kUH * 4, kImgBh = kImgB2 + kUH * 4;
-constexpr uint32_t kImgBytes = kImgBh + 32;
-static_assert(kImgBytes % 16 == 0, "one bulk copy");
+// weight image: fp32 b1 [H], b2 [H], bh [8]; then bf16 tiles W1 [H][K1], Wh [8][H], W2 [H][H] (the heads as an N = 16 operand: what lies
+// behind them gives columns that nobody reads)
+constexpr uint32_t kImgB1 = 0, kImgB2 = kImgB1 + kUH * 4, kImgBh = kImgB2 + kUH * 4, kImgW1 = kImgBh + 32;
+constexpr uint32_t kImgWh = kImgW1 + kUH * kUK1 * 2, kImgW2 = kImgWh + kUHeadRows * kUH * 2, kImgBytes = kImgW2 + kUH * kUH * 2;
+static_assert(kImgBytes % 16 == 0 && kImgWh % 16 == 0, "bulk copies");
 
-// tensor-memory columns
-constexpr uint32_t kColAcc = 0, kColDW2 = 128, kColDW1 = 256, kColHead = 352, kColDWh = 384, kColDB2 = 416, kColDB1 = 448;
+// tensor-memory columns: an accumulator per tile in flight, used by z1, z2, the heads, d h2 and d h1 in turn; the weight gradients
+constexpr uint32_t kColAcc = 0, kColDW2 = 256, kColDW1 = 384, kColDWh = 464, kColDB2 = 480, kColDB1 = 496;
 constexpr uint32_t kTmemCols = 512;
 
-struct UtcSmem {
-  alignas(128) unsigned char img[(kImgBytes + 127) / 128 * 128];
-  alignas(128) unsigned char x[2][(kUR / 8) * (kUK1 / 8) * kALbo];  // feature chunks 144 bytes apart (see a_offset): the
-                                                                    // converter's 2-byte stores then spread over the banks
-  alignas(128) unsigned char h1[kUR * kUH * 2];
-  alignas(128) unsigned char h2[kUR * kUH * 2];   // d z1 once h2's last reader is done
-  alignas(128) unsigned char dz2[kUR * kUH * 2];
-  alignas(128) unsigned char dhead[kUR * kUHeads * 2];
-  int rmap[kUR];  // trajectory rows of the tile that is being fetched
-  float red[4][8];
-  alignas(8) uint64_t bar_load, bar_mma, bar_end, x_full[2];
+// The x tile is [feature chunk][row], 16 bytes more than the rows need from chunk to chunk: the loaders' stores (lane = two
+// features) then spread over the banks.
+constexpr uint32_t kXChunk = kUR * 16 + 16, kXTile = (kUK1 / 8) * kXChunk;
+constexpr uint32_t kHTile = kUR * kUH * 2;
+// At the end, in W2's place (its last reader is done): sums over the CTA's rows of the heads' bias gradients and of the loss terms
+struct UtcSums { double term[4][3]; float bias[4][8]; };
+
+// Products that an epilogue waits for, and epilogues that a product waits for: a barrier each, one phase per tile.
+enum { kZ1, kZ2, kLogits, kDh2, kDWh, kDh1, kDW2, kProducts };
+enum { kH1, kH2, kLoss, kDz2, kDz1, kEpilogues };
+
+struct UtcSmem {  // two tiles are in flight, an even and an odd one
+  alignas(128) unsigned char h1[2][kHTile];  // d z1 once d W2 has read h1
+  alignas(128) unsigned char h2[2][kHTile];  // d z2 once d Wh has read h2
+  alignas(128) unsigned char x[2][kXTile];
+  alignas(128) unsigned char dhead[kUR * kUHeadRows * 2];  // of either tile: one's last reader is done before the other's loss
+  alignas(128) unsigned char img[kImgBytes];
+  // what the loss needs of a tile's rows (the old log-probs and advantages take the place of the biases, which are in registers by then)
+  float value_old[kUR], ret[kUR];
+  unsigned char action[kUR];  // 0xFF: no such row
+  alignas(8) uint64_t bar_load[2], done[kProducts], ready[kEpilogues], x_full[2], x_empty[2], rows_full, bar_end;
   uint32_t tmem_base;
-  int abort;  // the main threads gave up
+  int abort;  // a warp gave up
 };
+static_assert(sizeof(UtcSmem) <= 232448, "shared memory of a block");
 
 struct PrepImage {
   const float *params;
@@ -69,7 +92,7 @@ struct PrepImage {
   __device__ void operator()(int tid, int nth) const;
 };
 // One element per thread: a kernel that everything behind it waits for (as loops over the parts with 8 k threads it took 3 us more).
-constexpr int kPrepW1 = kUH * kUK1, kPrepW2 = kUH * kUH, kPrepWh = kUHeads * kUH, kPrepTotal = kPrepW1 + kPrepW2 + kPrepWh + 2 * kUH + 8;
+constexpr int kPrepW1 = kUH * kUK1, kPrepW2 = kUH * kUH, kPrepWh = kUHeadRows * kUH, kPrepTotal = kPrepW1 + kPrepW2 + kPrepWh + 2 * kUH + 8;
 constexpr int kPrepBlocks = (kPrepTotal + 255) / 256;
 __device__ __forceinline__ void PrepImage::operator()(int tid, int nth) const {
   for (int i = tid; i < kPrepTotal; i += nth) {
@@ -98,13 +121,17 @@ __device__ __forceinline__ void PrepImage::operator()(int tid, int nth) const {
   }
 }
 
-// Descriptor of a canonical tile of C features read with the feature index as K (step k = features 16 k ..).
-__device__ __forceinline__ uint64_t desc_k(uint32_t tile, int C, int k) { return smem_desc(tile + k * 256, 128, C * 16); }
-// The same tile read with the row index as K (step k = rows 16 k ..): the 8-row groups are the K groups, the feature
-// chunks the MN groups: the descriptor's leading-dimension offset is then the step between K groups (C*16 bytes) and
-// its stride offset the step between MN groups (128 bytes).
-__device__ __forceinline__ uint64_t desc_mn(uint32_t tile, int C, int k) { return smem_desc(tile + k * 2 * C * 16, C * 16, 128); }
+// A canonical tile of C features read with the feature index as K: chunks (K groups) 128 bytes apart, 8-row groups C*16.  The same tile
+// read with the row index as K: the 8-row groups are the K groups, the feature chunks the MN groups, so the descriptor's
+// leading-dimension offset is C*16 and its stride offset 128.
 constexpr uint32_t kAmn = 1u << 15, kBmn = 1u << 16;  // operand is MN-major
+// A descriptor from an address in 16-byte units: one addition to a word that is otherwise constant (14 bits hold any address of a block).
+template <uint32_t LBO, uint32_t SBO>
+__device__ __forceinline__ uint64_t desc16(uint32_t addr16) {
+  constexpr uint32_t lo = (LBO >> 4) << 16;
+  constexpr uint64_t hi = (static_cast<uint64_t>(SBO >> 4) << 32) | (1ull << 46);
+  return hi | (addr16 + lo);
+}
 
 // A CTA's slice of the partial gradients, matrices as [column / 4][unit][4] so that the lanes of a warp (= units) write whole
 // lines (written row by row in the parameters' order, a slice took 33 k cycles to leave; like this 2 k):
@@ -132,19 +159,68 @@ struct SliceMap {
   }
 };
 
+constexpr int kLoadRows = kUR / kULoaders;  // per loader warp, all of their loads in flight at once
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) { asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory"); }
+// One arrival per warp, after all its lanes are done with what the barrier guards.
+__device__ __forceinline__ void warp_arrive(uint32_t bar, int lane) {
+  __syncwarp();
+  if (lane == 0) mbar_arrive(bar);
+}
+__device__ __forceinline__ void prefetch_l2(const float *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void sts_u32(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+// 16 lanes x 32 columns: thread t gets of lanes t / 4 (r[4 j], r[4 j + 1]) and t / 4 + 8 (r[4 j + 2], r[4 j + 3]) the columns 8 j + 2 (t % 4)
+// and the one behind it.  A thread then has the same eight columns of every row: their biases stay in registers (with a row per
+// thread each warp read all biases again for every tile, as many shared-memory cycles as the stores take).
+__device__ __forceinline__ void tmem_ld_16x32_nowait(uint32_t taddr, uint32_t *r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld_row8(uint32_t taddr, float *v) {  // thread = lane
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+  tmem_ld_wait();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    asm volatile("" : "+r"(r[i]));
+    v[i] = __uint_as_float(r[i]);
+  }
+}
+// Four core matrices (8 rows x 16 bytes) out of registers in the layout above; lane l has the address of row l % 8 of matrix l / 8.
+__device__ __forceinline__ void stmatrix4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+// Waits for the tensor-memory loads; what they brought is not touched before.
+__device__ __forceinline__ void tmem_ld_wait32(uint32_t *r) {
+  tmem_ld_wait();
+#pragma unroll
+  for (int i = 0; i < 32; ++i) asm volatile("" : "+r"(r[i]));
+}
+
 template <class U>  // row numbers of the batch (real_row)
 __global__ void __launch_bounds__(kUThreads, 1)
 ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const double *adv_stats,
-                  float *partial, double *term_partial, int *status, int D, bool rows_ready) {
+                  float *partial, double *term_partial, int *status, int D, int H, bool rows_ready) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   UtcSmem &sm = *reinterpret_cast<UtcSmem *>(smem_raw);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int row = tid & (kUR - 1), half = tid >> 7;
-  const int role = __shfl_sync(0xFFFFFFFFu, warp, 0);  // (uniform to the compiler)
-  const uint32_t bar_load = smem_u32(&sm.bar_load), bar_mma = smem_u32(&sm.bar_mma), bar_end = smem_u32(&sm.bar_end), x_full0 = smem_u32(&sm.x_full[0]);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);  // (uniform to the compiler)
+  const int wq = warp & 3, cq = (warp >> 2) & 3;  // of an epilogue warp: its rows (32, = tensor-memory lanes) and columns (32)
+  const uint32_t bar_load = smem_u32(&sm.bar_load[0]), done0 = smem_u32(&sm.done[0]), ready0 = smem_u32(&sm.ready[0]), x_full0 = smem_u32(&sm.x_full[0]),
+                 x_empty0 = smem_u32(&sm.x_empty[0]), rows_full = smem_u32(&sm.rows_full), bar_end = smem_u32(&sm.bar_end);
   if (tid == 0) {
     sm.abort = 0;
-    mbar_init(bar_load, 1); mbar_init(bar_mma, 1); mbar_init(bar_end, 1); mbar_init(x_full0, kULoaders); mbar_init(x_full0 + 8, kULoaders);
+    for (uint32_t i = 0; i < 2; ++i) { mbar_init(bar_load + 8 * i, 1); mbar_init(x_full0 + 8 * i, kULoaders); mbar_init(x_empty0 + 8 * i, 1); }
+    for (uint32_t i = 0; i < kProducts; ++i) mbar_init(done0 + 8 * i, 1);
+    for (uint32_t i = 0; i < kEpilogues; ++i) mbar_init(ready0 + 8 * i, i == kLoss ? kLossWarps : kUMain / 32);
+    mbar_init(rows_full, 1); mbar_init(bar_end, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -152,347 +228,463 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  // the x tiles' pad columns and the dhead tile's upper eight columns stay zero for the whole run
-  for (int i = tid; i < static_cast<int>(sizeof(sm.x) / 16); i += kUThreads) sts_zero16(smem_u32(sm.x) + 16u * i);
-  for (int i = tid; i < static_cast<int>(sizeof(sm.dhead) / 16); i += kUThreads) sts_zero16(smem_u32(sm.dhead) + 16u * i);
-  fence_async_smem();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  // barrier of the main threads and the MMA warp; `any`: also whether one of them has given up
-  auto step_barrier = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(kUMain + 32) : "memory"); };
-  auto step_any = [&](bool pred) {
-    uint32_t out;
-    asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.or.pred q, 1, %2, p;\nselp.u32 %0, 1, 0, q;\n}"
-                 : "=r"(out) : "r"(static_cast<uint32_t>(pred)), "n"(kUMain + 32) : "memory");
-    return out != 0;
-  };
-  // The loaders need neither the weights nor the moments: the first tile's rows come while both are on their way.
-  const bool loader = role >= kUMain / 32 && role < kUMain / 32 + kULoaders;
-  bool timed_out = false;
-  if (!loader || !rows_ready) wait_for_predecessor();
-  if (!loader) {
-    dependents_may_start();  // (after the wait: launch_ppo_grad)
-    if (tid == 0) {
-      mbar_expect_tx(bar_load, kImgBytes);
-      constexpr uint32_t kChunk = 16384;
-      for (uint32_t o = 0; o < kImgBytes; o += kChunk) bulk_load(smem_u32(sm.img + o), image + o, min(kChunk, kImgBytes - o), bar_load);
-    }
-    timed_out = step_any(!mbar_wait(bar_load, 0));
-    if (timed_out) *reinterpret_cast<volatile int *>(&sm.abort) = 1;
+  // What fetches rows needs neither the weights nor the moments: the first tile's come while both are on their way.
+  const bool loader = warp >= kUMain / 32 && warp < kUMain / 32 + kULoaders;
+  const bool fetches = loader || warp == kUMain / 32 + kULoaders + 1;
+  if (!fetches || !rows_ready) wait_for_predecessor();
+  if (!fetches) dependents_may_start();  // (after the wait: launch_ppo_grad)
+  if (tid == 0) {  // the first layer's weights and the biases, then the rest
+    constexpr uint32_t kChunk = 16384;
+    mbar_expect_tx(bar_load, kImgWh);
+    for (uint32_t o = 0; o < kImgWh; o += kChunk) bulk_load(smem_u32(sm.img + o), image + o, min(kChunk, kImgWh - o), bar_load);
+    mbar_expect_tx(bar_load + 8, kImgBytes - kImgWh);
+    for (uint32_t o = kImgWh; o < kImgBytes; o += kChunk) bulk_load(smem_u32(sm.img + o), image + o, min(kChunk, kImgBytes - o), bar_load + 8);
   }
 
   const uint32_t tmem = sm.tmem_base;
-  const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
-  const uint32_t w1 = smem_u32(sm.img + kImgW1), w2 = smem_u32(sm.img + kImgW2), wh = smem_u32(sm.img + kImgWh);
-  const uint32_t h1t = smem_u32(sm.h1), h2t = smem_u32(sm.h2), dz2t = smem_u32(sm.dz2), dz1t = h2t,
-                 dht = smem_u32(sm.dhead);
-  const uint32_t b1 = smem_u32(sm.img + kImgB1), b2 = smem_u32(sm.img + kImgB2);
-  const float *bh = reinterpret_cast<const float *>(sm.img + kImgBh);
-  const float mean = loader ? 0.0f : static_cast<float>(__ldcg(adv_stats));
-  const float inv_std = loader ? 0.0f : 1.0f / (static_cast<float>(__ldcg(adv_stats + 1)) + 1e-8f);
-  const float inv_n = 1.0f / static_cast<float>(rows.n);
+  const uint32_t lane_off = static_cast<uint32_t>(wq * 32) << 16;
+  const uint32_t h1t = smem_u32(sm.h1[0]), h2t = smem_u32(sm.h2[0]), xt0 = smem_u32(sm.x[0]), dht = smem_u32(sm.dhead);
   const long long n_tiles = (rows.n + kUR - 1) / kUR;
   const int my_tiles = blockIdx.x < n_tiles ? static_cast<int>((n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
   auto tile_of = [&](int i) { return static_cast<long long>(blockIdx.x) + static_cast<long long>(i) * gridDim.x; };
+  volatile int *abort_flag = &sm.abort;
+  bool ok = true;
 
-  uint32_t ph_mma = 0;
-  double t_actor = 0.0, t_ent = 0.0, t_value = 0.0;
-  float gbh[kActions + 1];  // gradient of the heads' biases, this thread's rows
+  if (loader) {
+    // ---- the rows.  A tile's rows are in registers (as bf16) before its x tile is free, which is late: d W1 of the tile two before, the
+    // last of its products, reads it.  A lane has two neighbouring columns (one 4-byte store) below 64, and two of the sixteen
+    // above of every fourth row; the second load of a pair finds its sectors in L1.
+    const int lw = warp - kUMain / 32, sub = lane >> 3, c2 = 64 + 2 * (lane & 7);
+    const bool has0 = c2 < D, has1 = c2 + 1 < D;
+    auto row_of = [&](int i) {
+      const long long q = tile_of(i) * kUR + kLoadRows * lw + lane;
+      return row_lookup<U>(rows, q, lane < kLoadRows && i < my_tiles && q < rows.n);
+    };
+    RowLookup next = row_of(0);
+    for (int i = 0; i < my_tiles && ok; ++i) {
+      const int src = row_found(rows, next);
+      next = row_of(i + 1);
+      float v[kLoadRows][2], t[kLoadRows / 4][2];
 #pragma unroll
-  for (int k = 0; k <= kActions; ++k) gbh[k] = 0.0f;
-
-  // d W1 [out][in] += d z1^T . x and d b1 [out] += d z1^T . ones (K = rows) of a tile, one lane
-  auto weight_grad_1 = [&](uint32_t xt, uint32_t keep) {
-#pragma unroll
-    for (int k = 0; k < kUR / 16; ++k)
-      mma_bf16(tmem + kColDW1, desc_mn(dz1t, kUH, k), smem_desc(xt + k * 2 * (kUK1 / 8) * kALbo, (kUK1 / 8) * kALbo, kALbo),
-               instr_desc(kUH, kUK1) | kAmn | kBmn, keep | (k > 0));
-#pragma unroll
-    for (int k = 0; k < kUR / 16; ++k)
-      mma_bf16(tmem + kColDB1, desc_mn(dz1t, kUH, k), desc_mn(dht, kUHeads, k), instr_desc(kUH, kUHeads) | kAmn | kBmn, keep | (k > 0));
-    mma_commit(bar_end);
-  };
-  // hidden-layer epilogue: this thread's 64 accumulator columns + bias -> ReLU -> bf16 -> its row of `dst`; one gate bit per
-  // unit out (pair i of 32 columns: bits 15 - i and 31 - i of gate[columns / 32]).  Two columns per instruction throughout
-  // (column by column, with the gate bits shifted in one by one, an epilogue took 1.5 k cycles).
-  auto fwd_epilogue = [&](uint32_t bias, uint32_t dst, uint32_t *gate) {
-    uint32_t r[64];
-    tmem_ld32_nowait(tmem + kColAcc + lane_off + 64u * half, r);
-    tmem_ld32_nowait(tmem + kColAcc + lane_off + 64u * half + 32u, r + 32);
-    tmem_ld_wait();
-    const uint32_t drow = dst + static_cast<uint32_t>((row >> 3) * (kUH * 16) + (row & 7) * 16 + half * 8 * 128);
-    gate[0] = gate[1] = 0;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const float4 ba = lds_float4(bias + 256u * half + 32u * q), bb = lds_float4(bias + 256u * half + 32u * q + 16u);
-      add2(r[8 * q], r[8 * q + 1], ba.x, ba.y); add2(r[8 * q + 2], r[8 * q + 3], ba.z, ba.w);
-      add2(r[8 * q + 4], r[8 * q + 5], bb.x, bb.y); add2(r[8 * q + 6], r[8 * q + 7], bb.z, bb.w);
-      uint32_t pk[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        pk[e] = relu_pack_bf16(r[8 * q + 2 * e], r[8 * q + 2 * e + 1]);
-        gate[q / 4] |= positive_mask(pk[e]) & (0x80008000u >> (4 * (q & 3) + e));
-      }
-      sts_v4(drow + static_cast<uint32_t>(q * 128), pk[0], pk[1], pk[2], pk[3]);
-    }
-  };
-  // backward epilogue: d h (accumulator) gated by the layer's ReLU -> bf16 -> this thread's row of `dst`
-  auto bwd_epilogue = [&](const uint32_t *gate, uint32_t dst) {
-    uint32_t r[64];
-    tmem_ld32_nowait(tmem + kColAcc + lane_off + 64u * half, r);
-    tmem_ld32_nowait(tmem + kColAcc + lane_off + 64u * half + 32u, r + 32);
-    tmem_ld_wait();
-    const uint32_t drow = dst + static_cast<uint32_t>((row >> 3) * (kUH * 16) + (row & 7) * 16 + half * 8 * 128);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      uint32_t pk[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        pk[e] = pack_bf16(__uint_as_float(r[8 * q + 2 * e]), __uint_as_float(r[8 * q + 2 * e + 1])) & sign_mask(gate[q / 4] << (4 * (q & 3) + e));
-      sts_v4(drow + static_cast<uint32_t>(q * 128), pk[0], pk[1], pk[2], pk[3]);
-    }
-  };
-
-  if (timed_out) {
-    // nothing was started
-  } else if (loader) {
-    // ---- the rows: sixteen at a time, the warps in turn, consecutive lanes consecutive features; a
-    // tile ahead of the products (with the conversion on the main threads' chain a tile of 11 k cycles took 17 k)
-    const int lw = role - kUMain / 32;
-    const bool third = lane + 64 < D;
-    for (int i = 0; i < my_tiles && !timed_out; ++i) {
-      __syncwarp();
-#pragma unroll
-      for (int e = lane; e < 64; e += 32) {  // where this warp's rows lie (both look-ups in flight, before the wait)
-        const int c = lw + kULoaders * (e / 16);
-        const long long q = tile_of(i) * kUR + 16 * c + (e & 15);
-        if (c < kUR / 16) sm.rmap[16 * c + (e & 15)] = static_cast<int>(q < rows.n ? real_row<U>(rows, q) : -1);
-      }
-      __syncwarp();
-      if (i >= 2) timed_out = !mbar_wait_warp(bar_end, static_cast<uint32_t>(i) & 1u);  // d W1 of tile i - 2 has read this x tile
-      if (timed_out || *reinterpret_cast<volatile int *>(&sm.abort)) break;
-#pragma unroll 1
-      for (int c = lw; c < kUR / 16; c += kULoaders) {
-        const uint32_t rmap = smem_u32(&sm.rmap[16 * c]);
-        const uint32_t my_col = smem_u32(sm.x[i & 1]) + a_offset<kUK1>(16 * c, lane);
-        float v[16][3];
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-          const int src = lds_s32(rmap + 4u * static_cast<uint32_t>(r));
-          const float *p = rows.x + static_cast<long long>(src) * D + lane;
-          v[r][0] = ldg_if(p, src >= 0);  // (D > 64: the first two are columns of every row)
-          v[r][1] = ldg_if(p + 32, src >= 0);
-          v[r][2] = ldg_if(p + 64, src >= 0 && third);
+      for (int r = 0; r < kLoadRows; ++r) {
+        const int s = __shfl_sync(0xFFFFFFFFu, src, r);
+        const float *p = rows.x + static_cast<long long>(s) * D + 2 * lane;
+        v[r][0] = ldg_if_cached(p, s >= 0);  // (D > 64: these are columns of every row)
+        v[r][1] = ldg_if_cached(p + 1, s >= 0);
+        if ((r & 3) == 0) {
+          const int s4 = __shfl_sync(0xFFFFFFFFu, src, r + sub);
+          const float *p4 = rows.x + static_cast<long long>(s4) * D + c2;
+          t[r / 4][0] = ldg_if_cached(p4, s4 >= 0 && has0);
+          t[r / 4][1] = ldg_if_cached(p4 + 1, s4 >= 0 && has1);
         }
+      }
+      const int ahead = row_found(rows, next);
+      if (ahead >= 0) {  // into L2 (D > 64: the row's first, middle and last lines)
+        const float *p = rows.x + static_cast<long long>(ahead) * D;
+        prefetch_l2(p); prefetch_l2(p + 32); prefetch_l2(p + 64); prefetch_l2(p + D - 1);
+      }
+      uint32_t pk[kLoadRows], pt[kLoadRows / 4];
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {  // (a chunk of eight features is 144 bytes on: 32 features are 576)
-          const uint32_t at = my_col + static_cast<uint32_t>(r >> 3) * ((kUK1 / 8) * kALbo) + (r & 7) * 16;
-          sts_u16(at, bf16_bits(v[r][0]));
-          sts_u16(at + 576u, bf16_bits(v[r][1]));
-          if (third) sts_u16(at + 1152u, bf16_bits(v[r][2]));
-        }
+      for (int r = 0; r < kLoadRows; ++r) pk[r] = pack_bf16(v[r][0], v[r][1]);
+#pragma unroll
+      for (int r = 0; r < kLoadRows / 4; ++r) pt[r] = pack_bf16(t[r][0], t[r][1]);
+      if (i >= 2) ok = ok && mbar_sleep_warp(x_empty0 + 8u * (i & 1), static_cast<uint32_t>((i >> 1) - 1) & 1u);
+      if (!ok || *abort_flag) break;
+      const uint32_t xt = xt0 + kXTile * static_cast<uint32_t>(i & 1) + 16u * static_cast<uint32_t>(kLoadRows * lw);
+      const uint32_t at = xt + static_cast<uint32_t>(lane >> 2) * kXChunk + (lane & 3) * 4;
+      const uint32_t at4 = xt + static_cast<uint32_t>(8 + ((lane & 7) >> 2)) * kXChunk + (lane & 3) * 4 + 16u * static_cast<uint32_t>(sub);
+#pragma unroll
+      for (int r = 0; r < kLoadRows; ++r) {
+        sts_u32(at + 16u * r, pk[r]);
+        if ((r & 3) == 0) sts_u32(at4 + 16u * r, pt[r / 4]);  // (columns from D on: zeros)
       }
       fence_async_smem();
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(x_full0 + 8u * (i & 1)) : "memory");
+      warp_arrive(x_full0 + 8u * (i & 1), lane);
     }
-  } else if (role == kUMain / 32 + kULoaders) {
-    // ---- the MMAs, in the order of the chain; the products that only the weight gradients need follow the one that the chain
-    // waits for.  tcgen05.commit covers everything issued before it, so a main thread that has waited for a later product
-    // knows that the earlier ones have read their tiles.
-    for (int i = 0; i < my_tiles && !timed_out; ++i) {
-      const uint32_t xt = smem_u32(sm.x[i & 1]);
-      const uint32_t keep = i > 0 ? 1u : 0u;  // the weight-gradient accumulators start at the CTA's first tile
-      timed_out = !mbar_wait_warp(x_full0 + 8u * (i & 1), static_cast<uint32_t>(i >> 1) & 1u);
+  } else if (warp >= kUMain / 32 + kULoaders) {
+    if (warp == kUMain / 32 + kULoaders) {
+    // ---- the MMAs: tile s goes forward while tile s - 1 goes backward.  The products that only a weight gradient needs are behind
+    // those that a chain waits for.  tcgen05.commit covers everything issued before it, so who has waited for a later product
+    // knows that the earlier ones have read their tiles.  The order of the products is fixed, so that of every sum is.
+    auto handed_over = [&](int what, int tile) {
+      ok = ok && mbar_sleep_warp(ready0 + 8u * what, static_cast<uint32_t>(tile) & 1u);
       tc_fence_after();
-      if (elect_one()) {  // z1
+    };
+    constexpr uint32_t kFwd = instr_desc(kUR, kUH), kHead = instr_desc(kUR, kUHeads), kGrad = kAmn | kBmn;
+    // operands of step k (16 features or rows), `at` = the tile's address in 16-byte units
+    auto act_k = [](uint32_t at, int k) { return desc16<128, kUH * 16>(at + k * 16); };              // activations, feature as K
+    auto act_mn = [](uint32_t at, int k) { return desc16<kUH * 16, 128>(at + k * 2 * kUH); };        // row as K
+    auto dh_mn = [](uint32_t at, int k) { return desc16<128, 0>(at + k * 16); };                     // dhead, row as K, its columns twice
+    constexpr uint32_t kX16 = kXTile / 16, kH16 = kHTile / 16;
+    const uint32_t block16 = smem_u32(&sm) >> 4;
+    uint32_t base = block16;
+    // not a loop invariant to the compiler: it would keep every product's descriptors in registers that it does not have
+    auto fresh = [&]() { asm volatile("mov.u32 %0, %1;" : "=r"(base) : "r"(block16)); };
+#define AT16(member) (base + static_cast<uint32_t>(offsetof(UtcSmem, member) / 16))
+#define IMG16(off) (base + static_cast<uint32_t>((offsetof(UtcSmem, img) + (off)) / 16))
+    ok = mbar_sleep_warp(bar_load, 0);
+#pragma unroll 1
+    for (int s = 0; s <= my_tiles && ok; ++s) {
+      const bool fwd = s < my_tiles, bwd = s > 0;
+      const int pf = s & 1, pb = pf ^ 1;
+      const uint32_t accf = tmem + kColAcc + 128u * pf, accb = tmem + kColAcc + 128u * pb;
+      const uint32_t hf = kH16 * pf, hb = kH16 * pb, xf = kX16 * pf, xb = kX16 * pb;
+      const uint32_t keep = s > 1 ? 1u : 0u;  // the weight-gradient accumulators start at the CTA's first tile
+      if (bwd) {
+        handed_over(kLoss, s - 1);
+        fresh();
+        if (ok && elect_one()) {
+          // d h2 = dhead . Wh: K = 16 is the eight columns of either operand twice (step 0 from one to the other half), so dhead
+          // is kept at half its size
+          mma_bf16(accb, desc16<0, 128>(AT16(dhead)), desc16<0, 128>(IMG16(kImgWh)), kFwd | kBmn, 0);
+          mma_commit(done0 + 8 * kDh2);
+          // d Wh^T [unit][head column] += h2^T . dhead (K = rows)
 #pragma unroll
-        for (int k = 0; k < kUK1 / 16; ++k)
-          mma_bf16(tmem + kColAcc, smem_desc(xt + k * 2 * kALbo, kALbo, (kUK1 / 8) * kALbo), desc_k(w1, kUK1, k), instr_desc(kUR, kUH), k > 0);
-        mma_commit(bar_mma);
-        if (i > 0) weight_grad_1(smem_u32(sm.x[(i - 1) & 1]), i > 1 ? 1u : 0u);
+          for (int k = 0; k < kUR / 16; ++k)
+            mma_bf16(tmem + kColDWh, act_mn(AT16(h2) + hb, k), dh_mn(AT16(dhead), k), instr_desc(kUH, kUHeads) | kGrad, keep | (k > 0));
+          mma_commit(done0 + 8 * kDWh);  // (d z2 takes h2's place)
+        }
+        __syncwarp();
       }
-      __syncwarp();
-      step_barrier();
-      tc_fence_after();
-      if (elect_one()) {  // z2
+      if (fwd) {
+        ok = ok && mbar_sleep_warp(x_full0 + 8u * pf, static_cast<uint32_t>(s >> 1) & 1u);
+        tc_fence_after();
+        fresh();
+        if (ok && elect_one()) {  // z1
 #pragma unroll
-        for (int k = 0; k < kUH / 16; ++k) mma_bf16(tmem + kColAcc, desc_k(h1t, kUH, k), desc_k(w2, kUH, k), instr_desc(kUR, kUH), k > 0);
-        mma_commit(bar_mma);
+          for (int k = 0; k < kUK1 / 16; ++k)
+            mma_bf16(accf, desc16<kXChunk, 128>(AT16(x) + xf + k * (2 * kXChunk / 16)), desc16<128, kUK1 * 16>(IMG16(kImgW1) + k * 16), kFwd, k > 0);
+          mma_commit(done0 + 8 * kZ1);
+        }
+        __syncwarp();
+        if (s == 0) ok = ok && mbar_sleep_warp(bar_load + 8, 0);
       }
-      __syncwarp();
-      step_barrier();
-      tc_fence_after();
-      if (elect_one()) {  // heads
+      if (bwd) {
+        handed_over(kDz2, s - 1);
+        fresh();
+        if (ok && elect_one()) {
+          // d h1 = d z2 . W2 (K = the out units of layer 2)
 #pragma unroll
-        for (int k = 0; k < kUH / 16; ++k) mma_bf16(tmem + kColHead, desc_k(h2t, kUH, k), desc_k(wh, kUH, k), instr_desc(kUR, kUHeads), k > 0);
-        mma_commit(bar_mma);
+          for (int k = 0; k < kUH / 16; ++k) mma_bf16(accb, act_k(AT16(h2) + hb, k), act_mn(IMG16(kImgW2), k), kFwd | kBmn, k > 0);
+          mma_commit(done0 + 8 * kDh1);
+          // d W2 [out][in] += d z2^T . h1 (K = rows)
+#pragma unroll
+          for (int k = 0; k < kUR / 16; ++k)
+            mma_bf16(tmem + kColDW2, act_mn(AT16(h2) + hb, k), act_mn(AT16(h1) + hb, k), kFwd | kGrad, keep | (k > 0));
+          mma_commit(done0 + 8 * kDW2);  // (d z1 takes h1's place)
+        }
+        __syncwarp();
       }
-      __syncwarp();
-      step_barrier();
-      tc_fence_after();
-      if (elect_one()) {
-        // d h2 = dhead . Wh (K = the 16 head columns)
-        mma_bf16(tmem + kColAcc, desc_k(dht, kUHeads, 0), desc_mn(wh, kUH, 0), instr_desc(kUR, kUH) | kBmn, 0);
-        mma_commit(bar_mma);
-        // d Wh^T [unit][head column] += h2^T . dhead (K = rows)
+      if (fwd) {
+        handed_over(kH1, s);
+        fresh();
+        if (ok && elect_one()) {  // z2
 #pragma unroll
-        for (int k = 0; k < kUR / 16; ++k)
-          mma_bf16(tmem + kColDWh, desc_mn(h2t, kUH, k), desc_mn(dht, kUHeads, k), instr_desc(kUH, kUHeads) | kAmn | kBmn, keep | (k > 0));
+          for (int k = 0; k < kUH / 16; ++k) mma_bf16(accf, act_k(AT16(h1) + hf, k), act_k(IMG16(kImgW2), k), kFwd, k > 0);
+          mma_commit(done0 + 8 * kZ2);
+        }
+        __syncwarp();
       }
-      __syncwarp();
-      step_barrier();
-      tc_fence_after();
-      if (elect_one()) {
-        // d h1 = d z2 . W2 (K = the out units of layer 2)
+      if (bwd) {
+        fresh();
+        if (ok && elect_one()) {  // d b2 [out] += d z2^T . ones (column 7 of dhead, of whichever tile)
 #pragma unroll
-        for (int k = 0; k < kUH / 16; ++k) mma_bf16(tmem + kColAcc, desc_k(dz2t, kUH, k), desc_mn(w2, kUH, k), instr_desc(kUR, kUH) | kBmn, k > 0);
-        mma_commit(bar_mma);
-        // d W2 [out][in] += d z2^T . h1 and d b2 [out] += d z2^T . ones (K = rows)
+          for (int k = 0; k < kUR / 16; ++k)
+            mma_bf16(tmem + kColDB2, act_mn(AT16(h2) + hb, k), dh_mn(AT16(dhead), k), instr_desc(kUH, kUHeads) | kGrad, keep | (k > 0));
+        }
+        __syncwarp();
+        handed_over(kDz1, s - 1);
+        fresh();
+        if (ok && elect_one()) {  // d W1 [out][in] += d z1^T . x
 #pragma unroll
-        for (int k = 0; k < kUR / 16; ++k)
-          mma_bf16(tmem + kColDW2, desc_mn(dz2t, kUH, k), desc_mn(h1t, kUH, k), instr_desc(kUH, kUH) | kAmn | kBmn, keep | (k > 0));
-#pragma unroll
-        for (int k = 0; k < kUR / 16; ++k)
-          mma_bf16(tmem + kColDB2, desc_mn(dz2t, kUH, k), desc_mn(dht, kUHeads, k), instr_desc(kUH, kUHeads) | kAmn | kBmn, keep | (k > 0));
+          for (int k = 0; k < kUR / 16; ++k)
+            mma_bf16(tmem + kColDW1, act_mn(AT16(h1) + hb, k), desc16<128, kXChunk>(AT16(x) + xb + k * 16), instr_desc(kUH, kUK1) | kGrad, keep | (k > 0));
+          mma_commit(x_empty0 + 8u * pb);
+        }
+        __syncwarp();
       }
-      __syncwarp();
-      if (step_any(timed_out)) timed_out = true;
+      if (fwd) {
+        handed_over(kH2, s);
+        fresh();
+        if (ok && elect_one()) {  // heads
+#pragma unroll
+          for (int k = 0; k < kUH / 16; ++k) mma_bf16(accf, act_k(AT16(h2) + hf, k), act_k(IMG16(kImgWh), k), kHead, k > 0);
+          mma_commit(done0 + 8 * kLogits);
+        }
+        __syncwarp();
+      }
+      if (bwd) {
+        fresh();
+        if (ok && elect_one()) {  // d b1 [out] += d z1^T . ones
+#pragma unroll
+          for (int k = 0; k < kUR / 16; ++k)
+            mma_bf16(tmem + kColDB1, act_mn(AT16(h1) + hb, k), dh_mn(AT16(dhead), k), instr_desc(kUH, kUHeads) | kGrad, keep | (k > 0));
+        }
+        __syncwarp();
+      }
     }
-    if (!timed_out && my_tiles > 0) {
-      tc_fence_after();
-      if (elect_one()) weight_grad_1(smem_u32(sm.x[(my_tiles - 1) & 1]), my_tiles > 1 ? 1u : 0u);
-      __syncwarp();
+#undef AT16
+#undef IMG16
+    if (elect_one()) mma_commit(bar_end);  // covers every MMA issued, after a time-out too
+    __syncwarp();
+    } else if (warp == kUMain / 32 + kULoaders + 1) {
+      // ---- what the loss needs of the rows, four rows per lane.  The place for it is free once the loss of the tile before, or the first
+      // tile's first epilogue (it has the biases), is done.
+      float *logp_old = reinterpret_cast<float *>(sm.img + kImgB1), *adv = reinterpret_cast<float *>(sm.img + kImgB2);
+      auto row_of = [&](int i, int k) {
+        const long long q = tile_of(i) * kUR + 32 * k + lane;
+        return row_lookup<U>(rows, q, i < my_tiles && q < rows.n);
+      };
+      RowLookup next[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) next[k] = row_of(0, k);
+#pragma unroll 1
+      for (int i = 0; i < my_tiles && ok; ++i) {
+        float v[4][5];
+        bool real[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int src = row_found(rows, next[k]);
+          real[k] = src >= 0;
+          v[k][0] = ldg_if(rows.logp_old + src, real[k]); v[k][1] = ldg_if(rows.adv + src, real[k]);
+          v[k][2] = ldg_if(rows.value_old + static_cast<long long>(src) * rows.vstride, real[k]);
+          v[k][3] = ldg_if(rows.ret + static_cast<long long>(src) * rows.vstride, real[k]);
+          v[k][4] = ldg_if(reinterpret_cast<const float *>(rows.actions) + src, real[k]);
+          if (!real[k] && tile_of(i) * kUR + 32 * k + lane < rows.n) atomicExch(status, kStatusBadIndex);
+          next[k] = row_of(i + 1, k);
+        }
+        ok = i == 0 ? mbar_sleep_warp(ready0 + 8 * kH1, 0) : mbar_sleep_warp(ready0 + 8 * kLoss, static_cast<uint32_t>(i - 1) & 1u);
+        if (!ok) break;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int r = 32 * k + lane, a = __float_as_int(v[k][4]);
+          logp_old[r] = v[k][0]; adv[r] = v[k][1]; sm.value_old[r] = v[k][2]; sm.ret[r] = v[k][3];
+          sm.action[r] = static_cast<unsigned char>(real[k] ? (a >= 0 && a < kActions ? a : 0xFE) : 0xFF);
+        }
+        warp_arrive(rows_full, lane);
+      }
     }
   } else {
-  for (int i = 0; i < my_tiles && !timed_out; ++i) {
-    const long long row0 = tile_of(i) * kUR;
-    const int n_valid = static_cast<int>(min(static_cast<long long>(kUR), rows.n - row0));
-    const long long my_row = row < n_valid ? real_row<U>(rows, row0 + row) : -1;
-    int action = 0;
-    float logp_old = 0.0f, adv = 0.0f, v_old = 0.0f, ret = 0.0f;
-    if (half == 0) {
-      if (row < n_valid && my_row < 0) atomicExch(status, kStatusBadIndex);
-      if (my_row >= 0) {  // used after the heads: the loads are in flight meanwhile
-        action = rows.actions[my_row]; logp_old = rows.logp_old[my_row]; adv = rows.adv[my_row];
-        v_old = rows.value_old[my_row * rows.vstride]; ret = rows.ret[my_row * rows.vstride];
+    // ---- the epilogues, every warp its part of either tile's: while the products of one are under way, the other's turn
+    const uint32_t acc0 = tmem + kColAcc + lane_off;
+    // where stmatrix4 puts the matrices (row group, chunk), (+1, chunk), (row group, +1), (+1, +1) of this warp's rows and columns
+    const uint32_t my_at = static_cast<uint32_t>((wq * 4 + ((lane >> 3) & 1)) * (kUH * 16) + (cq * 4 + (lane >> 4)) * 128 + (lane & 7) * 16);
+    const float mean = static_cast<float>(__ldcg(adv_stats));
+    const float inv_std = 1.0f / (static_cast<float>(__ldcg(adv_stats + 1)) + 1e-8f);
+    const float inv_n = 1.0f / static_cast<float>(rows.n);
+    const bool is_actor = cq == 0, is_value = cq == 1;  // this warp's part of the loss
+    double t0 = 0.0, t1 = 0.0;  // surrogate and entropy, or value
+    float gbh[kActions];        // gradient of the heads' biases, this thread's rows (value: [0])
+#pragma unroll
+    for (int k = 0; k < kActions; ++k) gbh[k] = 0.0f;
+    auto product = [&](int what, int tile) { ok = ok && mbar_sleep_warp(done0 + 8u * what, static_cast<uint32_t>(tile) & 1u); tc_fence_after(); };
+    auto hand_over = [&](int what) { fence_async_smem(); tc_fence_before(); warp_arrive(ready0 + 8u * what, lane); };
+    // this warp's 32 x 32 accumulators of tile parity p
+    auto load_acc = [&](int p, uint32_t (&r)[32]) {
+      const uint32_t at = acc0 + 128u * p + 32u * cq;
+      tmem_ld_16x32_nowait(at, r);
+      tmem_ld_16x32_nowait(at + (16u << 16), r + 16);
+      tmem_ld_wait32(r);
+    };
+    auto store = [&](uint32_t tile, const uint32_t *pk) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int j = 0; j < 4; j += 2)
+          stmatrix4(tile + my_at + static_cast<uint32_t>(c * 2 * kUH * 16 + j * 128), pk[8 * c + 2 * j], pk[8 * c + 2 * j + 1], pk[8 * c + 2 * j + 2], pk[8 * c + 2 * j + 3]);
+    };
+    // hidden-layer epilogue: + bias -> ReLU -> bf16 -> `tile`; one gate bit per unit out (pair i: bits 15 - i and 31 - i).  Two
+    // columns per instruction throughout.
+    auto fwd_epilogue = [&](int p, const float2 *bias, uint32_t tile) {
+      uint32_t r[32], pk[16], gate[2] = {0, 0};
+      load_acc(p, r);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const float2 b = bias[(i & 7) >> 1];
+        add2(r[2 * i], r[2 * i + 1], b.x, b.y);
+        pk[i] = relu_pack_bf16(r[2 * i], r[2 * i + 1]);
+        gate[i & 1] |= positive_mask(pk[i]) & (0x80008000u >> i);
+      }
+      store(tile, pk);
+      return gate[0] | gate[1];
+    };
+    // backward epilogue: d h (accumulator) gated by the layer's ReLU, as bf16 pairs
+    auto bwd_epilogue = [&](int p, uint32_t gate, uint32_t *pk) {
+      uint32_t r[32];
+      load_acc(p, r);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])) & sign_mask(gate << i);
+    };
+    ok = mbar_sleep_warp(bar_load, 0);
+    float2 b1[4], b2[4];
+    {
+      const float *src = reinterpret_cast<const float *>(sm.img) + 32 * cq + 2 * (lane & 3);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        b1[j] = *reinterpret_cast<const float2 *>(src + kImgB1 / 4 + 8 * j);
+        b2[j] = *reinterpret_cast<const float2 *>(src + kImgB2 / 4 + 8 * j);
       }
     }
-    timed_out |= !mbar_wait(bar_mma, ph_mma); ph_mma ^= 1;
-    tc_fence_after();
-    uint32_t gate1[2], gate2[2];
-    fwd_epilogue(b1, h1t, gate1);
-    fence_async_smem(); tc_fence_before();
-    step_barrier();
-    timed_out |= !mbar_wait(bar_mma, ph_mma); ph_mma ^= 1;
-    tc_fence_after();
-    fwd_epilogue(b2, h2t, gate2);
-    fence_async_smem(); tc_fence_before();
-    step_barrier();
-    timed_out |= !mbar_wait(bar_mma, ph_mma); ph_mma ^= 1;
-    tc_fence_after();
-    // ---- loss terms and the per-row derivatives with respect to the six logits and the value (thread = row)
-    if (half == 0) {
-      float hv[16], d[8];
-      tmem_ld16(tmem + kColHead + lane_off, hv);
+    const float *bh = reinterpret_cast<const float *>(sm.img + kImgBh);
+    uint32_t gate1 = 0, gate2 = 0;
+#pragma unroll 1
+    for (int s = 0; s <= my_tiles && ok; ++s) {
+      const bool fwd = s < my_tiles, bwd = s > 0;
+      const int pf = s & 1, pb = pf ^ 1;
+      if (bwd) {  // d z2
+        uint32_t pk[16];
+        product(kDh2, s - 1);
+        bwd_epilogue(pb, gate2, pk);
+        product(kDWh, s - 1);
+        store(h2t + kHTile * pb, pk);
+        hand_over(kDz2);
+      }
+      const uint32_t gate1_b = gate1;
+      if (fwd) {
+        product(kZ1, s);
+        gate1 = fwd_epilogue(pf, b1, h1t + kHTile * pf);
+        hand_over(kH1);
+      }
+      if (bwd) {  // d z1
+        uint32_t pk[16];
+        product(kDh1, s - 1);
+        bwd_epilogue(pb, gate1_b, pk);
+        product(kDW2, s - 1);
+        store(h1t + kHTile * pb, pk);
+        hand_over(kDz1);
+      }
+      if (fwd) {
+        product(kZ2, s);
+        gate2 = fwd_epilogue(pf, b2, h2t + kHTile * pf);
+        hand_over(kH2);
+      }
+      if (fwd && (is_actor || is_value)) ok = ok && mbar_sleep_warp(rows_full, static_cast<uint32_t>(s) & 1u);
+      const int row = 32 * wq + lane, action = sm.action[row];
+      const bool real = action != 0xFF;
+      // loss terms and the per-row derivatives with respect to the six logits and the value.  dhead: columns 0..6 the derivatives at
+      // half their size; column 7: one (it turns the d z^T products into column sums)
+      if (fwd && is_actor) {
+        product(kLogits, s);
+        const float in0 = reinterpret_cast<const float *>(sm.img + kImgB1)[row], in1 = reinterpret_cast<const float *>(sm.img + kImgB2)[row];
+        float l[8], p[kActions], d[kActions], m = -INFINITY, sum = 0.0f;
+        tmem_ld_row8(acc0 + 128u * pf, l);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) d[k] = 0.0f;
-      if (my_row >= 0) {
-        float l[kActions], m = -INFINITY, sum = 0.0f;
-#pragma unroll
-        for (int k = 0; k < kActions; ++k) { l[k] = hv[k] + bh[k]; m = fmaxf(m, l[k]); }
+        for (int k = 0; k < kActions; ++k) { l[k] += bh[k]; m = fmaxf(m, l[k]); }
 #pragma unroll
         for (int k = 0; k < kActions; ++k) sum += expf(l[k] - m);
         const float lse = m + logf(sum);
-        float ent = 0.0f, p[kActions], lp[kActions], lpa = 0.0f;
+        float ent = 0.0f, lpa = 0.0f;
 #pragma unroll
         for (int k = 0; k < kActions; ++k) {
-          lp[k] = l[k] - lse; p[k] = expf(lp[k]); ent -= p[k] * lp[k];
-          if (k == action) lpa = lp[k];
+          l[k] -= lse; p[k] = expf(l[k]); ent -= p[k] * l[k];
+          if (k == action) lpa = l[k];
         }
-        const float rho = expf(lpa - logp_old);
-        const float ahat = (adv - mean) * inv_std;
+        const float rho = expf(lpa - in0);
+        const float ahat = (in1 - mean) * inv_std;
         const float clipped = fminf(fmaxf(rho, 1.0f - hp.clip_eps), 1.0f + hp.clip_eps);
         const float s1 = rho * ahat, s2 = clipped * ahat;
         const bool inside = rho >= 1.0f - hp.clip_eps && rho <= 1.0f + hp.clip_eps;
         const float d_logp = (inside || s1 < s2) ? -s1 * inv_n : 0.0f;  // the clipped branch is constant in rho
 #pragma unroll
-        for (int k = 0; k < kActions; ++k)
-          d[k] = d_logp * ((k == action ? 1.0f : 0.0f) - p[k]) + hp.ent_coef * inv_n * p[k] * (lp[k] + ent);
-        t_actor += fminf(s1, s2);
-        t_ent += ent;
-        const float v = hv[kActions] + bh[kActions];
-        const float u = v - ret, uc = v_old + fminf(fmaxf(v - v_old, -hp.clip_eps), hp.clip_eps) - ret;
-        const bool in_range = fabsf(v - v_old) <= hp.clip_eps;
-        d[kActions] = (in_range || u * u > uc * uc) ? hp.vf_coef * u * inv_n : 0.0f;
-        t_value += 0.5 * fmaxf(u * u, uc * uc);
+        for (int k = 0; k < kActions; ++k) {
+          d[k] = d_logp * ((k == action ? 1.0f : 0.0f) - p[k]) + hp.ent_coef * inv_n * p[k] * (l[k] + ent);
+          if (!real) d[k] = 0.0f;
+        }
+        const uint32_t at = dht + 16u * static_cast<uint32_t>(row);
+        asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at), "r"(pack_bf16(0.5f * d[0], 0.5f * d[1])), "r"(pack_bf16(0.5f * d[2], 0.5f * d[3])) : "memory");
+        sts_u32(at + 8u, pack_bf16(0.5f * d[4], 0.5f * d[5]));
+        hand_over(kLoss);
+#pragma unroll
+        for (int k = 0; k < kActions; ++k) gbh[k] += d[k];  // (unrounded)
+        if (real) { t0 += fminf(s1, s2); t1 += ent; }
       }
-      // columns 0..6: the derivatives; column 7: one (it turns the d z^T products into column sums)
-      sts_v4(dht + static_cast<uint32_t>((row >> 3) * (kUHeads * 16) + (row & 7) * 16), pack_bf16(d[0], d[1]), pack_bf16(d[2], d[3]),
-             pack_bf16(d[4], d[5]), pack_bf16(d[6], 1.0f));
-#pragma unroll
-      for (int k = 0; k <= kActions; ++k) gbh[k] += d[k];  // the heads' bias gradients sum the unrounded derivatives
+      if (fwd && is_value) {
+        product(kLogits, s);
+        const float in0 = sm.value_old[row], in1 = sm.ret[row];
+        float l[8], d = 0.0f;
+        tmem_ld_row8(acc0 + 128u * pf, l);
+        if (real) {
+          const float v = l[kActions] + bh[kActions], u = v - in1, uc = in0 + fminf(fmaxf(v - in0, -hp.clip_eps), hp.clip_eps) - in1;
+          const bool in_range = fabsf(v - in0) <= hp.clip_eps;
+          d = (in_range || u * u > uc * uc) ? hp.vf_coef * u * inv_n : 0.0f;
+          t0 += 0.5 * fmaxf(u * u, uc * uc);
+        }
+        sts_u32(dht + 16u * static_cast<uint32_t>(row) + 12u, pack_bf16(0.5f * d, 1.0f));
+        hand_over(kLoss);
+        gbh[0] += d;
+      }
     }
-    fence_async_smem(); tc_fence_before();
-    step_barrier();
-    timed_out |= !mbar_wait(bar_mma, ph_mma); ph_mma ^= 1;
-    tc_fence_after();
-    bwd_epilogue(gate2, dz2t);
-    fence_async_smem(); tc_fence_before();
-    step_barrier();
-    timed_out |= !mbar_wait(bar_mma, ph_mma); ph_mma ^= 1;  // d h1 is there, and h2's last reader (d Wh) is done
-    tc_fence_after();
-    bwd_epilogue(gate1, dz1t);
-    fence_async_smem(); tc_fence_before();
-    if (step_any(timed_out)) timed_out = true;
-  }
-  if (timed_out) *reinterpret_cast<volatile int *>(&sm.abort) = 1;
+    if (is_actor || is_value) {
+      UtcSums &sums = *reinterpret_cast<UtcSums *>(sm.img + kImgW2);
 #pragma unroll
-  for (int k = 0; k <= kActions; ++k) {
-    for (int o = 16; o > 0; o >>= 1) gbh[k] += __shfl_xor_sync(0xFFFFFFFFu, gbh[k], o);
-    if (lane == 0 && half == 0) sm.red[warp][k] = gbh[k];
+      for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int k = 0; k < kActions; ++k) gbh[k] += __shfl_xor_sync(0xFFFFFFFFu, gbh[k], o);
+        t0 += __shfl_xor_sync(0xFFFFFFFFu, t0, o); t1 += __shfl_xor_sync(0xFFFFFFFFu, t1, o);
+      }
+      if (lane == 0 && is_actor) {
+#pragma unroll
+        for (int k = 0; k < kActions; ++k) sums.bias[wq][k] = gbh[k];
+        sums.term[wq][0] = t0; sums.term[wq][1] = t1;
+      }
+      if (lane == 0 && is_value) { sums.bias[wq][kActions] = gbh[0]; sums.term[wq][2] = t0; }
+    }
   }
-  }
-  // ---- the CTA's slice: accumulators out of tensor memory, once
-  timed_out = __syncthreads_or(timed_out) != 0;  // (the last products have been issued)
-  if (my_tiles > 0 && !timed_out) timed_out = !mbar_wait(bar_end, static_cast<uint32_t>(my_tiles - 1) & 1u);
-  timed_out = __syncthreads_or(timed_out) != 0;
-  if (!timed_out && my_tiles > 0 && warp < kUMain / 32) {
+  // ---- the CTA's slice: accumulators out of tensor memory, once (what belongs to real units)
+  if (!ok) *abort_flag = 1;
+  ok = __syncthreads_and(ok) != 0;  // (the last products have been issued)
+  ok &= mbar_wait(bar_end, 0);
+  ok = __syncthreads_and(ok) != 0;
+  const UtcSums &sums = *reinterpret_cast<const UtcSums *>(sm.img + kImgW2);
+  if (ok && my_tiles > 0 && warp < kUMain / 32) {
     tc_fence_after();
     float *part = partial + static_cast<size_t>(blockIdx.x) * kSlice;
-    const int unit = (warp & 3) * 32 + lane;  // tensor-memory lane = out unit (d W2, d W1, d b) or hidden unit (d Wh)
-    auto put16 = [&](float *dst, uint32_t col, int n) {  // n columns from accumulator column `col` on
-      float v[16];
-      tmem_ld16(tmem + lane_off + col, v);
+    const int unit = 32 * wq + lane;  // tensor-memory lane = out unit (d W2, d W1, d b) or hidden unit (d Wh)
+    auto put = [&](float *dst, const uint32_t *v, int n, float scale) {  // n columns
+      if (unit < H)
 #pragma unroll
-      for (int c = 0; c < 16; c += 4)
-        if (c < n) *reinterpret_cast<float4 *>(dst + (static_cast<size_t>(c / 4) * kUH + unit) * 4) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+        for (int c = 0; c < n; c += 4)
+          *reinterpret_cast<float4 *>(dst + (static_cast<size_t>(c / 4) * kUH + unit) * 4) =
+              make_float4(scale * __uint_as_float(v[c]), scale * __uint_as_float(v[c + 1]), scale * __uint_as_float(v[c + 2]), scale * __uint_as_float(v[c + 3]));
     };
-    if (half == 0) {
-      for (int c0 = 0; c0 < kUH; c0 += 16) put16(part + kSlW2 + c0 * kUH, kColDW2 + c0, 16);
+    uint32_t v[32];
+    const uint32_t from = tmem + lane_off;
+    if (cq < 3) {  // 32 columns of d W2 (0, 32, 96 ..) and those of d W1 from 0, 32, 64 on
+      if (cq < 2 || H > 96) {
+        const int c0 = cq < 2 ? 32 * cq : 96;
+        if (c0 < H) {
+          tmem_ld32_nowait(from + kColDW2 + c0, v);
+          tmem_ld_wait32(v);
+          put(part + kSlW2 + c0 * kUH, v, 32, 1.0f);
+        }
+      }
+      tmem_ld32_nowait(from + kColDW1 + (cq < 2 ? 32 * cq : 48), v);
+      tmem_ld_wait32(v);
+      if (cq < 2) put(part + kSlW1 + 32 * cq * kUH, v, 32, 1.0f);
+      else put(part + kSlW1 + 64 * kUH, v + 16, 16, 1.0f);
     } else {
-      for (int c0 = 0; c0 < kUK1; c0 += 16) put16(part + kSlW1 + c0 * kUH, kColDW1 + c0, 16);
-      put16(part + kSlWh, kColDWh, 8);
-      float v[16];
-      tmem_ld16(tmem + kColDB2 + lane_off, v);
-      part[kSlB2 + unit] = v[7];
-      tmem_ld16(tmem + kColDB1 + lane_off, v);
-      part[kSlB1 + unit] = v[7];
-    }
-    if (tid <= kActions) part[kSlBh + tid] = (sm.red[0][tid] + sm.red[1][tid]) + (sm.red[2][tid] + sm.red[3][tid]);
-  }
-  if (warp < kUMain / 32) {  // loss-term sums of the warp, lane 0 writes them (warps 4..7 hold zeros)
-    double s[3] = {t_actor, t_ent, t_value};
+      if (64 < H) {
+        tmem_ld32_nowait(from + kColDW2 + 64, v);
+        tmem_ld_wait32(v);
+        put(part + kSlW2 + 64 * kUH, v, 32, 1.0f);
+      }
+      float w[16];
+      tmem_ld16(from + kColDWh, w);
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
-      for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xFFFFFFFFu, s[k], o);
-    if (lane == 0) {
-      double *tp = term_partial + (static_cast<size_t>(blockIdx.x) * 8 + warp) * 3;
-      tp[0] = s[0]; tp[1] = s[1]; tp[2] = s[2];
+      for (int c = 0; c < 8; ++c) v[c] = __float_as_uint(w[c]);
+      put(part + kSlWh, v, 8, 2.0f);  // (dhead at half its size)
+      tmem_ld16(from + kColDB2, w);
+      if (unit < H) part[kSlB2 + unit] = w[7];
+      tmem_ld16(from + kColDB1, w);
+      if (unit < H) part[kSlB1 + unit] = w[7];
     }
+    if (tid <= kActions) part[kSlBh + tid] = (sums.bias[0][tid] + sums.bias[1][tid]) + (sums.bias[2][tid] + sums.bias[3][tid]);
   }
-  if (timed_out && tid == 0) atomicExch(status, kStatusTimeout);
+  if (tid < 12) term_partial[static_cast<size_t>(blockIdx.x) * 12 + tid] = (&sums.term[0][0])[tid];
+  if (!ok && tid == 0) atomicExch(status, kStatusTimeout);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
@@ -522,7 +714,7 @@ cudaError_t launch_ppo_net_tc(mava_rollout *h, const float *params_dev, const Pa
   err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (err != cudaSuccess) return err;
   err = launch_dependent(kern, slices, kUThreads, smem, h->stream, static_cast<const unsigned char *>(image), rows, hp,
-                         static_cast<const double *>(adv.out), partial, term_partial, h->d_status, h->D, adv.early);
+                         static_cast<const double *>(adv.out), partial, term_partial, h->d_status, h->D, h->cfg.hidden, adv.early);
   if (err != cudaSuccess) return err;
   h->launches += 3;
   return launch_dependent(reduce_slices_kernel<SliceMap>, kReduceBlocks, kReduceThreads, 0, h->stream, static_cast<const float *>(partial), kSlice, slices, grad,
