@@ -291,18 +291,11 @@ __global__ void __launch_bounds__(256) moments_kernel(Moments m) {  // of the ad
   moments_block<U>(m);
 }
 
-__global__ void adam_kernel(float *params, const float *grad, float *m, float *v, size_t n, const double *stats, float max_norm, float lr,
-                            float beta1, float beta2, float eps, float corr1, float corr2) {
+__global__ void __launch_bounds__(256) adam_kernel(AdamArgs a, size_t n) {
   dependents_may_start();
   wait_for_predecessor();
-  const float norm = static_cast<float>(__ldcg(stats + 2));
-  const float scale = max_norm / fmaxf(norm, max_norm);
-  for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const float g = __ldcg(grad + i) * scale;
-    const float mi = beta1 * m[i] + (1.0f - beta1) * g, vi = beta2 * v[i] + (1.0f - beta2) * g * g;
-    m[i] = mi; v[i] = vi;
-    params[i] -= lr * (mi / corr1) / (sqrtf(vi / corr2) + eps);
-  }
+  const float scale = adam_scale(a);
+  for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += static_cast<size_t>(gridDim.x) * blockDim.x) adam_element(a, scale, i);
 }
 
 // Scratch of the update block, made on first use: [moments of the advantages and of the gradient, counters][their partials][term partials][transposed
@@ -314,12 +307,15 @@ size_t upd_smem_bytes(int Din, int H) {
 
 // The head of the scratch, the same in every layout of the rest.
 constexpr size_t kHeadBytes = 128 + 3 * sizeof(double) * 2 * kMomentBlocks;
-enum { kAdvMoments = 0, kGradMoments = 1, kAdvMoments2 = 2 };  // (two places for the advantages': see launch_ppo_grad)
+enum { kAdvMoments = 0, kAdvMoments2 = 2 };  // (two places for the advantages': see launch_ppo_grad)
 Moments moments_of(mava_rollout *h, int which, const float *x, long long n, const UpdRows &map, bool early = false) {
   unsigned char *p = static_cast<unsigned char *>(h->d_upd);
   return Moments{x, n, map, reinterpret_cast<double *>(p + 128) + which * 2 * kMomentBlocks, reinterpret_cast<double *>(p) + 4 * which,
                  reinterpret_cast<unsigned *>(p + 96) + which, early};
 }
+// The gradient's sums of squares, between the two places of the moments' partial sums.
+double *grad_squares_of(mava_rollout *h) { return reinterpret_cast<double *>(static_cast<unsigned char *>(h->d_upd) + 128) + 2 * kMomentBlocks; }
+Moments adv_moments_of(mava_rollout *h, int seq, const UpdRows &rows) { return moments_of(h, seq & 1 ? kAdvMoments2 : kAdvMoments, h->buf.adv, rows.n, rows, seq > 0); }
 
 struct UpdScratch {
   double *term_part;
@@ -334,9 +330,9 @@ UpdScratch carve(mava_rollout *h, size_t n_params, int slices) {
   unsigned char *p = static_cast<unsigned char *>(h->d_upd);
   UpdScratch s{};
   p += kHeadBytes;
+  s.image = p; p += image_room();  // (the same place for every number of slices: a step leaves it to the next minibatch)
   s.term_part = reinterpret_cast<double *>(p); p += sizeof(double) * 3 * 8 * slices;
   s.wt = reinterpret_cast<float *>(p); p += sizeof(float) * ((n_params + 3) / 4 * 4);
-  s.image = p; p += image_room();
   s.partial = reinterpret_cast<float *>(p);
   s.slices = slices;
   return s;
@@ -431,12 +427,23 @@ cudaError_t reserve_update(mava_rollout *h, int n_small, int n_large) {
   return ensure_update(h, plan);
 }
 
+// The rows of a minibatch of environments (nullptr: all) of the last run.
+static UpdRows rows_of(const mava_rollout *h, const int32_t *env_ids_dev, int n_env) {
+  UpdRows rows{};
+  rows.x = h->buf.obs; rows.actions = h->buf.actions; rows.logp_old = h->buf.logp; rows.adv = h->buf.adv;
+  rows.n = static_cast<long long>(h->last_T) * n_env * h->cfg.n_agents;
+  rows.env_ids = env_ids_dev; rows.n_ids = n_env; rows.E = h->cfg.n_envs; rows.per_env = h->cfg.n_agents;
+  if (h->cfg.net_kind != MAVA_NET_CENTRAL_CRITIC) { rows.value_old = h->buf.values; rows.ret = h->buf.ret; rows.vstride = 1; }
+  return rows;
+}
+
 // `seq`: how many gradients and optimiser steps, and nothing else, this call's caller has launched directly before.  From the second
 // on the advantages' moments need not wait for the optimiser step: the gradient kernel lets its successors start only after
 // its own wait, so whatever was launched before the gradient in front (seq >= 1) is complete when this one's first kernel
 // starts.  That gradient may still read its moments: every other call has another place for them.
+// `prepared`: launch_adam_step was told of this minibatch (its `next`).
 cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava_ppo_hyper_t &hyper, float *grad_dev,
-                            float *terms_dev, const int32_t *env_ids_dev, int32_t n_ids, int seq) {
+                            float *terms_dev, const int32_t *env_ids_dev, int32_t n_ids, int seq, bool prepared) {
   const mava_config_t &cfg = h->cfg;
   const int T = h->last_T, E = cfg.n_envs, N = cfg.n_agents, D = h->D, H = cfg.hidden;
   const ParamLayout L = param_layout(cfg, D, 1);
@@ -451,16 +458,13 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
   const bool central = cfg.net_kind == MAVA_NET_CENTRAL_CRITIC;
   const UpdHyper hp{hyper.clip_eps, hyper.ent_coef, hyper.vf_coef};
   cudaStream_t st = h->stream;
-  UpdRows rows{};
-  rows.x = h->buf.obs; rows.actions = h->buf.actions; rows.logp_old = h->buf.logp; rows.adv = h->buf.adv; rows.n = R;
-  rows.env_ids = env_ids_dev; rows.n_ids = n_env; rows.E = E; rows.per_env = N;
-  if (!central) { rows.value_old = h->buf.values; rows.ret = h->buf.ret; rows.vstride = 1; }
+  const UpdRows rows = rows_of(h, env_ids_dev, n_env);
 
   if (update_takes_tensor_cores(cfg, D)) {
     const UpdScratch sc = carve(h, ppo_tc_slice_floats(), slices);
     const TermSums terms{sc.term_part, sc.term_part, 4 * slices, 4 * slices, R, R, hp, terms_dev};
-    return launch_ppo_net_tc(h, params_dev, L, rows, hp, moments_of(h, seq & 1 ? kAdvMoments2 : kAdvMoments, h->buf.adv, R, rows, seq > 0), sc.image, sc.partial, sc.term_part, slices,
-                             grad_dev, terms, moments_of(h, kGradMoments, grad_dev, static_cast<long long>(P), UpdRows{}));
+    return launch_ppo_net_tc(h, params_dev, L, rows, hp, adv_moments_of(h, seq, rows), prepared, sc.image, sc.partial, sc.term_part, slices, grad_dev, terms,
+                             grad_squares_of(h));
   }
 
   UpdRows crows{};  // the centralised critic's: a row is an environment-step
@@ -531,30 +535,36 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
   const TermSums terms{sc.term_part, sc.term_part, 8 * slices, 8 * slices, R, central ? S : R, hp, terms_dev};
   h->launches += 1;
   return launch_dependent(reduce_slices_kernel<IdentityMap>, kReduceBlocks, kReduceThreads, 0, st, static_cast<const float *>(sc.partial), static_cast<int>(P), slices,
-                          grad_dev, terms, moments_of(h, kGradMoments, grad_dev, static_cast<long long>(P), UpdRows{}), IdentityMap{});
+                          grad_dev, terms, grad_squares_of(h), IdentityMap{});
 }
 
 cudaError_t launch_adam_step(mava_rollout *h, float *params_dev, const float *grad_dev, float *m_dev, float *v_dev, int32_t step,
-                             const mava_ppo_hyper_t &hp, bool norm_known) {
-  const size_t P = param_layout(h->cfg, h->D, 1).total;
+                             const mava_ppo_hyper_t &hp, bool norm_known, const NextMinibatch *next) {
+  const ParamLayout L = param_layout(h->cfg, h->D, 1);
+  const size_t P = L.total;
+  const bool tc = update_takes_tensor_cores(h->cfg, h->D);
   cudaError_t err = ensure_update_bytes(h, update_scratch_bytes(P, 1));
   if (err != cudaSuccess) return err;
-  const Moments norm = moments_of(h, kGradMoments, grad_dev, static_cast<long long>(P), UpdRows{});
+  double *squares = grad_squares_of(h);
   if (!norm_known) {
-    err = update_takes_tensor_cores(h->cfg, h->D)
-              ? launch_grad_moments_tc(h, param_layout(h->cfg, h->D, 1), norm)
-              : launch_dependent(grad_moments_kernel<IdentityMap>, kMomentBlocks, 256, 0, h->stream, norm, static_cast<int>(P), IdentityMap{});
+    err = tc ? launch_grad_squares_tc(h, L, grad_dev, squares)
+             : launch_dependent(grad_squares_kernel<IdentityMap>, kMomentBlocks, 256, 0, h->stream, grad_dev, squares, static_cast<int>(P), IdentityMap{});
     if (err != cudaSuccess) return err;
     h->launches += 1;
   }
   const float corr1 = static_cast<float>(1.0 - pow(static_cast<double>(hp.beta1), step));
   const float corr2 = static_cast<float>(1.0 - pow(static_cast<double>(hp.beta2), step));
+  const AdamArgs adam{params_dev, grad_dev, m_dev, v_dev, squares, hp.max_grad_norm, hp.lr, hp.beta1, hp.beta2, hp.adam_eps, corr1, corr2};
+  if (next && tc)
+    return launch_step_tc(h, adam, L, adv_moments_of(h, next->seq, rows_of(h, next->env_ids, next->n)), carve(h, ppo_tc_slice_floats(), 1).image);
   h->launches += 1;
-  return launch_dependent(adam_kernel, 2 * 148, 256, 0, h->stream, params_dev, grad_dev, m_dev, v_dev, P, static_cast<const double *>(norm.out),
-                          hp.max_grad_norm, hp.lr, hp.beta1, hp.beta2, hp.adam_eps, corr1, corr2);
+  const int blocks = static_cast<int>((P + 255) / 256 < 2 * 148 ? (P + 255) / 256 : 2 * 148);
+  return launch_dependent(adam_kernel, blocks, 256, 0, h->stream, adam, P);
 }
 
-// Whether a gradient call leaves the gradient's moments behind (update_takes_tensor_cores_256: its reduction does not).
+// Whether a gradient call leaves the gradient's sums of squares behind (update_takes_tensor_cores_256: its reduction does not).
 bool ppo_grad_leaves_norm(const mava_rollout *h) { return !update_takes_tensor_cores_256(h->cfg, h->D); }
+// Whether a step prepares the minibatch that it is told of.
+bool adam_step_prepares(const mava_rollout *h) { return update_takes_tensor_cores(h->cfg, h->D); }
 
 }  // namespace mava

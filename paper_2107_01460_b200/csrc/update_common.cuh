@@ -97,7 +97,7 @@ __device__ __forceinline__ float4 lds_float4(uint32_t addr) {
   return v;
 }
 
-// ---- mean, population std and 2-norm of a vector, by the first kMomentBlocks blocks (256 threads each) of a kernel: block
+// ---- mean and population std of a vector, by the first kMomentBlocks blocks (256 threads each) of a kernel: block
 // partial sums of x and x^2 in double; the block that finishes last adds them.  Fixed orders throughout: the same bytes on
 // every call, and from every kernel that does it.
 constexpr int kMomentBlocks = 256;
@@ -106,7 +106,7 @@ struct Moments {
   long long n;
   UpdRows map;         // which elements (env_ids == nullptr: all n)
   double *part;        // [kMomentBlocks][2]
-  double *out;         // mean, std, 2-norm
+  double *out;         // mean, std
   unsigned *finished;  // zero before and after
   bool early;          // what it reads was complete before the kernel in front of this one was launched (launch_ppo_grad)
 };
@@ -140,7 +140,7 @@ __device__ __forceinline__ void moments_finish(const Moments &m, double a, doubl
   block_sum2(a, b);
   if (t != 0) return;
   const double mean = a / static_cast<double>(m.n), var = fmax(b / static_cast<double>(m.n) - mean * mean, 0.0);
-  m.out[0] = mean; m.out[1] = sqrt(var); m.out[2] = sqrt(b);
+  m.out[0] = mean; m.out[1] = sqrt(var);
 }
 template <class U>
 __device__ __forceinline__ void moments_block(const Moments &m) {
@@ -186,14 +186,17 @@ bool ppo_tc_supported(const mava_config_t &cfg, int D);
 size_t ppo_tc_image_bytes();
 size_t ppo_tc_slice_floats();
 struct TermSums;
-// Enqueues the prologue (moments of the advantages, weight image), the loss/gradient kernel and the reduction of its slices
-// into `grad`, the loss terms and the gradient's moments; `partial` holds `slices` slices of ppo_tc_slice_floats() floats (one
-// per CTA), `term_partial` 4 x 3 doubles per slice.
+struct AdamArgs;
+// Enqueues the prologue (moments of the advantages, weight image; not if launch_step_tc has left both), the loss/gradient kernel and
+// the reduction of its slices into `grad`, the loss terms and the gradient's sums of squares; `partial` holds `slices` slices of
+// ppo_tc_slice_floats() floats (one per CTA), `term_partial` 4 x 3 doubles per slice.
 cudaError_t launch_ppo_net_tc(mava_rollout *h, const float *params_dev, const ParamLayout &L, const UpdRows &rows, const UpdHyper &hp,
-                              const Moments &adv, void *image, float *partial, double *term_partial, int slices, float *grad, const TermSums &terms,
-                              const Moments &norm);
-// The moments that launch_ppo_net_tc leaves, of a gradient that comes from elsewhere: the same order of additions.
-cudaError_t launch_grad_moments_tc(mava_rollout *h, const ParamLayout &L, const Moments &norm);
+                              const Moments &adv, bool prepared, void *image, float *partial, double *term_partial, int slices, float *grad,
+                              const TermSums &terms, double *squares);
+// The sums of squares that launch_ppo_net_tc leaves, of a gradient that comes from elsewhere: the same order of additions.
+cudaError_t launch_grad_squares_tc(mava_rollout *h, const ParamLayout &L, const float *grad, double *squares);
+// An optimiser step with what the next gradient starts with: its weight image and its advantages' moments (`next`, early).
+cudaError_t launch_step_tc(mava_rollout *h, const AdamArgs &adam, const ParamLayout &L, const Moments &next, void *image);
 
 // Where the loss-term sums of a call lie, [n][3] doubles (surrogate, entropy, value) per list: the actor's list gives the
 // first two, the value net's the third (one net with both heads: the same list).
@@ -244,7 +247,34 @@ __device__ __forceinline__ void loss_terms(const TermSums &t) {
   t.out[3] = static_cast<float>(val);
 }
 
-// grad[map(j)] = sum of element j over the CTAs' slices of `len` floats, in a fixed order, and the gradient's moments (its
+// ---- optimiser step.  The gradient's 2-norm comes as kMomentBlocks sums of squares from the kernel in front; every block adds them
+// for itself (when the last block of that kernel did, the step started 4 us later).
+struct AdamArgs {
+  float *params;
+  const float *grad;
+  float *m, *v;
+  const double *squares;  // [kMomentBlocks]
+  float max_norm, lr, beta1, beta2, eps, corr1, corr2;
+};
+// The factor that takes the gradient to max_norm at most (by a whole block of 256 threads, after its wait).
+__device__ __forceinline__ float adam_scale(const AdamArgs &a) {
+  __shared__ float scale;
+  double none = 0.0, b = __ldcg(a.squares + threadIdx.x);
+  block_sum2(none, b);
+  if (threadIdx.x == 0) scale = a.max_norm / fmaxf(static_cast<float>(sqrt(b)), a.max_norm);
+  __syncthreads();
+  return scale;
+}
+__device__ __forceinline__ float adam_element(const AdamArgs &a, float scale, size_t i) {
+  const float g = __ldcg(a.grad + i) * scale;
+  const float mi = a.beta1 * a.m[i] + (1.0f - a.beta1) * g, vi = a.beta2 * a.v[i] + (1.0f - a.beta2) * g * g;
+  a.m[i] = mi; a.v[i] = vi;
+  const float p = a.params[i] - a.lr * (mi / a.corr1) / (sqrtf(vi / a.corr2) + a.eps);
+  a.params[i] = p;
+  return p;
+}
+
+// grad[map(j)] = sum of element j over the CTAs' slices of `len` floats, in a fixed order, and each block's sum of squares (the
 // 2-norm is what an optimiser step needs next); a block of its own turns the term sums into the loss terms.  Four threads per
 // element take a quarter of the slices each, 20 loads in flight; one round for 32 k elements (bound by the latency
 // of its loads; 148 slices of 28 k: 10.7 us from a cold cache; 16.7 with two rounds, batches of 16 and the loss terms added by block 0).
@@ -255,7 +285,7 @@ struct IdentityMap {
 };
 template <class Map>
 __global__ void __launch_bounds__(kReduceThreads) reduce_slices_kernel(const float *partial, int len, int n_slices, float *grad, TermSums terms,
-                                                            Moments norm, Map map) {
+                                                            double *squares, Map map) {
   dependents_may_start();
   wait_for_predecessor();
   if (blockIdx.x == kMomentBlocks) {
@@ -266,7 +296,7 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_slices_kernel(const flo
   __shared__ float quarter[4][kGradLanes];
   const int col = threadIdx.x % kGradLanes, q = threadIdx.x / kGradLanes;
   const int c_lo = n_slices * q / 4, c_hi = n_slices * (q + 1) / 4;
-  double a = 0.0, b = 0.0;
+  double none = 0.0, b = 0.0;
   for (int j0 = static_cast<int>(blockIdx.x) * kGradLanes; j0 < len; j0 += kMomentBlocks * kGradLanes) {
     const int j = j0 + col;
     const long long out = j < len ? map(j) : -1;
@@ -284,25 +314,27 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_slices_kernel(const flo
     if (q == 0 && out >= 0) {
       s = (s + quarter[1][col]) + (quarter[2][col] + quarter[3][col]);
       grad[out] = s;
-      a += s; b += static_cast<double>(s) * s;
+      b += static_cast<double>(s) * s;
     }
     __syncthreads();
   }
-  moments_finish(norm, a, b);
+  block_sum2(none, b);
+  if (threadIdx.x == 0) squares[blockIdx.x] = b;
 }
-// The moments of a gradient with the additions of reduce_slices_kernel.
+// The same sums of squares of a gradient that comes from elsewhere, with the additions of reduce_slices_kernel.
 template <class Map>
-__global__ void __launch_bounds__(256) grad_moments_kernel(Moments m, int len, Map map) {
+__global__ void __launch_bounds__(256) grad_squares_kernel(const float *grad, double *squares, int len, Map map) {
   dependents_may_start();
   wait_for_predecessor();
-  double a = 0.0, b = 0.0;
+  double none = 0.0, b = 0.0;
   if (threadIdx.x < kGradLanes)
     for (int j = static_cast<int>(blockIdx.x) * kGradLanes + static_cast<int>(threadIdx.x); j < len; j += kMomentBlocks * kGradLanes) {
       const long long p = map(j);
-      const float v = p >= 0 ? __ldcg(m.x + p) : 0.0f;
-      if (p >= 0) { a += v; b += static_cast<double>(v) * v; }
+      const float v = p >= 0 ? __ldcg(grad + p) : 0.0f;
+      if (p >= 0) b += static_cast<double>(v) * v;
     }
-  moments_finish(m, a, b);
+  block_sum2(none, b);
+  if (threadIdx.x == 0) squares[blockIdx.x] = b;
 }
 
 // Tensor-core path for H = 256 (update_tc256.cu): a net with hidden width 256 whose first layer takes `slabs` observation

@@ -89,12 +89,19 @@ struct PrepImage {
   unsigned char *image;
   ParamLayout L;
   int D, H;
-  __device__ void operator()(int tid, int nth) const;
+  template <class F>
+  __device__ void each(int tid, int nth, const F &value) const;  // value(p): parameter p
+  __device__ void operator()(int tid, int nth) const {
+    const float *from = params;
+    each(tid, nth, [from](size_t p) { return __ldcg(from + p); });
+  }
 };
 // One element per thread: a kernel that everything behind it waits for (as loops over the parts with 8 k threads it took 3 us more).
+// Every parameter has one place in the image.
 constexpr int kPrepW1 = kUH * kUK1, kPrepW2 = kUH * kUH, kPrepWh = kUHeadRows * kUH, kPrepTotal = kPrepW1 + kPrepW2 + kPrepWh + 2 * kUH + 8;
 constexpr int kPrepBlocks = (kPrepTotal + 255) / 256;
-__device__ __forceinline__ void PrepImage::operator()(int tid, int nth) const {
+template <class F>
+__device__ __forceinline__ void PrepImage::each(int tid, int nth, const F &value) const {
   for (int i = tid; i < kPrepTotal; i += nth) {
     size_t src = 0, at;    // parameter, place in the image
     bool real, wide = false;  // whether there is such a parameter; fp32 instead of bf16
@@ -115,10 +122,23 @@ __device__ __forceinline__ void PrepImage::operator()(int tid, int nth) const {
       j -= 2 * kUH;
       real = j <= kActions; src = j < kActions ? L.ba + j : L.bv; at = kImgBh + 4 * j; wide = true;
     }
-    const float v = real ? __ldcg(params + src) : 0.0f;
+    const float v = real ? value(src) : 0.0f;
     if (wide) *reinterpret_cast<float *>(image + at) = v;
     else *reinterpret_cast<__nv_bfloat16 *>(image + at) = __float2bfloat16_rn(v);
   }
+}
+
+// An optimiser step that leaves the next gradient its weight image and, by blocks of their own while the kernels in front still run,
+// its advantages' moments: two launches and a wait less between two minibatches than a step, then moments and image.
+template <class U>
+__global__ void __launch_bounds__(256) step_image_kernel(AdamArgs adam, PrepImage prep, Moments next) {
+  dependents_may_start();
+  if (static_cast<int>(blockIdx.x) < kMomentBlocks) moments_block<U>(next);
+  wait_for_predecessor();
+  if (static_cast<int>(blockIdx.x) < kMomentBlocks) return;
+  const float scale = adam_scale(adam);
+  prep.each((static_cast<int>(blockIdx.x) - kMomentBlocks) * 256 + static_cast<int>(threadIdx.x), (static_cast<int>(gridDim.x) - kMomentBlocks) * 256,
+            [&](size_t p) { return adam_element(adam, scale, p); });
 }
 
 // A canonical tile of C features read with the feature index as K: chunks (K groups) 128 bytes apart, 8-row groups C*16.  The same tile
@@ -704,11 +724,14 @@ size_t ppo_tc_image_bytes() { return kImgBytes; }
 size_t ppo_tc_slice_floats() { return kSlice; }
 
 cudaError_t launch_ppo_net_tc(mava_rollout *h, const float *params_dev, const ParamLayout &L, const UpdRows &rows, const UpdHyper &hp,
-                              const Moments &adv, void *image, float *partial, double *term_partial, int slices, float *grad, const TermSums &terms,
-                              const Moments &norm) {
-  const PrepImage prep{params_dev, static_cast<unsigned char *>(image), L, h->D, h->cfg.hidden};
-  cudaError_t err = launch_prologue(adv, prep, kPrepBlocks, h->stream);
-  if (err != cudaSuccess) return err;
+                              const Moments &adv, bool prepared, void *image, float *partial, double *term_partial, int slices, float *grad,
+                              const TermSums &terms, double *squares) {
+  cudaError_t err = cudaSuccess;
+  if (!prepared) {
+    err = launch_prologue(adv, PrepImage{params_dev, static_cast<unsigned char *>(image), L, h->D, h->cfg.hidden}, kPrepBlocks, h->stream);
+    if (err != cudaSuccess) return err;
+    h->launches += 1;
+  }
   const size_t smem = sizeof(UtcSmem);
   const auto kern = rows_need_64_bits(rows, rows.n) ? ppo_net_tc_kernel<uint64_t> : ppo_net_tc_kernel<uint32_t>;
   err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -716,12 +739,17 @@ cudaError_t launch_ppo_net_tc(mava_rollout *h, const float *params_dev, const Pa
   err = launch_dependent(kern, slices, kUThreads, smem, h->stream, static_cast<const unsigned char *>(image), rows, hp,
                          static_cast<const double *>(adv.out), partial, term_partial, h->d_status, h->D, h->cfg.hidden, adv.early);
   if (err != cudaSuccess) return err;
-  h->launches += 3;
+  h->launches += 2;
   return launch_dependent(reduce_slices_kernel<SliceMap>, kReduceBlocks, kReduceThreads, 0, h->stream, static_cast<const float *>(partial), kSlice, slices, grad,
-                          terms, norm, SliceMap{L, h->D, h->cfg.hidden});
+                          terms, squares, SliceMap{L, h->D, h->cfg.hidden});
 }
-cudaError_t launch_grad_moments_tc(mava_rollout *h, const ParamLayout &L, const Moments &norm) {
-  return launch_dependent(grad_moments_kernel<SliceMap>, kMomentBlocks, 256, 0, h->stream, norm, kSlice, SliceMap{L, h->D, h->cfg.hidden});
+cudaError_t launch_grad_squares_tc(mava_rollout *h, const ParamLayout &L, const float *grad, double *squares) {
+  return launch_dependent(grad_squares_kernel<SliceMap>, kMomentBlocks, 256, 0, h->stream, grad, squares, kSlice, SliceMap{L, h->D, h->cfg.hidden});
+}
+cudaError_t launch_step_tc(mava_rollout *h, const AdamArgs &adam, const ParamLayout &L, const Moments &next, void *image) {
+  h->launches += 1;
+  return launch_dependent(rows_need_64_bits(next.map, next.n) ? step_image_kernel<uint64_t> : step_image_kernel<uint32_t>, kMomentBlocks + kPrepBlocks, 256, 0,
+                          h->stream, adam, PrepImage{adam.params, static_cast<unsigned char *>(image), L, h->D, h->cfg.hidden}, next);
 }
 
 }  // namespace mava

@@ -413,6 +413,26 @@ def test_update_loop_with_several_ragged_tiles_per_sm(idx, n_envs, T, epochs, mi
     ro.close()
 
 
+@pytest.mark.parametrize("idx,n_envs,T", [(1, 148, 64), (1, 149, 64), (0, 297, 64), (2, 395, 48)])
+def test_tensor_core_update_where_its_tiles_in_flight_turn_over(idx, n_envs, T):
+    """H <= 128, two tiles of 128 rows in flight per SM (148): exactly one tile on every SM, a second one on some, a third (the first
+    that reuses buffers), three and a ragged end.  Tolerance: that of the bf16-operand mode above."""
+    import torch
+
+    w, ro, params = _rolled_out(idx, n_envs, T, BF16, flags=0)
+    g = torch.Generator(device="cuda").manual_seed(idx)
+    new = params + 0.6 * torch.randn(params.shape, generator=g, device="cuda") * params.std()
+    terms, grad = ro.ppo_grad(new)
+    assert ro.status() == binding.MAVA_OK
+    shapes = ppo.layer_shapes(wl.obs_dim(w), w["hidden"], w["n_agents"], w["net_kind"])
+    ref, ref_grad = _tensor_path_reference(w, shapes, new.cpu().numpy().astype(np.float64), _oracle_batch(w, ro, T), binding.ppo_defaults(), True)
+    t, gg = terms.cpu().numpy(), grad.cpu().numpy().astype(np.float64)
+    for k, name in enumerate(("total", "actor", "entropy", "value")):
+        assert abs(t[k] - ref[name]) <= 2e-4 * (1 + abs(ref[name])), (name, t[k], ref[name])
+    assert np.max(np.abs(gg - ref_grad)) <= 2e-3 * np.max(np.abs(ref_grad))
+    ro.close()
+
+
 def test_centralised_critics_gradient_where_its_ring_turns_over():
     """1024 tiles of the critic's net: its ring of at most 3 x 148 slots is used more than twice (each use is read by the W2 SM and
     by a W1 SM per pair of input slabs) and every weight SM adds its accumulators to memory after 48 tiles, which smaller
