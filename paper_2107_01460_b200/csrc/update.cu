@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(256) adam_kernel(AdamArgs a, size_t n) {
   dependents_may_start();
   wait_for_predecessor();
   const float scale = adam_scale(a);
-  for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += static_cast<size_t>(gridDim.x) * blockDim.x) adam_element(a, scale, i);
+  for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += static_cast<size_t>(gridDim.x) * blockDim.x) adam_element(a, adam_load(a, i), __ldcg(a.grad + i), scale, i);
 }
 
 // Scratch of the update block, made on first use: [moments of the advantages and of the gradient, counters][their partials][term partials][transposed
@@ -548,7 +548,7 @@ cudaError_t launch_adam_step(mava_rollout *h, float *params_dev, const float *gr
   double *squares = grad_squares_of(h);
   if (!norm_known) {
     err = tc ? launch_grad_squares_tc(h, L, grad_dev, squares)
-             : launch_dependent(grad_squares_kernel<IdentityMap>, kMomentBlocks, 256, 0, h->stream, grad_dev, squares, static_cast<int>(P), IdentityMap{});
+             : launch_dependent(grad_squares_kernel<IdentityMap>, kMomentBlocks, kGradLanes, 0, h->stream, grad_dev, squares, static_cast<int>(P), IdentityMap{});
     if (err != cudaSuccess) return err;
     h->launches += 1;
   }

@@ -207,14 +207,17 @@ struct TermSums {
   UpdHyper hp;
   float *out;                  // [4] total, actor, entropy, value; nullptr: not wanted
 };
-// Called by one whole block of at most 512 threads: every thread adds every nt-th entry, eight loads in flight, then a tree
+// Called by one whole block, done by its first kTermThreads threads at most: each adds every nt-th entry, eight loads in flight, then a tree
 // (a fixed order for a block size; one thread adding 256 shares took longer than the rest of the reduction).
+constexpr int kTermThreads = 512;
 __device__ __forceinline__ void loss_terms(const TermSums &t) {
   constexpr int kBatch = 8;
+  const int nt = min(static_cast<int>(blockDim.x), kTermThreads);
   __shared__ double st[3][16];
   if (!t.out) return;
-  const int i = threadIdx.x, nt = static_cast<int>(blockDim.x);
+  const int i = static_cast<int>(threadIdx.x);
   double a = 0.0, e = 0.0, v = 0.0;
+  if (i < nt) {
   for (int k0 = i; k0 < t.n_actor_part; k0 += kBatch * nt) {
     double x[kBatch], y[kBatch];
 #pragma unroll
@@ -236,6 +239,7 @@ __device__ __forceinline__ void loss_terms(const TermSums &t) {
     a += __shfl_xor_sync(0xFFFFFFFFu, a, o); e += __shfl_xor_sync(0xFFFFFFFFu, e, o); v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
   }
   if ((i & 31) == 0) { st[0][i >> 5] = a; st[1][i >> 5] = e; st[2][i >> 5] = v; }
+  }
   __syncthreads();
   if (i != 0) return;
   a = e = v = 0.0;
@@ -265,21 +269,27 @@ __device__ __forceinline__ float adam_scale(const AdamArgs &a) {
   __syncthreads();
   return scale;
 }
-__device__ __forceinline__ float adam_element(const AdamArgs &a, float scale, size_t i) {
-  const float g = __ldcg(a.grad + i) * scale;
-  const float mi = a.beta1 * a.m[i] + (1.0f - a.beta1) * g, vi = a.beta2 * a.v[i] + (1.0f - a.beta2) * g * g;
+// A parameter and its moments: the parts of a step that do not need the gradient can come before the wait for it.
+struct AdamState { float p, m, v; };
+__device__ __forceinline__ AdamState adam_load(const AdamArgs &a, size_t i) { return AdamState{__ldcg(a.params + i), __ldcg(a.m + i), __ldcg(a.v + i)}; }
+__device__ __forceinline__ float adam_element(const AdamArgs &a, const AdamState &s, float grad, float scale, size_t i) {
+  const float g = grad * scale;
+  const float mi = a.beta1 * s.m + (1.0f - a.beta1) * g, vi = a.beta2 * s.v + (1.0f - a.beta2) * g * g;
   a.m[i] = mi; a.v[i] = vi;
-  const float p = a.params[i] - a.lr * (mi / a.corr1) / (sqrtf(vi / a.corr2) + a.eps);
+  const float p = s.p - a.lr * (mi / a.corr1) / (sqrtf(vi / a.corr2) + a.eps);
   a.params[i] = p;
   return p;
 }
 
-// grad[map(j)] = sum of element j over the CTAs' slices of `len` floats, in a fixed order, and each block's sum of squares (the
-// 2-norm is what an optimiser step needs next); a block of its own turns the term sums into the loss terms.  Four threads per
-// element take a quarter of the slices each, 20 loads in flight; one round for 32 k elements (bound by the latency
-// of its loads; 148 slices of 28 k: 10.7 us from a cold cache; 16.7 with two rounds, batches of 16 and the loss terms added by block 0).
-constexpr int kGradLanes = 128;  // elements per block and round
-constexpr int kReduceBlocks = kMomentBlocks + 1, kReduceThreads = 4 * kGradLanes;
+__device__ __forceinline__ double squares_of_group(const double *warps) { return ((warps[0] + warps[1]) + warps[2]) + warps[3]; }
+
+// grad[map(j)] = sum of element j over the CTAs' slices of `len` floats, in a fixed order, and the sum of squares of each group of
+// kGradLanes elements (the 2-norm is what an optimiser step needs next); a block of its own turns the term sums into the loss terms.
+// Four threads per element take a quarter of the slices each, 20 loads in flight; two groups per block, so that all blocks run at
+// once: behind a kernel that fills the SMs only one block per SM was resident, and of 257 blocks of one group the last 109 started
+// when the first were done (six reductions of 28 k elements over 148 slices: 346 -> 338 us with the loads of the step before its wait).
+constexpr int kGradLanes = 128, kGroups = 2;  // elements per group; groups per block and round
+constexpr int kReduceBlocks = kMomentBlocks / kGroups + 1, kReduceThreads = 4 * kGradLanes * kGroups;
 struct IdentityMap {
   __device__ __forceinline__ long long operator()(int j) const { return j; }
 };
@@ -288,17 +298,19 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_slices_kernel(const flo
                                                             double *squares, Map map) {
   dependents_may_start();
   wait_for_predecessor();
-  if (blockIdx.x == kMomentBlocks) {
+  if (blockIdx.x == kMomentBlocks / kGroups) {
     loss_terms(terms);
     return;
   }
   constexpr int kBatch = 20;
-  __shared__ float quarter[4][kGradLanes];
-  const int col = threadIdx.x % kGradLanes, q = threadIdx.x / kGradLanes;
+  __shared__ float quarter[kGroups][4][kGradLanes];
+  __shared__ double warp_squares[kGroups][kGradLanes / 32];
+  const int col = threadIdx.x % kGradLanes, q = threadIdx.x / kGradLanes % 4, g = threadIdx.x / (4 * kGradLanes);
+  const int group = static_cast<int>(blockIdx.x) * kGroups + g;
   const int c_lo = n_slices * q / 4, c_hi = n_slices * (q + 1) / 4;
-  double none = 0.0, b = 0.0;
-  for (int j0 = static_cast<int>(blockIdx.x) * kGradLanes; j0 < len; j0 += kMomentBlocks * kGradLanes) {
-    const int j = j0 + col;
+  double b = 0.0;
+  for (int r0 = 0; r0 < len; r0 += kMomentBlocks * kGradLanes) {
+    const int j = r0 + group * kGradLanes + col;
     const long long out = j < len ? map(j) : -1;
     const float *src = partial + (out >= 0 ? j : 0);
     float s = 0.0f;
@@ -309,32 +321,41 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_slices_kernel(const flo
 #pragma unroll
       for (int k = 0; k < kBatch; ++k) s = c0 + k < c_hi ? s + v[k] : s;
     }
-    quarter[q][col] = s;
+    quarter[g][q][col] = s;
     __syncthreads();
     if (q == 0 && out >= 0) {
-      s = (s + quarter[1][col]) + (quarter[2][col] + quarter[3][col]);
+      s = (s + quarter[g][1][col]) + (quarter[g][2][col] + quarter[g][3][col]);
       grad[out] = s;
       b += static_cast<double>(s) * s;
     }
     __syncthreads();
   }
-  block_sum2(none, b);
-  if (threadIdx.x == 0) squares[blockIdx.x] = b;
+  if (q == 0) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xFFFFFFFFu, b, o);
+    if ((col & 31) == 0) warp_squares[g][col >> 5] = b;
+  }
+  __syncthreads();
+  if (q == 0 && col == 0) squares[group] = squares_of_group(warp_squares[g]);
 }
-// The same sums of squares of a gradient that comes from elsewhere, with the additions of reduce_slices_kernel.
+// The same sums of squares of a gradient that comes from elsewhere, with the additions of reduce_slices_kernel: a group per block.
 template <class Map>
-__global__ void __launch_bounds__(256) grad_squares_kernel(const float *grad, double *squares, int len, Map map) {
+__global__ void __launch_bounds__(kGradLanes) grad_squares_kernel(const float *grad, double *squares, int len, Map map) {
   dependents_may_start();
   wait_for_predecessor();
-  double none = 0.0, b = 0.0;
-  if (threadIdx.x < kGradLanes)
-    for (int j = static_cast<int>(blockIdx.x) * kGradLanes + static_cast<int>(threadIdx.x); j < len; j += kMomentBlocks * kGradLanes) {
-      const long long p = map(j);
-      const float v = p >= 0 ? __ldcg(grad + p) : 0.0f;
-      if (p >= 0) b += static_cast<double>(v) * v;
-    }
-  block_sum2(none, b);
-  if (threadIdx.x == 0) squares[blockIdx.x] = b;
+  __shared__ double warp_squares[kGradLanes / 32];
+  const int col = threadIdx.x;
+  double b = 0.0;
+  for (int j = static_cast<int>(blockIdx.x) * kGradLanes + col; j < len; j += kMomentBlocks * kGradLanes) {
+    const long long p = map(j);
+    const float v = p >= 0 ? __ldcg(grad + p) : 0.0f;
+    if (p >= 0) b += static_cast<double>(v) * v;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xFFFFFFFFu, b, o);
+  if ((col & 31) == 0) warp_squares[col >> 5] = b;
+  __syncthreads();
+  if (col == 0) squares[blockIdx.x] = squares_of_group(warp_squares);
 }
 
 // Tensor-core path for H = 256 (update_tc256.cu): a net with hidden width 256 whose first layer takes `slabs` observation

@@ -89,56 +89,64 @@ struct PrepImage {
   unsigned char *image;
   ParamLayout L;
   int D, H;
-  template <class F>
-  __device__ void each(int tid, int nth, const F &value) const;  // value(p): parameter p
-  __device__ void operator()(int tid, int nth) const {
-    const float *from = params;
-    each(tid, nth, [from](size_t p) { return __ldcg(from + p); });
+  // Element i of the image: its parameter (if there is one; every parameter has one place in the image) and where it lies.
+  struct Place { size_t param; uint32_t at; bool real, wide /* fp32 instead of bf16 */; };
+  __device__ Place place(int i) const;
+  __device__ void put(const Place &p, float v) const {
+    if (p.wide) *reinterpret_cast<float *>(image + p.at) = v;
+    else *reinterpret_cast<__nv_bfloat16 *>(image + p.at) = __float2bfloat16_rn(v);
   }
+  __device__ void operator()(int tid, int nth) const;
 };
 // One element per thread: a kernel that everything behind it waits for (as loops over the parts with 8 k threads it took 3 us more).
-// Every parameter has one place in the image.
 constexpr int kPrepW1 = kUH * kUK1, kPrepW2 = kUH * kUH, kPrepWh = kUHeadRows * kUH, kPrepTotal = kPrepW1 + kPrepW2 + kPrepWh + 2 * kUH + 8;
 constexpr int kPrepBlocks = (kPrepTotal + 255) / 256;
-template <class F>
-__device__ __forceinline__ void PrepImage::each(int tid, int nth, const F &value) const {
+__device__ __forceinline__ PrepImage::Place PrepImage::place(int j) const {
+  if (j < kPrepW1) {
+    const int n = j / kUK1, k = j - n * kUK1;
+    return Place{L.W1 + static_cast<size_t>(n) * D + k, kImgW1 + canon_offset(n, k, kUK1), n < H && k < D, false};
+  }
+  if ((j -= kPrepW1) < kPrepW2) {
+    const int n = j / kUH, k = j - n * kUH;
+    return Place{L.W2 + static_cast<size_t>(n) * H + k, kImgW2 + canon_offset(n, k, kUH), n < H && k < H, false};
+  }
+  if ((j -= kPrepW2) < kPrepWh) {
+    const int n = j / kUH, k = j - n * kUH;
+    return Place{n < kActions ? L.Wa + static_cast<size_t>(n) * H + k : L.Wv + k, kImgWh + canon_offset(n, k, kUH), k < H && n <= kActions, false};
+  }
+  if ((j -= kPrepWh) < 2 * kUH) {
+    const int n = j % kUH;
+    return Place{(j < kUH ? L.b1 : L.b2) + n, (j < kUH ? kImgB1 : kImgB2) + 4 * n, n < H, true};
+  }
+  j -= 2 * kUH;
+  return Place{j < kActions ? L.ba + j : L.bv, kImgBh + 4 * j, j <= kActions, true};
+}
+__device__ __forceinline__ void PrepImage::operator()(int tid, int nth) const {
   for (int i = tid; i < kPrepTotal; i += nth) {
-    size_t src = 0, at;    // parameter, place in the image
-    bool real, wide = false;  // whether there is such a parameter; fp32 instead of bf16
-    int j = i;
-    if (j < kPrepW1) {
-      const int n = j / kUK1, k = j - n * kUK1;
-      real = n < H && k < D; src = L.W1 + static_cast<size_t>(n) * D + k; at = kImgW1 + canon_offset(n, k, kUK1);
-    } else if ((j -= kPrepW1) < kPrepW2) {
-      const int n = j / kUH, k = j - n * kUH;
-      real = n < H && k < H; src = L.W2 + static_cast<size_t>(n) * H + k; at = kImgW2 + canon_offset(n, k, kUH);
-    } else if ((j -= kPrepW2) < kPrepWh) {
-      const int n = j / kUH, k = j - n * kUH;
-      real = k < H && n <= kActions; src = n < kActions ? L.Wa + static_cast<size_t>(n) * H + k : L.Wv + k; at = kImgWh + canon_offset(n, k, kUH);
-    } else if ((j -= kPrepWh) < 2 * kUH) {
-      const int n = j % kUH;
-      real = n < H; src = (j < kUH ? L.b1 : L.b2) + n; at = (j < kUH ? kImgB1 : kImgB2) + 4 * n; wide = true;
-    } else {
-      j -= 2 * kUH;
-      real = j <= kActions; src = j < kActions ? L.ba + j : L.bv; at = kImgBh + 4 * j; wide = true;
-    }
-    const float v = real ? value(src) : 0.0f;
-    if (wide) *reinterpret_cast<float *>(image + at) = v;
-    else *reinterpret_cast<__nv_bfloat16 *>(image + at) = __float2bfloat16_rn(v);
+    const Place p = place(i);
+    put(p, p.real ? __ldcg(params + p.param) : 0.0f);
   }
 }
 
 // An optimiser step that leaves the next gradient its weight image and, by blocks of their own while the kernels in front still run,
-// its advantages' moments: two launches and a wait less between two minibatches than a step, then moments and image.
+// its advantages' moments.  Everything but the gradient is read before the wait: what was launched before the gradient in front is
+// complete when this starts (launch_ppo_grad), the step before this one too.
 template <class U>
 __global__ void __launch_bounds__(256) step_image_kernel(AdamArgs adam, PrepImage prep, Moments next) {
   dependents_may_start();
-  if (static_cast<int>(blockIdx.x) < kMomentBlocks) moments_block<U>(next);
+  if (static_cast<int>(blockIdx.x) < kMomentBlocks) {
+    moments_block<U>(next);
+    wait_for_predecessor();
+    return;
+  }
+  const int i = (static_cast<int>(blockIdx.x) - kMomentBlocks) * 256 + static_cast<int>(threadIdx.x);
+  PrepImage::Place p{0, 0, false, false};
+  if (i < kPrepTotal) p = prep.place(i);
+  AdamState state{0.0f, 0.0f, 0.0f};
+  if (p.real) state = adam_load(adam, p.param);
   wait_for_predecessor();
-  if (static_cast<int>(blockIdx.x) < kMomentBlocks) return;
-  const float scale = adam_scale(adam);
-  prep.each((static_cast<int>(blockIdx.x) - kMomentBlocks) * 256 + static_cast<int>(threadIdx.x), (static_cast<int>(gridDim.x) - kMomentBlocks) * 256,
-            [&](size_t p) { return adam_element(adam, scale, p); });
+  const float grad = p.real ? __ldcg(adam.grad + p.param) : 0.0f, scale = adam_scale(adam);
+  if (i < kPrepTotal) prep.put(p, p.real ? adam_element(adam, state, grad, scale, p.param) : 0.0f);
 }
 
 // A canonical tile of C features read with the feature index as K: chunks (K groups) 128 bytes apart, 8-row groups C*16.  The same tile
@@ -744,7 +752,7 @@ cudaError_t launch_ppo_net_tc(mava_rollout *h, const float *params_dev, const Pa
                           terms, squares, SliceMap{L, h->D, h->cfg.hidden});
 }
 cudaError_t launch_grad_squares_tc(mava_rollout *h, const ParamLayout &L, const float *grad, double *squares) {
-  return launch_dependent(grad_squares_kernel<SliceMap>, kMomentBlocks, 256, 0, h->stream, grad, squares, kSlice, SliceMap{L, h->D, h->cfg.hidden});
+  return launch_dependent(grad_squares_kernel<SliceMap>, kMomentBlocks, kGradLanes, 0, h->stream, grad, squares, kSlice, SliceMap{L, h->D, h->cfg.hidden});
 }
 cudaError_t launch_step_tc(mava_rollout *h, const AdamArgs &adam, const ParamLayout &L, const Moments &next, void *image) {
   h->launches += 1;
