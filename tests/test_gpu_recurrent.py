@@ -73,6 +73,30 @@ def test_two_calls_continue_like_one_and_reset_replays(precision):
     assert a.status() == 0 and b.status() == 0
 
 
+@pytest.mark.parametrize("name,n_envs,T", [(REC2, 6001, 60), (REC1, 1999, 21), (REC1, 9601, 5)])
+def test_an_environments_rows_do_not_depend_on_the_batch_around_it(name, n_envs, T):
+    """Environments rolled out alone (global indices kept) against the same ones inside a batch: other tiles, other warps and lanes,
+    several tiles per SM (148 x 40 environments of three agents, 148 x 64 of two, at most), odd batches whose rows
+    start off the 16-byte boundaries.  Same bytes."""
+    import torch
+
+    w = wl.workload(name)
+    params = torch.from_numpy(wl.make_params(w, bias_scale=0.1)).cuda()
+    names = ("obs", "actions", "logp", "values", "rewards", "dones")
+    whole = binding.Rollout(binding.make_config(w, precision=BF16, max_T=T, n_envs=n_envs))
+    whole.run(params, T)
+    for lo, n in ((0, 37), (n_envs // 2, 1), (n_envs - 41, 41)):
+        part = binding.Rollout(binding.make_config(w, precision=BF16, max_T=T, n_envs=n, first_env=lo))
+        part.run(params, T)
+        for k in names:
+            assert torch.equal(getattr(whole, k)[:, lo: lo + n], getattr(part, k)), (lo, k)
+        assert np.array_equal(whole.get_hidden()[lo: lo + n], part.get_hidden())
+        assert part.status() == binding.MAVA_OK
+        part.close()
+    assert whole.status() == binding.MAVA_OK
+    whole.close()
+
+
 @pytest.mark.parametrize("name", [REC1, REC2])
 def test_recurrent_full_size(name):
     """The full-size recurrent workloads in the precision the benchmark times: environment arrays for every environment,
