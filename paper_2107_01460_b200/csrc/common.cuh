@@ -94,6 +94,25 @@ __device__ __forceinline__ int greedy_action(const float *l) {
   return best;
 }
 
+// Inverse-CDF draw from the softmax of six logits: the smallest k with u * sum < e_0 + ... + e_k (else the last), which is as many as there
+// are partial sums that do not exceed u * sum, because those never fall.  Gives the largest logit and the sum too.
+__device__ __forceinline__ int draw_action(const float *l, float u, float &top, float &sum) {
+  static_assert(kActions == 6, "the maximum's tree");
+  top = fmaxf(fmaxf(fmaxf(l[0], l[1]), fmaxf(l[2], l[3])), fmaxf(l[4], l[5]));
+  float upto[kActions];
+#pragma unroll
+  for (int k = 0; k < kActions; ++k) {
+    const float e = __expf(l[k] - top);
+    upto[k] = k == 0 ? e : upto[k - 1] + e;
+  }
+  sum = upto[kActions - 1];
+  const float target = u * sum;
+  int action = 0;
+#pragma unroll
+  for (int k = 0; k < kActions - 1; ++k) action += target < upto[k] ? 0 : 1;
+  return action;
+}
+
 // Re-laid-out fp32 weights of the SIMT path: every dense layer transposed to [in][out].
 struct SimtWeights {
   const float *W1t, *b1, *W2t, *b2, *Wa, *ba, *Wv, *bv;  // Wa [6][H], Wv [H] stay row-major

@@ -635,22 +635,8 @@ rollout_tc_kernel(RolloutArgs a, const unsigned char *image, int ept, int n_tile
         if (active) {
           pend = !ev; pend_step = !last; pend_row0 = row0; pend_value = hv[kActions];
           if (!last) {
-            float e[kActions];
-            float m = hv[0];
-#pragma unroll
-            for (int k = 1; k < kActions; ++k) m = fmaxf(m, hv[k]);
-            float sum = 0.0f;
-#pragma unroll
-            for (int k = 0; k < kActions; ++k) { e[k] = __expf(hv[k] - m); sum += e[k]; }
-            const float target = u * sum;
-            action = kActions - 1;
-            float cdf = 0.0f;
-            bool found = false;
-#pragma unroll
-            for (int k = 0; k < kActions; ++k) {
-              cdf += e[k];
-              if (!found && target < cdf) { action = k; found = true; }
-            }
+            float m, sum;
+            action = draw_action(hv, u, m, sum);
             if (a.forced) {
               action = a.forced[row0 + crow];
               if (action < 0 || action >= kActions) action = 0;

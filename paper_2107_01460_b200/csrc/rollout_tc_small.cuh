@@ -358,22 +358,8 @@ rollout_tc_small_kernel(RolloutArgs a, const unsigned char *image, int ept) {
           out_value = hv[kActions];
           if (!last) {
             const float u = lds_f32(uni_addr + 4u * static_cast<uint32_t>((t & 3) * RB + lane));
-            float e[kActions];
-            float m = hv[0];
-#pragma unroll
-            for (int k = 1; k < kActions; ++k) m = fmaxf(m, hv[k]);
-            float sum = 0.0f;
-#pragma unroll
-            for (int k = 0; k < kActions; ++k) { e[k] = __expf(hv[k] - m); sum += e[k]; }
-            const float target = u * sum;
-            action = kActions - 1;
-            float cdf = 0.0f;
-            bool found = false;
-#pragma unroll
-            for (int k = 0; k < kActions; ++k) {
-              cdf += e[k];
-              if (!found && target < cdf) { action = k; found = true; }
-            }
+            float m, sum;
+            action = draw_action(hv, u, m, sum);
             const size_t row = static_cast<size_t>(t) * M + static_cast<size_t>(e0) * N + lane;
             if (a.forced) {
               action = a.forced[row];
