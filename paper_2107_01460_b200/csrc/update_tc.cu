@@ -287,6 +287,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
     // above of every fourth row; the second load of a pair finds its sectors in L1.
     const int lw = warp - kUMain / 32, sub = lane >> 3, c2 = 64 + 2 * (lane & 7);
     const bool has0 = c2 < D, has1 = c2 + 1 < D;
+    const float pad0 = c2 == D ? 1.0f : 0.0f, pad1 = c2 + 1 == D ? 1.0f : 0.0f;  // a spare column holds ones (d b1)
     auto row_of = [&](int i) {
       const long long q = tile_of(i) * kUR + kLoadRows * lw + lane;
       return row_lookup<U>(rows, q, lane < kLoadRows && i < my_tiles && q < rows.n);
@@ -318,7 +319,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
 #pragma unroll
       for (int r = 0; r < kLoadRows; ++r) pk[r] = pack_bf16(v[r][0], v[r][1]);
 #pragma unroll
-      for (int r = 0; r < kLoadRows / 4; ++r) pt[r] = pack_bf16(t[r][0], t[r][1]);
+      for (int r = 0; r < kLoadRows / 4; ++r) pt[r] = pack_bf16(has0 ? t[r][0] : pad0, has1 ? t[r][1] : pad1);
       if (i >= 2) ok = ok && mbar_sleep_warp(x_empty0 + 8u * (i & 1), static_cast<uint32_t>((i >> 1) - 1) & 1u);
       if (!ok || *abort_flag) break;
       const uint32_t xt = xt0 + kXTile * static_cast<uint32_t>(i & 1) + 16u * static_cast<uint32_t>(kLoadRows * lw);
@@ -327,7 +328,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
 #pragma unroll
       for (int r = 0; r < kLoadRows; ++r) {
         sts_u32(at + 16u * r, pk[r]);
-        if ((r & 3) == 0) sts_u32(at4 + 16u * r, pt[r / 4]);  // (columns from D on: zeros)
+        if ((r & 3) == 0) sts_u32(at4 + 16u * r, pt[r / 4]);  // (behind column D: zeros)
       }
       fence_async_smem();
       warp_arrive(x_full0 + 8u * (i & 1), lane);
@@ -446,7 +447,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
       }
       if (bwd) {
         fresh();
-        if (ok && elect_one()) {  // d b1 [out] += d z1^T . ones
+        if (D == kUK1 && ok && elect_one()) {  // d b1 [out] += d z1^T . ones (otherwise a column of d W1)
 #pragma unroll
           for (int k = 0; k < kUR / 16; ++k)
             mma_bf16(tmem + kColDB1, act_mn(AT16(h1) + hb, k), dh_mn(AT16(dhead), k), instr_desc(kUH, kUHeads) | kGrad, keep | (k > 0));
@@ -706,8 +707,11 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
       put(part + kSlWh, v, 8, 2.0f);  // (dhead at half its size)
       tmem_ld16(from + kColDB2, w);
       if (unit < H) part[kSlB2 + unit] = w[7];
-      tmem_ld16(from + kColDB1, w);
-      if (unit < H) part[kSlB1 + unit] = w[7];
+      uint32_t db1;
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(db1) : "r"(from + (D == kUK1 ? kColDB1 + 7u : kColDW1 + static_cast<uint32_t>(D))) : "memory");
+      tmem_ld_wait();
+      asm volatile("" : "+r"(db1));
+      if (unit < H) part[kSlB1 + unit] = __uint_as_float(db1);
     }
     if (tid <= kActions) part[kSlBh + tid] = (sums.bias[0][tid] + sums.bias[1][tid]) + (sums.bias[2][tid] + sums.bias[3][tid]);
   }
