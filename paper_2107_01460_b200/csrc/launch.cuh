@@ -4,8 +4,9 @@
 // from it (barriers, tensor memory, zeroed tiles) and then waits until that one is complete and its writes are visible.
 // Rules for a kernel that is launched like this:
 //   - Every block waits, whatever it does before: a kernel's completion then implies that of all before it.  All threads of a
-//     block wait, but for those that only read what an even earlier kernel is known to have finished (the row loaders of
-//     ppo_net_tc_kernel inside mava_ppo_update; launch_ppo_grad has the argument).
+//     block wait, but for those that only read what an even earlier kernel is known to have finished (what fetches rows in
+//     ppo_net_tc_kernel inside mava_ppo_update; launch_ppo_grad has the argument, which also lets step_image_kernel read the
+//     optimiser's state before its wait).
 //   - Memory that a kernel in front may still be writing is not constant for the kernel's lifetime, so it must not be declared
 //     so: no __restrict__ on its parameters and no load through the non-coherent path (__ldg, ld.global.nc).  Either lets the
 //     compiler take a load for an invariant and move it over the wait.  Where loads should go out in a batch they are __ldcg.
