@@ -10,7 +10,7 @@
 // MN-major B operand of d h1 = d z2 . W2.
 //   per tile:  x -> z1 -> h1 -> z2 -> h2 -> logits, value -> loss and its per-row derivatives (fp32, thread = row)
 //              -> d h2 -> d z2 -> d h1 -> d z1, and on the side d Wh^T += h2^T . dhead, d W2 += d z2^T . h1,
-//              d W1 += d z1^T . x, d b2 += d z2^T . 1, d b1 += d z1^T . 1 (the ones are column 7 of the dhead tile).
+//              d W1 += d z1^T . x, d b2 += d z2^T . 1, d b1 += d z1^T . 1 (the ones are a constant tile of 16 rows).
 // Two tiles are in flight: tile s goes forward while tile s - 1 goes backward, so that one's epilogue runs beside the other's products.
 // Both fit an SM because d z2 takes h2's place and d z1 h1's (behind the weight-gradient products that read them), and
 // the heads' derivatives are kept once, eight columns wide.  Sixteen warps share every epilogue (32 rows x 32 columns each), eight
@@ -41,7 +41,7 @@ namespace {
 constexpr int kUR = 128;        // rows per tile (M of the per-row products, K of the weight-gradient products)
 constexpr int kUH = 128;        // hidden width, padded
 constexpr int kUK1 = 80;        // input width, padded to the MMA's K step
-constexpr int kUHeads = 16;     // N of the products with the heads: six logits, the value, a column of ones; the other eight repeat or are not read
+constexpr int kUHeads = 16;     // N of the products with the heads: six logits, the value, a column of zeros; the other eight repeat or are not read
 constexpr int kUHeadRows = 8;   // of which these exist in memory
 constexpr int kUMain = 512;     // threads of the epilogues: a warp has 32 rows x 32 columns of a tile
 constexpr int kLossWarps = 8;   // of which these also do the loss: four the actor's part, four the value's, a row per thread
@@ -78,6 +78,7 @@ struct UtcSmem {  // two tiles are in flight, an even and an odd one
   // what the loss needs of a tile's rows (the old log-probs and advantages take the place of the biases, which are in registers by then)
   float value_old[kUR], ret[kUR];
   unsigned char action[kUR];  // 0xFF: no such row
+  alignas(16) unsigned char ones[16 * kUHeadRows * 2];  // bf16 ones, the rows of a K step: operand of the column sums, never rewritten
   alignas(8) uint64_t bar_load[2], done[kProducts], ready[kEpilogues], x_full[2], x_empty[2], rows_full, bar_end;
   uint32_t tmem_base;
   int abort;  // a warp gave up
@@ -256,6 +257,10 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  if (tid < static_cast<int>(sizeof(sm.ones) / 4)) {
+    sts_u32(smem_u32(sm.ones) + 4u * static_cast<uint32_t>(tid), 0x3F803F80u);
+    fence_async_smem();
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -347,6 +352,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
     auto act_k = [](uint32_t at, int k) { return desc16<128, kUH * 16>(at + k * 16); };              // activations, feature as K
     auto act_mn = [](uint32_t at, int k) { return desc16<kUH * 16, 128>(at + k * 2 * kUH); };        // row as K
     auto dh_mn = [](uint32_t at, int k) { return desc16<128, 0>(at + k * 16); };                     // dhead, row as K, its columns twice
+    auto ones_mn = [](uint32_t at) { return desc16<128, 0>(at); };                                   // the same rows of ones for every step
     constexpr uint32_t kX16 = kXTile / 16, kH16 = kHTile / 16;
     const uint32_t block16 = smem_u32(&sm) >> 4;
     uint32_t base = block16;
@@ -419,10 +425,10 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
       }
       if (bwd) {
         fresh();
-        if (ok && elect_one()) {  // d b2 [out] += d z2^T . ones (column 7 of dhead, of whichever tile)
+        if (ok && elect_one()) {  // d b2 [out] += d z2^T . ones
 #pragma unroll
           for (int k = 0; k < kUR / 16; ++k)
-            mma_bf16(tmem + kColDB2, act_mn(AT16(h2) + hb, k), dh_mn(AT16(dhead), k), instr_desc(kUH, kUHeads) | kGrad, keep | (k > 0));
+            mma_bf16(tmem + kColDB2, act_mn(AT16(h2) + hb, k), ones_mn(AT16(ones)), instr_desc(kUH, kUHeads) | kGrad, keep | (k > 0));
         }
         __syncwarp();
         handed_over(kDz1, s - 1);
@@ -450,7 +456,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
         if (D == kUK1 && ok && elect_one()) {  // d b1 [out] += d z1^T . ones (otherwise a column of d W1)
 #pragma unroll
           for (int k = 0; k < kUR / 16; ++k)
-            mma_bf16(tmem + kColDB1, act_mn(AT16(h1) + hb, k), dh_mn(AT16(dhead), k), instr_desc(kUH, kUHeads) | kGrad, keep | (k > 0));
+            mma_bf16(tmem + kColDB1, act_mn(AT16(h1) + hb, k), ones_mn(AT16(ones)), instr_desc(kUH, kUHeads) | kGrad, keep | (k > 0));
         }
         __syncwarp();
       }
@@ -594,7 +600,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
       const int row = 32 * wq + lane, action = sm.action[row];
       const bool real = action != 0xFF;
       // loss terms and the per-row derivatives with respect to the six logits and the value.  dhead: columns 0..6 the derivatives at
-      // half their size; column 7: one (it turns the d z^T products into column sums)
+      // half their size; column 7: zero
       if (fwd && is_actor) {
         product(kLogits, s);
         const float in0 = reinterpret_cast<const float *>(sm.img + kImgB1)[row], in1 = reinterpret_cast<const float *>(sm.img + kImgB2)[row];
@@ -641,7 +647,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
           d = (in_range || u * u > uc * uc) ? hp.vf_coef * u * inv_n : 0.0f;
           t0 += 0.5 * fmaxf(u * u, uc * uc);
         }
-        sts_u32(dht + 16u * static_cast<uint32_t>(row) + 12u, pack_bf16(0.5f * d, 1.0f));
+        sts_u32(dht + 16u * static_cast<uint32_t>(row) + 12u, pack_bf16(0.5f * d, 0.0f));
         hand_over(kLoss);
         gbh[0] += d;
       }
@@ -706,9 +712,9 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
       for (int c = 0; c < 8; ++c) v[c] = __float_as_uint(w[c]);
       put(part + kSlWh, v, 8, 2.0f);  // (dhead at half its size)
       tmem_ld16(from + kColDB2, w);
-      if (unit < H) part[kSlB2 + unit] = w[7];
+      if (unit < H) part[kSlB2 + unit] = w[0];
       uint32_t db1;
-      asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(db1) : "r"(from + (D == kUK1 ? kColDB1 + 7u : kColDW1 + static_cast<uint32_t>(D))) : "memory");
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(db1) : "r"(from + (D == kUK1 ? kColDB1 : kColDW1 + static_cast<uint32_t>(D))) : "memory");
       tmem_ld_wait();
       asm volatile("" : "+r"(db1));
       if (unit < H) part[kSlB1 + unit] = __uint_as_float(db1);

@@ -64,3 +64,15 @@ def test_inline_assembly_that_reads_memory_is_kept_in_order():
         for m in re.finditer(r"\basm\s*\(", text):  # (asm volatile does not match)
             statement = text[m.start():_closing(text, m.end() - 1, "()")]
             assert not re.search(r"\b(ld|tcgen05\.ld|ldmatrix|atom|red|st|mbarrier)\b", statement), (name, statement[:120])
+
+
+def test_head_derivatives_have_been_read_before_their_next_writer_is_let_on():
+    """The update kernel of H <= 128 keeps one tile of head derivatives for two tiles of rows in flight.  The loss that writes it waits
+    for the logits' products only, and a commit covers what was issued before it: no product that reads the tile may be issued
+    between that commit and the end of a turn."""
+    body = {k: b for _, k, _, b in _kernels()}["ppo_net_tc_kernel"]
+    reads = [m.start() for m in re.finditer(r"AT16\(dhead\)", body)]
+    writer = body.index("product(kLogits, s)")
+    commit = body.index("mma_commit(done0 + 8 * kLogits)")
+    assert len(reads) >= 2 and commit < writer
+    assert all(at < commit for at in reads), "a product that reads the tile is behind the commit its writer waits for"
