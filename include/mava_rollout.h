@@ -297,14 +297,17 @@ int mava_rollout_run_static(const mava_config_t *cfg, const mava_buffers_t *buff
  * mbarrier is bounded; when one runs out the kernel records it in the status word, lets the copies it still has
  * in flight land, frees its tensor memory and returns, and mava_rollout_status answers MAVA_ERR_DEVICE_TIMEOUT.
  * This call arms the NEXT launch of `which` (MAVA_EXPIRE_GAE: the copy-engine GAE kernel; MAVA_EXPIRE_ROLLOUT:
- * the 128-row tensor-core rollout kernel) so that one thread block makes one extra wait, with a limit of a few
- * thousand polls, on a barrier phase that nothing will complete, at a point where none of its copies or MMAs is
- * outstanding.  That block gives up exactly as after a real time-out; its outputs (and, for the rollout, the
- * environment states of its tile) are then incomplete, so the caller resets the handle afterwards.  One launch
- * only; a launch that takes another kernel (a shape the armed kernel does not serve) leaves the request armed.
+ * the 128-row tensor-core rollout kernel; MAVA_EXPIRE_UPDATE: the tensor-core gradient kernel for hidden widths of
+ * at most 128) so that one thread block makes one extra wait, with a limit of a few thousand polls, on a barrier
+ * phase that nothing will complete, at a point where none of its MMAs is outstanding (nor, but for the update's
+ * weight image, any of its copies).  That block gives up exactly as after a real time-out (the update's warps that
+ * wait for the one that gave up run into their own limits, a few seconds); its outputs are then incomplete (for the
+ * rollout also the environment states of its tile), so the caller resets the handle or repeats the gradient.  One
+ * launch only; a launch that takes another kernel (a shape the armed kernel does not serve) leaves the request armed.
  * Errors: INVALID_ARG. */
 #define MAVA_EXPIRE_GAE 1
 #define MAVA_EXPIRE_ROLLOUT 2
+#define MAVA_EXPIRE_UPDATE 4
 int mava_debug_expire_next_wait(mava_rollout_t *h, int32_t which);
 
 /* Number of kernels this handle has launched so far (for launch accounting). */

@@ -27,6 +27,7 @@ MAVA_FLAG_WIDE_TILES = 4
 MAVA_FLAG_UPDATE_FP32 = 8
 MAVA_EXPIRE_GAE = 1
 MAVA_EXPIRE_ROLLOUT = 2
+MAVA_EXPIRE_UPDATE = 4
 MAVA_GAE_MAX_T = 1024
 N_ACTIONS = 6
 

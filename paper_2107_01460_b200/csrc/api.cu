@@ -203,7 +203,7 @@ int mava_gae(mava_rollout_t *h, float gamma, float lambda) {
 }
 
 int mava_debug_expire_next_wait(mava_rollout_t *h, int32_t which) {
-  if (!h || (which != MAVA_EXPIRE_GAE && which != MAVA_EXPIRE_ROLLOUT)) return MAVA_ERR_INVALID_ARG;
+  if (!h || (which != MAVA_EXPIRE_GAE && which != MAVA_EXPIRE_ROLLOUT && which != MAVA_EXPIRE_UPDATE)) return MAVA_ERR_INVALID_ARG;
   h->expire_next |= which;
   return MAVA_OK;
 }

@@ -236,7 +236,7 @@ __device__ __forceinline__ void tmem_ld_wait32(uint32_t *r) {
 template <class U>  // row numbers of the batch (real_row)
 __global__ void __launch_bounds__(kUThreads, 1)
 ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const double *adv_stats,
-                  float *partial, double *term_partial, int *status, int D, int H, bool rows_ready) {
+                  float *partial, double *term_partial, int *status, int D, int H, bool rows_ready, int debug_expire) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   UtcSmem &sm = *reinterpret_cast<UtcSmem *>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31;
@@ -361,6 +361,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
 #define AT16(member) (base + static_cast<uint32_t>(offsetof(UtcSmem, member) / 16))
 #define IMG16(off) (base + static_cast<uint32_t>((offsetof(UtcSmem, img) + (off)) / 16))
     ok = mbar_sleep_warp(bar_load, 0);
+    if (debug_expire && blockIdx.x == 0) ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar_end, 0, 1u << 12)) != 0;  // (nothing completes this phase before the end)
 #pragma unroll 1
     for (int s = 0; s <= my_tiles && ok; ++s) {
       const bool fwd = s < my_tiles, bwd = s > 0;
@@ -671,6 +672,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
   // ---- the CTA's slice: accumulators out of tensor memory, once (what belongs to real units)
   if (!ok) *abort_flag = 1;
   ok = __syncthreads_and(ok) != 0;  // (the last products have been issued)
+  if (!ok) { mbar_wait(bar_load, 0); mbar_wait(bar_load + 8, 0); }  // who gave up may not have waited for the whole image: the copies land first
   ok &= mbar_wait(bar_end, 0);
   ok = __syncthreads_and(ok) != 0;
   const UtcSums &sums = *reinterpret_cast<const UtcSums *>(sm.img + kImgW2);
@@ -750,12 +752,14 @@ cudaError_t launch_ppo_net_tc(mava_rollout *h, const float *params_dev, const Pa
     if (err != cudaSuccess) return err;
     h->launches += 1;
   }
+  const int expire = (h->expire_next & MAVA_EXPIRE_UPDATE) ? 1 : 0;
+  h->expire_next &= ~MAVA_EXPIRE_UPDATE;
   const size_t smem = sizeof(UtcSmem);
   const auto kern = rows_need_64_bits(rows, rows.n) ? ppo_net_tc_kernel<uint64_t> : ppo_net_tc_kernel<uint32_t>;
   err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (err != cudaSuccess) return err;
   err = launch_dependent(kern, slices, kUThreads, smem, h->stream, static_cast<const unsigned char *>(image), rows, hp,
-                         static_cast<const double *>(adv.out), partial, term_partial, h->d_status, h->D, h->cfg.hidden, adv.early);
+                         static_cast<const double *>(adv.out), partial, term_partial, h->d_status, h->D, h->cfg.hidden, adv.early, expire);
   if (err != cudaSuccess) return err;
   h->launches += 2;
   return launch_dependent(reduce_slices_kernel<SliceMap>, kReduceBlocks, kReduceThreads, 0, h->stream, static_cast<const float *>(partial), kSlice, slices, grad,

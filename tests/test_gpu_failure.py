@@ -1,6 +1,6 @@
 """The give-up path of the kernels' bounded waits, exercised without faulting, trapping or hanging anything: one armed
 launch makes one thread block wait briefly on a barrier phase that nothing completes, at a point where none of its
-copies or MMAs is outstanding.  The block must record the time-out and leave in order (copies drained, tensor memory
+MMAs is outstanding (and no copy but the update's weight image).  The block must record the time-out and leave in order (copies drained, tensor memory
 freed, its partner thread group walked through the hand-over protocol), the status call must report it once, and the
 same handle must work again afterwards."""
 import numpy as np
@@ -55,6 +55,30 @@ def test_rollout_kernel_gives_up_and_recovers(idx, n_envs):
     assert ro.status() == binding.MAVA_ERR_DEVICE_TIMEOUT
     assert ro.status() == binding.MAVA_OK
     _fresh_run_matches(w, ro, params, p_dev, T, wl.sample_env_ids(n_envs, 4, 4, 8, seed=7))
+
+
+@pytest.mark.parametrize("idx,n_envs,T", [(0, 24, 16), (2, 395, 48)])
+def test_update_kernel_gives_up_and_recovers(idx, n_envs, T):
+    """The warp that issues the products gives up before its first, with the second half of the weight image possibly still on
+    its way: every other role of the block runs into its own limit (idx 2: three tiles per SM, so the row loaders stand
+    before an x tile that nobody frees), the image lands, and the block leaves.  The same call then gives the same bytes."""
+    import torch
+
+    w = wl.workload(idx)
+    ro = binding.Rollout(binding.make_config(w, precision=BF16, max_T=T, n_envs=n_envs))
+    params = torch.from_numpy(wl.make_params(w)).cuda()
+    ro.run(params, T)
+    ro.gae(wl.GAMMA, wl.LAMBDA)
+    want = [x.clone() for x in ro.ppo_grad(params)]
+    assert ro.status() == binding.MAVA_OK
+    ro.debug_expire_next_wait(binding.MAVA_EXPIRE_UPDATE)
+    ro.ppo_grad(params)
+    assert ro.status() == binding.MAVA_ERR_DEVICE_TIMEOUT
+    assert ro.status() == binding.MAVA_OK
+    got = ro.ppo_grad(params)
+    assert ro.status() == binding.MAVA_OK
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
+    ro.close()
 
 
 def test_gae_longer_than_its_limit_is_a_capacity_error():

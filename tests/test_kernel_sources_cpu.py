@@ -66,6 +66,13 @@ def test_inline_assembly_that_reads_memory_is_kept_in_order():
             assert not re.search(r"\b(ld|tcgen05\.ld|ldmatrix|atom|red|st|mbarrier)\b", statement), (name, statement[:120])
 
 
+def test_the_update_kernel_lets_its_weight_image_land_when_it_gives_up():
+    """The image comes on two barriers.  A role that gives up may have waited for neither; the block must, before it leaves."""
+    body = {k: b for _, k, _, b in _kernels()}["ppo_net_tc_kernel"]
+    end = body[body.index("__syncthreads_and(ok)"):]
+    assert re.search(r"mbar_wait\(bar_load, 0\)", end) and re.search(r"mbar_wait\(bar_load \+ 8, 0\)", end)
+
+
 def test_head_derivatives_have_been_read_before_their_next_writer_is_let_on():
     """The update kernel of H <= 128 keeps one tile of head derivatives for two tiles of rows in flight.  The loss that writes it waits
     for the logits' products only, and a commit covers what was issued before it: no product that reads the tile may be issued
