@@ -225,14 +225,14 @@ int mava_ppo_grad(mava_rollout_t *h, const float *params_dev, const mava_ppo_hyp
 }
 
 static int grad_envs(mava_rollout_t *h, const float *params_dev, const mava_ppo_hyper_t *hp, const int32_t *env_ids_dev,
-                     int32_t n_ids, float *grad_dev, float *terms_dev, int seq, bool prepared) {
+                     int32_t n_ids, float *grad_dev, float *terms_dev, int place, bool prepared) {
   if (!h || !params_dev || !hp || !grad_dev || !env_ids_dev || n_ids < 1 || h->last_T < 1 || !h->buf.adv || !h->buf.ret)
     return MAVA_ERR_INVALID_ARG;
   if (!(hp->clip_eps > 0.0f)) return MAVA_ERR_INVALID_ARG;
   if (h->cfg.net_kind == MAVA_NET_RECURRENT) return MAVA_ERR_UNSUPPORTED;
   DeviceGuard guard(h->device);
   if (!guard.ok) return cuda_failed();
-  return launch_ppo_grad(h, params_dev, *hp, grad_dev, terms_dev, env_ids_dev, n_ids, seq, prepared) == cudaSuccess ? MAVA_OK : cuda_failed();
+  return launch_ppo_grad(h, params_dev, *hp, grad_dev, terms_dev, env_ids_dev, n_ids, place, prepared) == cudaSuccess ? MAVA_OK : cuda_failed();
 }
 
 int mava_ppo_grad_envs(mava_rollout_t *h, const float *params_dev, const mava_ppo_hyper_t *hp, const int32_t *env_ids_dev,
@@ -263,15 +263,15 @@ int mava_ppo_update(mava_rollout_t *h, float *params_dev, float *m_dev, float *v
   }
   const bool prepares = adam_step_prepares(h);
   const int64_t total = static_cast<int64_t>(epochs) * minibatches;
-  auto piece = [&](int64_t i) {  // minibatch i of the call: its environments
+  auto piece = [&](int64_t i) {  // minibatch i of the call: its environments; neighbours' moments have different places
     const int64_t e = i / minibatches, k = i - e * minibatches;
     const int lo = static_cast<int>(static_cast<int64_t>(E) * k / minibatches), hi = static_cast<int>(static_cast<int64_t>(E) * (k + 1) / minibatches);
-    return NextMinibatch{perm_dev + static_cast<size_t>(e) * E + lo, hi - lo, i > 0 ? 2 - static_cast<int>(i & 1) : 0};  // (what counts is the parity, and the first)
+    return NextMinibatch{perm_dev + static_cast<size_t>(e) * E + lo, hi - lo, static_cast<int>(i & 1)};
   };
   for (int64_t i = 0; i < total; ++i) {
     const NextMinibatch now = piece(i);
     float *terms = terms_dev ? terms_dev + 4 * static_cast<size_t>(i) : nullptr;
-    const int rc = grad_envs(h, params_dev, hp, now.env_ids, now.n, grad_dev, terms, now.seq, prepares && i > 0);
+    const int rc = grad_envs(h, params_dev, hp, now.env_ids, now.n, grad_dev, terms, now.place, prepares && i > 0);
     if (rc != MAVA_OK) return rc;
     DeviceGuard guard(h->device);
     NextMinibatch next{};

@@ -180,11 +180,11 @@ size_t rec_tc_weight_bytes(const mava_config_t &cfg);
 
 // Update block.
 cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava_ppo_hyper_t &hp, float *grad_dev, float *terms_dev,
-                            const int32_t *env_ids_dev, int32_t n_ids, int seq = 0, bool prepared = false);
+                            const int32_t *env_ids_dev, int32_t n_ids, int place = 0, bool prepared = false);
 cudaError_t reserve_update(mava_rollout *h, int n_small, int n_large);  // scratch of gradients over n_small or n_large environments of the last run and
                                                                          // of their optimiser steps
-// The minibatch of the gradient that is launched directly behind a step, and its number in the chain (`seq` of launch_ppo_grad).
-struct NextMinibatch { const int32_t *env_ids; int n, seq; };
+// The minibatch of the gradient that is launched directly behind a step, and the place of its moments (launch_ppo_grad).
+struct NextMinibatch { const int32_t *env_ids; int n, place; };
 cudaError_t launch_adam_step(mava_rollout *h, float *params_dev, const float *grad_dev, float *m_dev, float *v_dev, int32_t step,
                              const mava_ppo_hyper_t &hp, bool norm_known, const NextMinibatch *next = nullptr);
 bool adam_step_prepares(const mava_rollout *h);    // (a step with `next` does what that gradient would start with: it is then `prepared`)

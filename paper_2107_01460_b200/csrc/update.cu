@@ -307,15 +307,14 @@ size_t upd_smem_bytes(int Din, int H) {
 
 // The head of the scratch, the same in every layout of the rest.
 constexpr size_t kHeadBytes = 128 + 3 * sizeof(double) * 2 * kMomentBlocks;
-enum { kAdvMoments = 0, kAdvMoments2 = 2 };  // (two places for the advantages': see launch_ppo_grad)
-Moments moments_of(mava_rollout *h, int which, const float *x, long long n, const UpdRows &map, bool early = false) {
+Moments adv_moments_of(mava_rollout *h, int place, const UpdRows &rows) {  // (`place`, 0 or 1: see launch_ppo_grad)
   unsigned char *p = static_cast<unsigned char *>(h->d_upd);
-  return Moments{x, n, map, reinterpret_cast<double *>(p + 128) + which * 2 * kMomentBlocks, reinterpret_cast<double *>(p) + 4 * which,
-                 reinterpret_cast<unsigned *>(p + 96) + which, early};
+  const int which = 2 * place;
+  return Moments{h->buf.adv, rows.n, rows, reinterpret_cast<double *>(p + 128) + which * 2 * kMomentBlocks, reinterpret_cast<double *>(p) + 4 * which,
+                 reinterpret_cast<unsigned *>(p + 96) + which};
 }
 // The gradient's sums of squares, between the two places of the moments' partial sums.
 double *grad_squares_of(mava_rollout *h) { return reinterpret_cast<double *>(static_cast<unsigned char *>(h->d_upd) + 128) + 2 * kMomentBlocks; }
-Moments adv_moments_of(mava_rollout *h, int seq, const UpdRows &rows) { return moments_of(h, seq & 1 ? kAdvMoments2 : kAdvMoments, h->buf.adv, rows.n, rows, seq > 0); }
 
 struct UpdScratch {
   double *term_part;
@@ -437,13 +436,13 @@ static UpdRows rows_of(const mava_rollout *h, const int32_t *env_ids_dev, int n_
   return rows;
 }
 
-// `seq`: how many gradients and optimiser steps, and nothing else, this call's caller has launched directly before.  From the second
-// on the advantages' moments need not wait for the optimiser step: the gradient kernel lets its successors start only after
-// its own wait, so whatever was launched before the gradient in front (seq >= 1) is complete when this one's first kernel
-// starts.  That gradient may still read its moments: every other call has another place for them.
-// `prepared`: launch_adam_step was told of this minibatch (its `next`).
+// `prepared`: the step directly in front, itself directly behind a gradient, was told of this minibatch (the `next` of launch_adam_step)
+// and leaves its weight image and its advantages' moments.  The gradient kernel lets its successors start only after its own wait,
+// so whatever was launched before the gradient in front is complete when that step starts: the step may take the moments, and
+// this call fetch its first rows, before their waits.  The gradient in front may still read its own moments then, so the two
+// have different places (`place`, 0 or 1).
 cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava_ppo_hyper_t &hyper, float *grad_dev,
-                            float *terms_dev, const int32_t *env_ids_dev, int32_t n_ids, int seq, bool prepared) {
+                            float *terms_dev, const int32_t *env_ids_dev, int32_t n_ids, int place, bool prepared) {
   const mava_config_t &cfg = h->cfg;
   const int T = h->last_T, E = cfg.n_envs, N = cfg.n_agents, D = h->D, H = cfg.hidden;
   const ParamLayout L = param_layout(cfg, D, 1);
@@ -463,7 +462,7 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
   if (update_takes_tensor_cores(cfg, D)) {
     const UpdScratch sc = carve(h, ppo_tc_slice_floats(), slices);
     const TermSums terms{sc.term_part, sc.term_part, 4 * slices, 4 * slices, R, R, hp, terms_dev};
-    return launch_ppo_net_tc(h, params_dev, L, rows, hp, adv_moments_of(h, seq, rows), prepared, sc.image, sc.partial, sc.term_part, slices, grad_dev, terms,
+    return launch_ppo_net_tc(h, params_dev, L, rows, hp, adv_moments_of(h, place, rows), prepared, sc.image, sc.partial, sc.term_part, slices, grad_dev, terms,
                              grad_squares_of(h));
   }
 
@@ -475,7 +474,7 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
   if (update_takes_tensor_cores_256(cfg, D)) {
     const int sms = plan.sms;
     unsigned char *p = static_cast<unsigned char *>(h->d_upd) + kHeadBytes;
-    const Moments adv = moments_of(h, kAdvMoments, h->buf.adv, R, rows);
+    const Moments adv = adv_moments_of(h, place, rows);
     const double *stats = adv.out;
     TermSums terms{nullptr, nullptr, 0, 0, R, central ? S : R, hp, terms_dev};
     if (!central) {
@@ -499,7 +498,7 @@ cudaError_t launch_ppo_grad(mava_rollout *h, const float *params_dev, const mava
   };
   tr(L.W1, H, D); tr(L.W2, H, H);
   if (central) { tr(L.C1, H, joint); tr(L.C2, H, H); }
-  const Moments adv = moments_of(h, kAdvMoments, h->buf.adv, R, rows);
+  const Moments adv = adv_moments_of(h, place, rows);
   err = launch_dependent(rows_need_64_bits(rows, R) ? moments_kernel<uint64_t> : moments_kernel<uint32_t>, kMomentBlocks, 256, 0, st, adv);
   h->launches += 1;
   if (err == cudaSuccess) err = cudaMemsetAsync(sc.term_part, 0, sizeof(double) * 3 * 8 * slices, st);
@@ -556,7 +555,7 @@ cudaError_t launch_adam_step(mava_rollout *h, float *params_dev, const float *gr
   const float corr2 = static_cast<float>(1.0 - pow(static_cast<double>(hp.beta2), step));
   const AdamArgs adam{params_dev, grad_dev, m_dev, v_dev, squares, hp.max_grad_norm, hp.lr, hp.beta1, hp.beta2, hp.adam_eps, corr1, corr2};
   if (next && tc)
-    return launch_step_tc(h, adam, L, adv_moments_of(h, next->seq, rows_of(h, next->env_ids, next->n)), carve(h, ppo_tc_slice_floats(), 1).image);
+    return launch_step_tc(h, adam, L, adv_moments_of(h, next->place, rows_of(h, next->env_ids, next->n)), carve(h, ppo_tc_slice_floats(), 1).image);
   h->launches += 1;
   const int blocks = static_cast<int>((P + 255) / 256 < 2 * 148 ? (P + 255) / 256 : 2 * 148);
   return launch_dependent(adam_kernel, blocks, 256, 0, h->stream, adam, P);

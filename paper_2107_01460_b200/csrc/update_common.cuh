@@ -108,7 +108,6 @@ struct Moments {
   double *part;        // [kMomentBlocks][2]
   double *out;         // mean, std
   unsigned *finished;  // zero before and after
-  bool early;          // what it reads was complete before the kernel in front of this one was launched (launch_ppo_grad)
 };
 // Sums of a and b over the block's first 256 threads, in thread 0.
 __device__ __forceinline__ void block_sum2(double &a, double &b) {
@@ -161,15 +160,14 @@ __device__ __forceinline__ void moments_block(const Moments &m) {
   moments_finish(m, a, b);
 }
 // What a gradient call starts with: the advantages' moments and, by the other blocks, the weight image (prep(i, n): thread i
-// of n).  Early moments are taken while the kernels in front (the last minibatch's reduction and optimiser step) still run.
+// of n).
 template <class U, class Prep>
 __global__ void __launch_bounds__(256) prologue_kernel(Moments m, Prep prep) {
   dependents_may_start();
   const int first = m.x ? kMomentBlocks : 0, b = static_cast<int>(blockIdx.x);
-  if (b < first && m.early) moments_block<U>(m);
   wait_for_predecessor();
   if (b < first) {
-    if (!m.early) moments_block<U>(m);
+    moments_block<U>(m);
     return;
   }
   prep((b - first) * 256 + static_cast<int>(threadIdx.x), (static_cast<int>(gridDim.x) - first) * 256);
@@ -195,7 +193,7 @@ cudaError_t launch_ppo_net_tc(mava_rollout *h, const float *params_dev, const Pa
                               const TermSums &terms, double *squares);
 // The sums of squares that launch_ppo_net_tc leaves, of a gradient that comes from elsewhere: the same order of additions.
 cudaError_t launch_grad_squares_tc(mava_rollout *h, const ParamLayout &L, const float *grad, double *squares);
-// An optimiser step with what the next gradient starts with: its weight image and its advantages' moments (`next`, early).
+// An optimiser step with what the next gradient starts with: its weight image and its advantages' moments (`next`).
 cudaError_t launch_step_tc(mava_rollout *h, const AdamArgs &adam, const ParamLayout &L, const Moments &next, void *image);
 
 // Where the loss-term sums of a call lie, [n][3] doubles (surrogate, entropy, value) per list: the actor's list gives the

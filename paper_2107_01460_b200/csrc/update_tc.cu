@@ -132,11 +132,10 @@ __device__ __forceinline__ void PrepImage::operator()(int tid, int nth) const {
 // An optimiser step that leaves the next gradient its weight image and, by blocks of their own while the kernels in front still run,
 // its advantages' moments.  Everything but the gradient is read before the wait: what was launched before the gradient in front is
 // complete when this starts (launch_ppo_grad), the step before this one too.
-template <class U>
 __global__ void __launch_bounds__(256) step_image_kernel(AdamArgs adam, PrepImage prep, Moments next) {
   dependents_may_start();
   if (static_cast<int>(blockIdx.x) < kMomentBlocks) {
-    moments_block<U>(next);
+    moments_block<uint32_t>(next);  // (at most n_envs environments: no more rows than the trajectory has, below 2^32 in any memory)
     wait_for_predecessor();
     return;
   }
@@ -759,7 +758,7 @@ cudaError_t launch_ppo_net_tc(mava_rollout *h, const float *params_dev, const Pa
   err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (err != cudaSuccess) return err;
   err = launch_dependent(kern, slices, kUThreads, smem, h->stream, static_cast<const unsigned char *>(image), rows, hp,
-                         static_cast<const double *>(adv.out), partial, term_partial, h->d_status, h->D, h->cfg.hidden, adv.early, expire);
+                         static_cast<const double *>(adv.out), partial, term_partial, h->d_status, h->D, h->cfg.hidden, prepared, expire);
   if (err != cudaSuccess) return err;
   h->launches += 2;
   return launch_dependent(reduce_slices_kernel<SliceMap>, kReduceBlocks, kReduceThreads, 0, h->stream, static_cast<const float *>(partial), kSlice, slices, grad,
@@ -770,8 +769,7 @@ cudaError_t launch_grad_squares_tc(mava_rollout *h, const ParamLayout &L, const 
 }
 cudaError_t launch_step_tc(mava_rollout *h, const AdamArgs &adam, const ParamLayout &L, const Moments &next, void *image) {
   h->launches += 1;
-  return launch_dependent(rows_need_64_bits(next.map, next.n) ? step_image_kernel<uint64_t> : step_image_kernel<uint32_t>, kMomentBlocks + kPrepBlocks, 256, 0,
-                          h->stream, adam, PrepImage{adam.params, static_cast<unsigned char *>(image), L, h->D, h->cfg.hidden}, next);
+  return launch_dependent(step_image_kernel, kMomentBlocks + kPrepBlocks, 256, 0, h->stream, adam, PrepImage{adam.params, static_cast<unsigned char *>(image), L, h->D, h->cfg.hidden}, next);
 }
 
 }  // namespace mava
