@@ -112,9 +112,6 @@ struct CriticSmem {
 };
 static_assert((CriticShape<4>::C1_BYTES / 2) % 1024 == 0, "the fp32 stages follow C1 on a swizzle-pattern boundary");
 
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ float4 lds_f32x4(uint32_t addr) {
   float4 v;
   asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));

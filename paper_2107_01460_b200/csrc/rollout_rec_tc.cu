@@ -105,24 +105,11 @@ __device__ __forceinline__ uint4 lds_v4(uint32_t addr) {
   asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
   return v;
 }
-// 16 lanes x 32 columns: thread t gets of lanes t / 4 (r[4 j], r[4 j + 1]) and t / 4 + 8 (r[4 j + 2], r[4 j + 3]) the columns 8 j + 2 (t % 4)
-// and the one behind it.  A thread then has the same eight units of every row, and their biases stay in registers.
-__device__ __forceinline__ void tmem_ld_16x32_nowait(uint32_t taddr, uint32_t *r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
 __device__ __forceinline__ void loaded16(uint32_t *r) {  // (after the wait: what the loads brought is not touched before)
 #pragma unroll
   for (int i = 0; i < 16; ++i) asm volatile("" : "+r"(r[i]));
 }
-// Four core matrices (8 rows x 16 bytes) in registers in the layout above; lane l has the address of row l % 8 of matrix l / 8.
-__device__ __forceinline__ void stmatrix4(uint32_t addr, const uint32_t *r) {
-  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
-}
+// The counterpart of stmatrix4.
 __device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t *r) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
@@ -197,7 +184,7 @@ rollout_rec_tc_kernel(RolloutArgs a, const unsigned char *image, float *hidden, 
         if (active && k < a.T)
           sts_f32(smem_u32(&sm.uniform[row]), action_uniform(a.env, a.t_global0 + static_cast<uint32_t>(k), env_id, static_cast<uint32_t>(ag)));
         __syncwarp();
-        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ev_empty) : "memory");
+        if (lane == 0) mbar_arrive(ev_empty);
         if (k >= 1 && active) {
           const size_t at = static_cast<size_t>(k - 1) * M + static_cast<size_t>(e0) * N + crow;
           a.buf.values[at] = __uint_as_float(rec[kEvValue]);
@@ -314,7 +301,7 @@ rollout_rec_tc_kernel(RolloutArgs a, const unsigned char *image, float *hidden, 
         for (int q = 0; q < kEvPitch; q += 4) sts_v4(event_addr + 4u * q, w[q], w[q + 1], w[q + 2], w[q + 3]);
       }
       __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ev_full) : "memory");
+      if (lane == 0) mbar_arrive(ev_full);
     };
     auto await_helper = [&]() {  // it has taken the last event over (and drawn its step's uniform)
       timed_out |= !mbar_wait_warp(ev_empty, ev_phase);

@@ -392,7 +392,7 @@ rollout_tc_kernel(RolloutArgs a, const unsigned char *image, int ept, int n_tile
           if (active && k < a.T)  // the uniform of the step's action draw
             sts_f32(frac_addr + 4u * static_cast<uint32_t>(row), action_uniform(a.env, a.t_global0 + static_cast<uint32_t>(k), env_id, static_cast<uint32_t>(ag)));
           __syncwarp();
-          if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ev_empty) : "memory");
+          if (lane == 0) mbar_arrive(ev_empty);
           if (EVAL) continue;
           if (k >= 1 && active) {
             const size_t at = static_cast<size_t>(k - 1) * M + static_cast<size_t>(e0) * N + crow;
@@ -532,7 +532,7 @@ rollout_tc_kernel(RolloutArgs a, const unsigned char *image, int ept, int n_tile
           asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(event_addr + 4u * q), "r"(w[q]), "r"(w[q + 1]), "r"(w[q + 2]), "r"(w[q + 3]) : "memory");
       }
       __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ev_full) : "memory");
+      if (lane == 0) mbar_arrive(ev_full);
     };
     // The helper has taken the last event over (and drawn its step's uniform).
     auto await_helper = [&]() {

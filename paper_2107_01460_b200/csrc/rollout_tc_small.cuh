@@ -262,7 +262,7 @@ rollout_tc_small_kernel(RolloutArgs a, const unsigned char *image, int ept) {
       }
       draw(k + 2);
       __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ev_empty0 + 8u * (k & 1)) : "memory");
+      if (lane == 0) mbar_arrive(ev_empty0 + 8u * (k & 1));
     }
   } else {
     // ---- warps 0..3
@@ -300,7 +300,7 @@ rollout_tc_small_kernel(RolloutArgs a, const unsigned char *image, int ept) {
           *reinterpret_cast<uint4 *>(rec + 16) = make_uint4(__float_as_uint(out_logit[2]), __float_as_uint(out_logit[3]), __float_as_uint(out_logit[4]), __float_as_uint(out_logit[5]));
       }
       __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ev_full0 + 8u * (k & 1)) : "memory");
+      if (lane == 0) mbar_arrive(ev_full0 + 8u * (k & 1));
     };
     EvalSums sums;                // lanes with ag == 0: their environment
     float frac = step_fraction(env.step, a.env.cap);

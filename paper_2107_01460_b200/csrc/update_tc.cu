@@ -189,25 +189,8 @@ struct SliceMap {
 
 constexpr int kLoadRows = kUR / kULoaders;  // per loader warp, all of their loads in flight at once
 
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) { asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory"); }
-// One arrival per warp, after all its lanes are done with what the barrier guards.
-__device__ __forceinline__ void warp_arrive(uint32_t bar, int lane) {
-  __syncwarp();
-  if (lane == 0) mbar_arrive(bar);
-}
 __device__ __forceinline__ void prefetch_l2(const float *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void sts_u32(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
-// 16 lanes x 32 columns: thread t gets of lanes t / 4 (r[4 j], r[4 j + 1]) and t / 4 + 8 (r[4 j + 2], r[4 j + 3]) the columns 8 j + 2 (t % 4)
-// and the one behind it.  A thread then has the same eight columns of every row: their biases stay in registers (with a row per
-// thread each warp read all biases again for every tile, as many shared-memory cycles as the stores take).
-__device__ __forceinline__ void tmem_ld_16x32_nowait(uint32_t taddr, uint32_t *r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
 __device__ __forceinline__ void tmem_ld_row8(uint32_t taddr, float *v) {  // thread = lane
   uint32_t r[8];
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -220,10 +203,6 @@ __device__ __forceinline__ void tmem_ld_row8(uint32_t taddr, float *v) {  // thr
     asm volatile("" : "+r"(r[i]));
     v[i] = __uint_as_float(r[i]);
   }
-}
-// Four core matrices (8 rows x 16 bytes) out of registers in the layout above; lane l has the address of row l % 8 of matrix l / 8.
-__device__ __forceinline__ void stmatrix4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 // Waits for the tensor-memory loads; what they brought is not touched before.
 __device__ __forceinline__ void tmem_ld_wait32(uint32_t *r) {
@@ -529,7 +508,7 @@ ppo_net_tc_kernel(const unsigned char *image, UpdRows rows, UpdHyper hp, const d
       for (int c = 0; c < 2; ++c)
 #pragma unroll
         for (int j = 0; j < 4; j += 2)
-          stmatrix4(tile + my_at + static_cast<uint32_t>(c * 2 * kUH * 16 + j * 128), pk[8 * c + 2 * j], pk[8 * c + 2 * j + 1], pk[8 * c + 2 * j + 2], pk[8 * c + 2 * j + 3]);
+          stmatrix4(tile + my_at + static_cast<uint32_t>(c * 2 * kUH * 16 + j * 128), pk + 8 * c + 2 * j);
     };
     // hidden-layer epilogue: + bias -> ReLU -> bf16 -> `tile`; one gate bit per unit out (pair i: bits 15 - i and 31 - i).  Two
     // columns per instruction throughout.
