@@ -1,5 +1,5 @@
 // Dependent launches.  A collection is three short kernels or more in a row (weight image, rollout, advantages) and a gradient
-// with its optimiser step four; launched one after the other each pays a launch gap of a few microseconds.  They are launched
+// with its optimiser step five; launched one after the other each pays a launch gap of a few microseconds.  They are launched
 // with programmatic serialization instead: a kernel may start while the one before it still runs, does what needs nothing
 // from it (barriers, tensor memory, zeroed tiles) and then waits until that one is complete and its writes are visible.
 // Rules for a kernel that is launched like this:

@@ -517,7 +517,7 @@ cudaError_t launch_rec_tc_variant(mava_rollout *h, const RolloutArgs &args) {
   int ept = (h->cfg.n_envs + sms - 1) / sms;
   if (ept > EPT_MAX) ept = EPT_MAX;
   if (ept < 1) ept = 1;
-  for (int e = ept; e <= EPT_MAX; ++e)  // a block that is a whole number of 16-byte pieces leaves as one bulk copy
+  for (int e = ept; e <= EPT_MAX; ++e)  // tiles that start on 16-byte boundaries: the rows of each helper warp then leave as a bulk copy
     if ((e * N * D) % 4 == 0) { ept = e; break; }
   const int n_tiles = (h->cfg.n_envs + ept - 1) / ept;
   h->launches += 1;

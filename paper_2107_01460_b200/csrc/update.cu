@@ -298,8 +298,9 @@ __global__ void __launch_bounds__(256) adam_kernel(AdamArgs a, size_t n) {
   for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += static_cast<size_t>(gridDim.x) * blockDim.x) adam_element(a, adam_load(a, i), __ldcg(a.grad + i), scale, i);
 }
 
-// Scratch of the update block, made on first use: [moments of the advantages and of the gradient, counters][their partials][term partials][transposed
-// weights][partial gradients: one slice per CTA].
+// Scratch of the update block, made on first use: the head (two places for the advantages' moments, their counters, and the partial sums of
+// one, the gradient's sums of squares, the partial sums of the other), then [weight image][term partials][transposed
+// weights][partial gradients: one slice per CTA].  The image directly behind the head: a step finds it without knowing the slices.
 size_t upd_smem_bytes(int Din, int H) {
   return sizeof(float) * (static_cast<size_t>(kUpdRows) * ((Din + 3) & ~3) + 2 * static_cast<size_t>(kUpdRows) * H +
                           static_cast<size_t>(H) * kUpdTS + kUpdRows * 8 + kUpdRows * 2);

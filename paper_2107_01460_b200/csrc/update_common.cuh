@@ -216,27 +216,27 @@ __device__ __forceinline__ void loss_terms(const TermSums &t) {
   const int i = static_cast<int>(threadIdx.x);
   double a = 0.0, e = 0.0, v = 0.0;
   if (i < nt) {
-  for (int k0 = i; k0 < t.n_actor_part; k0 += kBatch * nt) {
-    double x[kBatch], y[kBatch];
+    for (int k0 = i; k0 < t.n_actor_part; k0 += kBatch * nt) {
+      double x[kBatch], y[kBatch];
 #pragma unroll
-    for (int q = 0; q < kBatch; ++q) { const int k = min(k0 + q * nt, t.n_actor_part - 1); x[q] = t.actor[3 * k]; y[q] = t.actor[3 * k + 1]; }
+      for (int q = 0; q < kBatch; ++q) { const int k = min(k0 + q * nt, t.n_actor_part - 1); x[q] = t.actor[3 * k]; y[q] = t.actor[3 * k + 1]; }
 #pragma unroll
-    for (int q = 0; q < kBatch; ++q)
-      if (k0 + q * nt < t.n_actor_part) { a += x[q]; e += y[q]; }
-  }
-  for (int k0 = i; k0 < t.n_value_part; k0 += kBatch * nt) {
-    double x[kBatch];
+      for (int q = 0; q < kBatch; ++q)
+        if (k0 + q * nt < t.n_actor_part) { a += x[q]; e += y[q]; }
+    }
+    for (int k0 = i; k0 < t.n_value_part; k0 += kBatch * nt) {
+      double x[kBatch];
 #pragma unroll
-    for (int q = 0; q < kBatch; ++q) x[q] = t.value[3 * min(k0 + q * nt, t.n_value_part - 1) + 2];
+      for (int q = 0; q < kBatch; ++q) x[q] = t.value[3 * min(k0 + q * nt, t.n_value_part - 1) + 2];
 #pragma unroll
-    for (int q = 0; q < kBatch; ++q)
-      if (k0 + q * nt < t.n_value_part) v += x[q];
-  }
+      for (int q = 0; q < kBatch; ++q)
+        if (k0 + q * nt < t.n_value_part) v += x[q];
+    }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xFFFFFFFFu, a, o); e += __shfl_xor_sync(0xFFFFFFFFu, e, o); v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  }
-  if ((i & 31) == 0) { st[0][i >> 5] = a; st[1][i >> 5] = e; st[2][i >> 5] = v; }
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xFFFFFFFFu, a, o); e += __shfl_xor_sync(0xFFFFFFFFu, e, o); v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    }
+    if ((i & 31) == 0) { st[0][i >> 5] = a; st[1][i >> 5] = e; st[2][i >> 5] = v; }
   }
   __syncthreads();
   if (i != 0) return;

@@ -15,8 +15,10 @@
 // Both fit an SM because d z2 takes h2's place and d z1 h1's (behind the weight-gradient products that read them), and
 // the heads' derivatives are kept once, eight columns wide.  Sixteen warps share every epilogue (32 rows x 32 columns each), eight
 // bring the rows in, one issues the MMAs in a fixed order, one fetches what the loss needs.  What bounds it (10x10, 61 k rows a
-// gradient): 6.7 k cycles per tile and SM against 8 k for one tile at a time; the products are 3.4 k of them, the rest is the
-// row of dependent epilogues (0.6 to 0.8 k each, half of it conversions and gate bits at half rate) and the waits between them.
+// gradient): 6.7 k cycles per tile and SM against 8 k for one tile at a time.  Some 4.6 k of them are products: 30 of N = 128 at 65 cycles
+// and 8 of N = 80 at 41 (2.3 k), and 32 of N = 16 that each stream a 4 KB A operand from shared memory and take 65 to 80, as long as one
+// of N = 128 (24 where x has a spare column: 4.0 k).  Beside them the row of dependent epilogues (0.6 to 0.8 k each, half of it
+// conversions and gate bits at half rate) and the waits between them.
 // Rows: fewer than 40 KB can be on their way through the 28 KB of L1 that are left; with more loads in flight, or the look-up of a
 // row in front of an epilogue, every other access of the SM stalls behind them.  Two passes of three minibatches over 549 k rows:
 // 407 -> 376 us; sixteen minibatches of 33 k rows: 502 -> 478.
